@@ -8,6 +8,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <vector>
 
@@ -211,6 +212,22 @@ int balanced_splits(int items, int ntiles, int* tiles_per_split) {
 int tc_splits(int M, int Hkv, int nseq, int ntiles, int* tiles_per_split) {
   const int nqblk = (M + 127) / 128;
   return balanced_splits(nqblk * Hkv * nseq, ntiles, tiles_per_split);
+}
+
+// CTAs per cluster, and clusters per (sequence, KV head), of the decode kernel (four warps per CTA, two
+// CTAs per SM).  The cluster grows to eight CTAs while the grid stays within 512: one sequence of 2048
+// slots, 8 heads: 7.3 us with eight, 9.8 with four, 25 with one; 256 units of 512-8192 slots: 91 us with
+// two, 109 with eight (the waits for a cluster's slowest CTA; sixteen took 9 us for 300 slots against 4.8).
+// A unit gets more clusters, and a combine kernel, only where SMs are idle and a warp keeps six blocks
+// (about 2 us of the combine against 0.66 us a block): 8 units of 16384 slots 27.4 -> 18.7 us with four.
+int decode_cluster(int units, int nmax_slots, int max_splits, int* splits) {
+  const int nblocks = (nmax_slots + KVS_DECODE_BLOCK - 1) / KVS_DECODE_BLOCK;
+  int c = 1;
+  while (c < 8 && units * c * 2 <= 512 && c * 4 < nblocks) c *= 2;
+  int s = 1;
+  while (units * c * s * 2 <= 2 * kNumSMs && nblocks >= c * 4 * s * 2 * 6 && 2 * s <= max_splits) s *= 2;
+  *splits = s;
+  return c;
 }
 
 // upper bound of the number of attention partials per query row (workspace sizing)
@@ -805,6 +822,7 @@ kvs_status_t kvs_decode_attn(const kvs_params_t* p, const void* q_new, int32_t n
   const int B = p->batch;
   const int M = c.G * n_new;
   const CacheView view = make_view(p, const_cast<void*>(K), const_cast<void*>(V), const_cast<int32_t*>(counts), n_max);
+  const bool few_rows = M <= KVS_DECODE_ROWS;
   CUtensorMap tmK, tmV, tmQ;
   {
     const uint64_t kd[4] = {KVS_D, (uint64_t)n_max, (uint64_t)p->n_kv_heads, (uint64_t)p->batch};
@@ -812,8 +830,9 @@ kvs_status_t kvs_decode_attn(const kvs_params_t* p, const void* q_new, int32_t n
     const uint64_t vs[3] = {(uint64_t)p->v_stride_t * 2, (uint64_t)p->v_stride_h * 2, (uint64_t)p->v_stride_b * 2};
     const uint64_t qd[3] = {KVS_D, (uint64_t)M, (uint64_t)c.L.U};
     const uint64_t qs[2] = {KVS_D * 2, (uint64_t)M * KVS_D * 2};
-    if (!(make_tmap(&tmK, K, 4, kd, ks, 128) && make_tmap(&tmV, V, 4, kd, vs, 128) &&
-          make_tmap(&tmQ, q_new, 3, qd, qs, 128)))
+    const int box = few_rows ? KVS_DECODE_BLOCK : 128;
+    if (!(make_tmap(&tmK, K, 4, kd, ks, box) && make_tmap(&tmV, V, 4, kd, vs, box) &&
+          (few_rows || make_tmap(&tmQ, q_new, 3, qd, qs, 128))))
       return fail(KVS_ERR_CUDA, "cuTensorMapEncodeTiled failed or is unavailable");
   }
   for (int b0 = 0; b0 < B; b0 += KVS_SEQ_CHUNK) {
@@ -827,12 +846,30 @@ kvs_status_t kvs_decode_attn(const kvs_params_t* p, const void* q_new, int32_t n
     }
     if (tab.nseq == 0) continue;
     int n_part = 0;
-    s = enqueue_flash(p, c.ws, c.L, c.st, view, n_new, M, 0, tab, nmax_slots, tmK, tmV, tmQ, status_dev, false,
-                      [&](auto&& f) -> kvs_status_t {
-                        CUDA_TRY(launch(KVS_K_FLASH, c.st, f));
-                        return KVS_OK;
-                      }, &n_part);
-    if (s != KVS_OK) return s;
+    if (few_rows) {
+      // the longest sequences first: they are the ones that a wave would wait for
+      std::sort(tab.s, tab.s + tab.nseq, [](const SeqRound& x, const SeqRound& y) { return x.n > y.n; });
+      DecodeArgs da;
+      da.counts = view.counts;
+      da.status_dev = status_dev; da.wait_us = g_wait_us.load(); da.debug_stall = g_debug_stall.load();
+      da.n_max = n_max; da.Hkv = p->n_kv_heads; da.M = M;
+      da.scale_log2 = p->softmax_scale * 1.4426950408889634f;
+      da.q = static_cast<const __nv_bfloat16*>(q_new);
+      da.out = static_cast<__nv_bfloat16*>(out); da.lse = lse;
+      da.part_ml = reinterpret_cast<float2*>(c.ws + c.L.part_ml);
+      da.part_o = reinterpret_cast<float*>(c.ws + c.L.part_o);
+      const int ctas = decode_cluster(p->n_kv_heads * tab.nseq, nmax_slots, splits_bound(M, p->n_kv_heads), &da.splits);
+      CUDA_TRY(launch(KVS_K_FLASH, c.st, [&] { return kvs_launch_decode_rows(da, tab, tmK, tmV, ctas, c.st); }));
+      if (da.splits == 1) continue;
+      n_part = da.splits;
+    } else {
+      s = enqueue_flash(p, c.ws, c.L, c.st, view, n_new, M, 0, tab, nmax_slots, tmK, tmV, tmQ, status_dev, false,
+                        [&](auto&& f) -> kvs_status_t {
+                          CUDA_TRY(launch(KVS_K_FLASH, c.st, f));
+                          return KVS_OK;
+                        }, &n_part);
+      if (s != KVS_OK) return s;
+    }
     CombineArgs ca;
     ca.M = M; ca.splits = n_part; ca.Hkv = p->n_kv_heads;
     ca.part_ml = reinterpret_cast<float2*>(c.ws + c.L.part_ml);

@@ -143,6 +143,25 @@ cudaError_t kvs_launch_stats_tc(const StatsTcArgs& a, const RoundTable& t, const
                                 const CUtensorMap& tmOlo, cudaStream_t st);
 cudaError_t kvs_launch_flash_tc(const FlashTcArgs& a, const RoundTable& t, const CUtensorMap& tmK,
                                 const CUtensorMap& tmV, const CUtensorMap& tmQ, cudaStream_t st);
+// Attention of at most KVS_DECODE_ROWS query rows per KV head (kvs_decode.cu): `ctas` CTAs form the cluster of
+// a (unit, split); with one split the output is final, with more every cluster leaves a partial.
+#define KVS_DECODE_ROWS 16
+#define KVS_DECODE_BLOCK 16        // slots of one box of its K and V tensor maps
+struct DecodeArgs {
+  const int32_t* counts;   // [U, n_max]
+  int32_t n_max, Hkv, M, splits;
+  float scale_log2;
+  const __nv_bfloat16* q;  // [U, M, 128]
+  __nv_bfloat16* out;      // [U, M, 128]
+  float* lse;              // optional [U, M]
+  float2* part_ml;         // [U, splits, M]
+  float* part_o;           // [U, splits, M, 128]
+  int32_t* status_dev;
+  uint32_t wait_us;        // time limit of one device-side wait, microseconds
+  uint32_t debug_stall;    // test hook: bit 0 = no tiles are requested
+};
+cudaError_t kvs_launch_decode_rows(const DecodeArgs& a, const RoundTable& t, const CUtensorMap& tmK,
+                                   const CUtensorMap& tmV, int ctas, cudaStream_t st);
 // Chunk of fresh tokens appended after the slots in use (table entry n = slots in use).
 struct AppendArgs {
   CacheView c;
