@@ -169,7 +169,7 @@ void round_plan(const kvs_params_t* p, int n, int budget, int r, int* off, int* 
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct WsLayout {
-  size_t part_ml, part_o, qstat, qc2, norms, o, o_hi, o_lo, score, w, mask, tile_prefix, part4, part1, sync, total;
+  size_t part_ml, part_o, qc2, norms, o_hi, o_lo, score, w, mask, tile_prefix, part4, part1, sync, total;
   int splits_max, M_max, pair_stride, tile_stride, counter_stride, nqblk_w, U;
   size_t sync_bytes;
 };
@@ -256,9 +256,7 @@ WsLayout make_layout(const kvs_params_t* p, int n_max, int max_new) {
   size_t o = 0;
   L.part_ml = o; o += align_up((size_t)L.U * part_rows * sizeof(float2));
   L.part_o = o;  o += align_up((size_t)L.U * part_rows * KVS_D * sizeof(float));
-  L.qstat = o;   o += align_up((size_t)L.U * L.M_max * sizeof(float4));
   L.qc2 = o;     o += align_up((size_t)L.U * ((Mw + 127) / 128 * 128) * sizeof(float2));
-  L.o = o;       o += align_up((size_t)L.U * L.M_max * KVS_D * sizeof(float));
   L.norms = o;   o += align_up((size_t)L.U * L.pair_stride * sizeof(float4));
   L.score = o;   o += align_up((size_t)L.U * L.pair_stride * sizeof(float));
   L.w = o;       o += align_up((size_t)L.U * L.pair_stride * sizeof(float));
@@ -382,8 +380,6 @@ kvs_status_t enqueue_round_stats(const Common& c, const CacheView& view, const v
   ca.M = c.Mw; ca.splits = n_part; ca.Hkv = p->n_kv_heads;
   ca.part_ml = reinterpret_cast<float2*>(c.ws + c.L.part_ml);
   ca.part_o = reinterpret_cast<float*>(c.ws + c.L.part_o);
-  ca.qstat = reinterpret_cast<float4*>(c.ws + c.L.qstat);
-  ca.o = reinterpret_cast<float*>(c.ws + c.L.o);
   ca.o_hi = reinterpret_cast<__nv_bfloat16*>(c.ws + c.L.o_hi);
   ca.o_lo = reinterpret_cast<__nv_bfloat16*>(c.ws + c.L.o_lo);
   ca.qc2 = reinterpret_cast<float2*>(c.ws + c.L.qc2);
@@ -412,18 +408,16 @@ kvs_status_t enqueue_round_stats(const Common& c, const CacheView& view, const v
   CUDA_TRY(launch(KVS_K_STATS, c.st, [&] {
     return kvs_launch_stats_tc(ta, tab, c.tmKp, c.tmVp, c.tmQ, c.weight_mode ? c.tmE : c.tmOhi, c.tmOlo, c.st);
   }));
-  g_launches.fetch_add(1, std::memory_order_relaxed);   // (two kernels behind that call: the statistics and their finalize)
 
-  if (do_select) {
-    SelectArgs se;
-    se.Hkv = p->n_kv_heads;
-    se.pair_stride = c.L.pair_stride; se.tile_stride = c.L.tile_stride;
-    se.score = ta.score;
-    se.mask = mask_out ? mask_out : reinterpret_cast<uint8_t*>(c.ws + c.L.mask);
-    se.tile_prefix = reinterpret_cast<int32_t*>(c.ws + c.L.tile_prefix);
-    se.from_mask = 0;
-    CUDA_TRY(launch(KVS_K_SELECT, c.st, [&] { return kvs_launch_select(se, tab, c.st); }));
-  }
+  SelectArgs se;
+  se.Hkv = p->n_kv_heads;
+  se.pair_stride = c.L.pair_stride; se.tile_stride = c.L.tile_stride;
+  se.mask = mask_out ? mask_out : reinterpret_cast<uint8_t*>(c.ws + c.L.mask);
+  se.tile_prefix = reinterpret_cast<int32_t*>(c.ws + c.L.tile_prefix);
+  se.select = do_select ? 1 : 0;
+  int kernels = 1;
+  CUDA_TRY(launch(KVS_K_SELECT, c.st, [&] { return kvs_launch_finalize_select(ta, se, tab, c.st, &kernels); }));
+  g_launches.fetch_add((uint64_t)kernels - 1, std::memory_order_relaxed);
   return KVS_OK;
 }
 
@@ -527,11 +521,10 @@ kvs_status_t kvs_detail_compact_scratch(const kvs_params_t* p, void* K, void* V,
     SelectArgs se;
     se.Hkv = p->n_kv_heads;
     se.pair_stride = caller_stride; se.tile_stride = tile_stride;
-    se.score = nullptr;
     se.mask = const_cast<uint8_t*>(merge_mask);
     se.tile_prefix = tile_prefix;
-    se.from_mask = 1;
-    CUDA_TRY(launch(KVS_K_MISC, st, [&] { return kvs_launch_select(se, tab, st); }));
+    se.select = 1;
+    CUDA_TRY(launch(KVS_K_MISC, st, [&] { return kvs_launch_mask_prefix(se, tab, st); }));
     CompactArgs ka;
     ka.c = view;
     ka.pair_stride = caller_stride; ka.tile_stride = tile_stride;
@@ -786,11 +779,10 @@ kvs_status_t kvs_compact(const kvs_params_t* p, void* K, void* V, int32_t* count
     SelectArgs se;
     se.Hkv = p->n_kv_heads;
     se.pair_stride = caller_stride; se.tile_stride = c.L.tile_stride;
-    se.score = nullptr;
     se.mask = const_cast<uint8_t*>(merge_mask);
     se.tile_prefix = reinterpret_cast<int32_t*>(c.ws + c.L.tile_prefix);
-    se.from_mask = 1;
-    CUDA_TRY(launch(KVS_K_MISC, c.st, [&] { return kvs_launch_select(se, tab, c.st); }));
+    se.select = 1;
+    CUDA_TRY(launch(KVS_K_MISC, c.st, [&] { return kvs_launch_mask_prefix(se, tab, c.st); }));
     CompactArgs ka;
     ka.c = view;
     ka.pair_stride = caller_stride; ka.tile_stride = c.L.tile_stride;
@@ -874,7 +866,7 @@ kvs_status_t kvs_decode_attn(const kvs_params_t* p, const void* q_new, int32_t n
     ca.M = M; ca.splits = n_part; ca.Hkv = p->n_kv_heads;
     ca.part_ml = reinterpret_cast<float2*>(c.ws + c.L.part_ml);
     ca.part_o = reinterpret_cast<float*>(c.ws + c.L.part_o);
-    ca.qstat = nullptr; ca.qc2 = nullptr; ca.M_pad = 0; ca.o = nullptr; ca.o_hi = nullptr; ca.o_lo = nullptr;
+    ca.qc2 = nullptr; ca.M_pad = 0; ca.o_hi = nullptr; ca.o_lo = nullptr;
     ca.out_bf16 = static_cast<__nv_bfloat16*>(out);
     ca.lse_out = lse; ca.o_out = nullptr; ca.e = nullptr;
     CUDA_TRY(launch(KVS_K_COMBINE, c.st, [&] { return kvs_launch_combine(ca, tab, c.st); }));

@@ -4,7 +4,7 @@
 // are merged into the row's softmax normaliser and attention output
 //   o_q = sum_j alpha_qj Vsum_j / c_j,  alpha = softmax_j(scale <q, K_j> + ln c_j)   [Eq. attn_def_vec
 // with merged slots].  For the observation window the kernel writes what the statistics pass needs
-// (per-query constants, o in fp32 and as two bf16 terms); for the decode check the bf16 output.
+// (per-query constants, o as two bf16 terms); for the decode check the bf16 output.
 #include "kvs_internal.h"
 
 namespace {
@@ -12,6 +12,11 @@ namespace {
 // One warp per (query row, unit), eight rows per CTA; a lane owns four output channels.
 constexpr int kCombineRows = 8;
 
+// kBatch: partial outputs of a row that are requested together.  With few rows the kernel is a chain of L2
+// round trips, and shorter with eight (1024 rows of 9-37 ranges: 8.5-10 -> 5.3 us); with many rows it is
+// bound by bytes in flight, and the registers of a batch cost occupancy (8192 rows of 8 ranges: 9 us one by one,
+// 15 us in eights; 65536 rows of 2: 24 and 75 us).
+template <int kBatch>
 __global__ void __launch_bounds__(kCombineRows * 32)
 combine_partials(const CombineArgs a, const RoundTable tab) {
   kvs_pdl_launch_dependents();
@@ -27,18 +32,50 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
     return;
   }
   const size_t base = (size_t)unit * a.splits * a.M + m;
-  float mstar = -INFINITY;
-  for (int s = 0; s < a.splits; ++s) mstar = fmaxf(mstar, a.part_ml[base + (size_t)s * a.M].x);
-  float Z = 0.f;
+  float mstar = -INFINITY, Z = 0.f;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int s = 0; s < a.splits; ++s) {
-    const float2 ml = a.part_ml[base + (size_t)s * a.M];
-    if (ml.x == -INFINITY) continue;
-    const float f = fast_exp2(ml.x - mstar);
-    Z = fmaf(ml.y, f, Z);
-    const float4 po = *reinterpret_cast<const float4*>(a.part_o + (base + (size_t)s * a.M) * KVS_D + 4 * lane);
-    acc.x = fmaf(po.x, f, acc.x); acc.y = fmaf(po.y, f, acc.y);
-    acc.z = fmaf(po.z, f, acc.z); acc.w = fmaf(po.w, f, acc.w);
+  if constexpr (kBatch == 1) {
+    for (int s = 0; s < a.splits; ++s) mstar = fmaxf(mstar, a.part_ml[base + (size_t)s * a.M].x);
+    for (int s = 0; s < a.splits; ++s) {
+      const float2 ml = a.part_ml[base + (size_t)s * a.M];
+      if (ml.x == -INFINITY) continue;
+      const float f = fast_exp2(ml.x - mstar);
+      Z = fmaf(ml.y, f, Z);
+      const float4 po = *reinterpret_cast<const float4*>(a.part_o + (base + (size_t)s * a.M) * KVS_D + 4 * lane);
+      acc.x = fmaf(po.x, f, acc.x); acc.y = fmaf(po.y, f, acc.y);
+      acc.z = fmaf(po.z, f, acc.z); acc.w = fmaf(po.w, f, acc.w);
+    }
+  } else {
+    const float2* ml = a.part_ml + base;
+    const float2 first = lane < a.splits ? ml[(size_t)lane * a.M] : make_float2(-INFINITY, 0.f);
+    mstar = first.x;
+    for (int s = 32 + lane; s < a.splits; s += 32) mstar = fmaxf(mstar, ml[(size_t)s * a.M].x);
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) mstar = fmaxf(mstar, __shfl_xor_sync(0xffffffffu, mstar, k));
+    for (int s0 = 0; s0 < a.splits; s0 += 32) {
+      const int cnt = min(32, a.splits - s0);
+      float2 own = first;
+      if (s0 > 0) own = lane < cnt ? ml[(size_t)(s0 + lane) * a.M] : make_float2(-INFINITY, 0.f);
+      const float f = own.x == -INFINITY ? 0.f : fast_exp2(own.x - mstar);   // 0: an empty range, whose output is not read
+      Z = fmaf(own.y, f, Z);
+      for (int i0 = 0; i0 < cnt; i0 += kBatch) {
+        float4 po[kBatch];
+        float fi[kBatch];
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+          fi[i] = __shfl_sync(0xffffffffu, f, i0 + i);
+          po[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (fi[i] != 0.f) po[i] = *reinterpret_cast<const float4*>(a.part_o + (base + (size_t)(s0 + i0 + i) * a.M) * KVS_D + 4 * lane);
+        }
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+          acc.x = fmaf(po[i].x, fi[i], acc.x); acc.y = fmaf(po[i].y, fi[i], acc.y);
+          acc.z = fmaf(po[i].z, fi[i], acc.z); acc.w = fmaf(po[i].w, fi[i], acc.w);
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, k);
   }
   const float4 od = make_float4(acc.x / Z, acc.y / Z, acc.z / Z, acc.w / Z);
   // |o|^2 over the 128 channels
@@ -57,12 +94,10 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
     qconst = eo;
   }
   if (lane == 0) {
-    if (a.qstat) a.qstat[row] = make_float4(mstar, Z, on2, lse);
     if (a.qc2) a.qc2[(size_t)unit * a.M_pad + m] = make_float2(-(mstar + log2f(Z)), qconst);
     if (a.lse_out) a.lse_out[row] = lse;
   }
   const float v[4] = {od.x, od.y, od.z, od.w};
-  if (a.o) *reinterpret_cast<float4*>(a.o + row * KVS_D + 4 * lane) = od;
   if (a.o_out) *reinterpret_cast<float4*>(a.o_out + row * KVS_D + 4 * lane) = od;
   if (a.o_hi) {
     __nv_bfloat16 hi[4], lo[4];
@@ -87,5 +122,8 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
 cudaError_t kvs_launch_combine(const CombineArgs& a, const RoundTable& t, cudaStream_t st) {
   const int rows = a.qc2 ? a.M_pad : a.M;
   dim3 grid((rows + kCombineRows - 1) / kCombineRows, a.Hkv, t.nseq);
-  return kvs_launch_chained(combine_partials, grid, dim3(kCombineRows * 32), 0, st, a, t);
+  // (two CTAs per SM: one wave at the registers of a batch)
+  if ((long long)grid.x * grid.y * grid.z <= 2 * 148)
+    return kvs_launch_chained(combine_partials<8>, grid, dim3(kCombineRows * 32), 0, st, a, t);
+  return kvs_launch_chained(combine_partials<1>, grid, dim3(kCombineRows * 32), 0, st, a, t);
 }

@@ -23,8 +23,8 @@
 enum KvsKernelKind {
   KVS_K_FLASH = 0,     // window / decode attention partials
   KVS_K_COMBINE = 1,   // partial combine
-  KVS_K_STATS = 2,     // Hessian statistics + cosine + score + weight
-  KVS_K_SELECT = 3,    // exact R-smallest selection + tile prefix
+  KVS_K_STATS = 2,     // Hessian statistics
+  KVS_K_SELECT = 3,    // score + weight + exact R-smallest selection + tile prefix
   KVS_K_COMPACT = 4,   // merge + in-place compaction
   KVS_K_MISC = 5,      // mask scan for kvs_compact, chunk append, similarity diagnostics
   KVS_K_COUNT = 6
@@ -72,10 +72,8 @@ struct CombineArgs {
   int32_t M, splits, Hkv;
   const float2* part_ml;
   const float* part_o;
-  float4* qstat;           // [U, M]: (max log2, Z, |o|^2, lse natural)
   float2* qc2;             // [U, M_pad]: (-(max + log2 Z), |o|^2); rows M..M_pad-1 get (-inf, 0) (may be NULL)
   int32_t M_pad;           // M rounded up to a multiple of 128 (grid rows when qc2 is written)
-  float* o;                // [U, M, 128] fp32 (may be NULL)
   __nv_bfloat16* o_hi;     // [U, M, 128]: o = o_hi + o_lo to ~2^-17 relative (may be NULL)
   __nv_bfloat16* o_lo;
   __nv_bfloat16* out_bf16; // decode: [B, Hq, n_new, 128] == [U, M, 128] (may be NULL)
@@ -112,10 +110,9 @@ struct SelectArgs {
   int32_t Hkv;
   int32_t pair_stride;
   int32_t tile_stride;     // row length of tile_prefix
-  const float* score;
   uint8_t* mask;           // [U, pair_stride]
   int32_t* tile_prefix;    // [U, tile_stride]: merged pairs before each compaction tile
-  int32_t from_mask;       // 1: mask is an input (kvs_compact), only the prefix is built
+  int32_t select;          // 0: scores and weights only
 };
 
 struct CompactArgs {
@@ -170,7 +167,11 @@ struct AppendArgs {
   int32_t chunk_len;
 };
 cudaError_t kvs_launch_append(const AppendArgs& a, const RoundTable& t, cudaStream_t st);
-cudaError_t kvs_launch_select(const SelectArgs& a, const RoundTable& t, cudaStream_t st);
+// Scores and weights from the statistics' partial sums, then the selection (kvs_select.cu); and, for a mask that
+// the caller supplies, the merged pairs before each compaction tile.  *kernels: how many were launched.
+cudaError_t kvs_launch_finalize_select(const StatsTcArgs& sa, const SelectArgs& a, const RoundTable& t, cudaStream_t st,
+                                       int* kernels);
+cudaError_t kvs_launch_mask_prefix(const SelectArgs& a, const RoundTable& t, cudaStream_t st);
 // Adjacent-row cosine of a bf16 tensor [B, H, n_max, 128] (element strides sb, sh, st); table entry n = rows in use.
 cudaError_t kvs_launch_adjacent_cosine(const void* x, int64_t sb, int64_t sh, int64_t st, int H, int n_max,
                                        float* out, const RoundTable& t, cudaStream_t stream);

@@ -1,180 +1,303 @@
-// Exact selection of the R candidate pairs with the smallest (score, pair index) and the
-// per-tile exclusive counts that the compaction needs.
+// Scores, merge weights and the exact selection of a round.
 //
-// One CTA of 1024 threads per (sequence, KV head).  Scores are non-negative floats, so
-// their bit patterns order like unsigned integers: a four-pass, 8-bit radix select finds
-// the bit pattern of the R-th smallest score and how many pairs tied with it are still
-// needed; ties are taken in index order.  A second sweep writes the mask and, for every
-// compaction tile of 32 pairs, the number of merged pairs that precede it.
+// A cluster of up to eight CTAs owns a (sequence, KV head) unit; a CTA owns a run of compaction tiles
+// (32 candidate pairs each), a thread one pair of every 1024.  The cluster
+//   1. adds the statistics kernel's partial sums of every pair in a fixed order and forms the pair's
+//      score and left-key weight (for long rounds a kernel of its own does that, see below),
+//   2. finds the bit pattern of the R-th smallest score by a radix select in three passes of 11, 11
+//      and 10 bits (scores are non-negative floats: their bit patterns order like unsigned integers);
+//      every CTA counts its own keys in shared memory and adds up the cluster's histograms,
+//   3. writes the mask (ties at the cutoff are taken in index order) and, for every compaction tile,
+//      the number of merged pairs that precede it.
+// The keys stay in shared memory from the first step to the last.  Latency bound: barriers, L2 round trips
+// and instruction fetches -- every instruction runs a few times only, so the loops are kept rolled (keys
+// in registers and unrolled loops took 2.5 k cycles a pass).
+// Measured, statistics' finalize + selection of a round, one CTA per unit and four passes -> this:
+// 8 units of 2000 pairs 11.0 -> 7.9 us, of 16336 pairs 36.5 -> 24 us; 64 units of 2.5-32 k pairs 42 -> 27 us;
+// 8 units of 65 k pairs and 24 partials a pair 73 -> 47 us.  The counts of a given mask (65 k pairs): 18 -> 7.5 us.
+#include <cooperative_groups.h>
+
 #include "kvs_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
-__global__ void __launch_bounds__(1024)
-select_pairs_kernel(const SelectArgs a, const RoundTable tab) {
+constexpr int kThreads = 1024;
+constexpr int kWarps = kThreads / 32;
+constexpr int kKeep = 32;                  // keys of a thread held in shared memory (with more, all are read again)
+constexpr int kBins = 2048;
+constexpr int kMaxCluster = 8;
+constexpr int kPairsPerCta = 4096;         // (see cluster_of)
+constexpr int kFusedPairs = 4096;          // (see kvs_launch_finalize_select)
+
+// Sum of the partials of all (query block, statistics group) pairs in a fixed order, then score and
+// left-key weight of candidate pair p.  Weight modes:
+//   0: the sums are norms; w = (N1_l - N12) / (N1_l - 2 N12 + N1_r)                        [Eq. kstar_final]
+//   1: they are the signed sums G11, G22, G12 of g_ij = E^T c_ij; w = (G11 + G12) / (G11 + 2 G12 + G22)
+//                                                                            [Eq. kstar_weight_final_rewrite]
+//   2: as 1 with the coupling dropped, w = G11 / (G11 + G22)                              [Eq. simplified_k]
+// A denominator that is not safely positive gives 1/2; the weight is clipped to [0, 1].
+__device__ __forceinline__ float finalize_pair(const StatsTcArgs& a, int unit, int off, int p) {
+  const int jl = off + 2 * p;
+  const int nsub = a.nqblk * KVS_STATS_GROUPS;
+  const float4* p4 = a.part4 + (size_t)unit * nsub * a.pair_stride + p;
+  const float* p1 = a.part1 + (size_t)unit * nsub * a.pair_stride + p;
+  float Al = 0.f, Ar = 0.f, N1l = 0.f, N1r = 0.f, N12 = 0.f;
+  for (int sb = 0; sb < nsub; sb += KVS_STATS_GROUPS) {
+    float4 v[KVS_STATS_GROUPS];
+    float x[KVS_STATS_GROUPS];
+#pragma unroll
+    for (int i = 0; i < KVS_STATS_GROUPS; ++i) {
+      v[i] = p4[(size_t)(sb + i) * a.pair_stride];
+      x[i] = p1[(size_t)(sb + i) * a.pair_stride];
+    }
+#pragma unroll
+    for (int i = 0; i < KVS_STATS_GROUPS; ++i) { Al += v[i].x; Ar += v[i].y; N1l += v[i].z; N1r += v[i].w; N12 += x[i]; }
+  }
+  const float cosv = a.pair_norms[(size_t)unit * a.norm_stride + p].w;
+  const float mass = Al + Ar;
+  const float score = (a.score_mode == 0) ? mass * fmaxf(0.f, 1.f - cosv) : mass;
+  float w = 0.5f;
+  if (a.weight_mode == 0) {
+    const float D = N1l - 2.f * N12 + N1r;
+    if (D > 1e-6f * (N1l + N1r) && D < INFINITY) w = fminf(1.f, fmaxf(0.f, (N1l - N12) / D));
+  } else {
+    const float g12 = (a.weight_mode == 2) ? 0.f : N12;
+    const float gamma = N1l + 2.f * g12 + N1r;
+    if (gamma > 1e-6f * (fabsf(N1l) + fabsf(N1r)) && gamma < INFINITY) w = fminf(1.f, fmaxf(0.f, (N1l + g12) / gamma));
+  }
+  const size_t pi = (size_t)unit * a.pair_stride + p;
+  a.score[pi] = fabsf(score);
+  a.w[pi] = w;
+  if (a.N12) a.N12[pi] = N12;
+  if (a.cosv) a.cosv[pi] = cosv;
+  if (a.A) { a.A[(size_t)unit * a.n_max + jl] = Al; a.A[(size_t)unit * a.n_max + jl + 1] = Ar; }
+  if (a.N1) { a.N1[(size_t)unit * a.n_max + jl] = N1l; a.N1[(size_t)unit * a.n_max + jl + 1] = N1r; }
+  return fabsf(score);
+}
+
+// Exclusive prefix of `v` over the threads of the CTA (one barrier; `s_warp` is free again after the next one).
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* s_warp) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) s_warp[warp] = inc;
+  __syncthreads();
+  uint32_t w = s_warp[lane];                               // (32 warps, 32 lanes)
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, w, o);
+    if (lane >= o) w += t;
+  }
+  const uint32_t before = warp ? __shfl_sync(0xffffffffu, w, warp - 1) : 0u;
+  return before + inc - v;
+}
+
+// Step 1 alone, over the whole GPU: one thread per pair.
+__global__ void __launch_bounds__(256)
+finalize_kernel(const StatsTcArgs a, const RoundTable tab) {
   kvs_pdl_launch_dependents();
   kvs_pdl_wait();
-  const int seq = blockIdx.y;
-  const SeqRound sr = tab.s[seq];
-  const int n = sr.n;
-  if (n <= 0) return;
-  const int unit = sr.b * a.Hkv + blockIdx.x;
-  const int P = sr.P, R = sr.R;
+  const SeqRound sr = tab.s[blockIdx.z];
+  const int p = blockIdx.x * 256 + threadIdx.x;
+  if (sr.n <= 0 || p >= sr.P) return;
+  finalize_pair(a, sr.b * a.Hkv + blockIdx.y, tab.off, p);
+}
+
+// kFused: step 1 too; kScores: the scores are in memory; kMask: the mask is an input (kvs_compact) and only
+// the counts of step 3 are formed.
+enum { kFused = 0, kScores = 1, kMask = 2 };
+template <int kMode>
+__global__ void __launch_bounds__(kThreads, 2)
+select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
+  constexpr bool kFromMask = kMode == kMask;
+  extern __shared__ uint32_t s_key[];
+  __shared__ uint32_t s_hist[3][kBins];
+  __shared__ uint32_t s_warp[2][kWarps], s_digit, s_k, s_total[2], s_cnt[2][kWarps];
+  kvs_pdl_launch_dependents();
+  cg::cluster_group cluster = cg::this_cluster();
+  const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t* key = reinterpret_cast<const uint32_t*>(a.score) + (size_t)unit * a.pair_stride;
+  if (tid < 2) s_total[tid] = 0;
+  if (!kFromMask)
+    for (int i = tid; i < 3 * kBins; i += kThreads) (&s_hist[0][0])[i] = 0;
+  kvs_pdl_wait();
+  const SeqRound sr = tab.s[blockIdx.z];
+  const int n = sr.n;
+  if (n <= 0) return;                                      // (the whole cluster)
+  const int unit = sr.b * a.Hkv + blockIdx.y;
+  const int P = sr.P;
+  // this CTA's compaction tiles and pairs
+  const int ntiles = max(0, n - tab.off + KVS_CTILE - 1) / KVS_CTILE;
+  const int per_cta = (ntiles + ctas - 1) / ctas;
+  const int t0 = min(ntiles, rank * per_cta), t1 = min(ntiles, t0 + per_cta);
+  const int steps = (t1 - t0 + kWarps - 1) / kWarps;       // of 32 tiles = 1024 pairs
+  const int p_end = min(P, 32 * t1);
+  const int p_first = 32 * t0 + tid;
   uint8_t* mask = a.mask + (size_t)unit * a.pair_stride;
+  const uint32_t* score = reinterpret_cast<const uint32_t*>(sa.score) + (size_t)unit * a.pair_stride;
 
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t s_digit, s_k;
-  __shared__ uint32_t s_cnt[128], s_pre[128];
-  __shared__ uint32_t s_run_tie, s_run_sel;
-
-  uint32_t prefix = 0, pmask = 0, k = (uint32_t)R;
-  if (!a.from_mask) {
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
-      if (tid < 256) hist[tid] = 0;
-      __syncthreads();
-      // four loads in flight per thread: the sweep is a chain of L2 latencies otherwise
-      for (int p0 = 0; p0 < P; p0 += 4 * 1024) {
-        uint32_t v4[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int p = p0 + u * 1024 + tid;
-          v4[u] = (p < P) ? __ldg(key + p) : 0u;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int p = p0 + u * 1024 + tid;
-          const uint32_t v = v4[u];
-          const bool in = (p < P) && (v & pmask) == prefix;
-          const uint32_t d = (v >> shift) & 255u;
-          const uint32_t act = __ballot_sync(0xffffffffu, in);
-          if (in) {
-            const uint32_t same = __match_any_sync(act, d);
-            if (lane == (__ffs(same) - 1)) atomicAdd(&hist[d], (uint32_t)__popc(same));
-          }
-        }
-      }
-      __syncthreads();
-      if (warp == 0) {
-        // lane owns bins [8 lane, 8 lane + 8)
-        uint32_t loc[8], sum = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { loc[i] = hist[8 * lane + i]; sum += loc[i]; }
-        uint32_t inc = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-          if (lane >= o) inc += t;
-        }
-        uint32_t excl = inc - sum;
-        const bool mine = excl < k && k <= inc;      // the k-th element falls in my bins
-        if (mine) {
-          uint32_t cum = excl;
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            if (cum < k && k <= cum + loc[i]) { s_digit = 8 * lane + i; s_k = k - cum; }
-            cum += loc[i];
-          }
-        }
-      }
-      __syncthreads();
-      prefix |= s_digit << shift;
-      pmask |= 255u << shift;
-      k = s_k;
-      __syncthreads();
+  if (!kFromMask) {
+#pragma unroll 1
+    for (int u = 0, p = p_first; p < p_end; ++u, p += kThreads) {
+      const uint32_t x = kMode == kFused ? __float_as_uint(finalize_pair(sa, unit, tab.off, p)) : score[p];
+      if (steps <= kKeep) s_key[u * kThreads + tid] = x;
     }
   }
-  // prefix = bit pattern of the cutoff score, k = ties (in index order) still to take.
-  // The sweep takes 4096 pairs per step (four per thread, 128 warp-sized groups): the groups'
-  // tie counts and, after the ranks are known, their selection counts are scanned by the first
-  // warp, which also gives the number of merged pairs in front of every compaction tile.
-  if (tid == 0) { s_run_tie = 0; s_run_sel = 0; }
+  // the keys of this CTA (every thread reads only what it has written itself)
+  const uint32_t* keys = steps <= kKeep ? s_key + tid : score + p_first;
+  auto key_of = [&](int u, int p) -> uint32_t {
+    if (p >= p_end) return 0u;
+    return kFromMask ? (uint32_t)mask[p] : keys[(size_t)u * kThreads];
+  };
+  auto cluster_barrier = [&] { if (ctas > 1) cluster.sync(); else __syncthreads(); };
+
+  // ---- cutoff: bit pattern of the R-th smallest score; k of its ties are taken
+  uint32_t cutoff = 0, k = kFromMask ? 0u : (uint32_t)sr.R;
   __syncthreads();
-  const int ntiles = (n - tab.off + KVS_CTILE - 1) / KVS_CTILE;
-  int32_t* tp = a.tile_prefix + (size_t)unit * a.tile_stride;
-  const int sweep = ((ntiles * 32 + 4095) / 4096) * 4096;
-  // exclusive scan of the 128 group counts in s_cnt by warp 0 (lane i owns groups 4 i .. 4 i + 3)
-  auto scan_groups = [&](uint32_t* run_total) {
-    if (warp == 0) {
-      uint32_t c[4], sum = 0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { c[i] = s_cnt[4 * lane + i]; sum += c[i]; }
-      uint32_t inc = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
+  if (!kFromMask) {
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+      const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
+      const int bits = pass == 2 ? 10 : 11;
+#pragma unroll 1
+      for (int u = 0, p = p_first; p < p_end; ++u, p += kThreads) {
+        const uint32_t v = key_of(u, p);
+        if (pass == 0 || ((v ^ cutoff) >> (shift + bits)) == 0) atomicAdd(&s_hist[pass][(v >> shift) & ((1u << bits) - 1u)], 1u);
       }
-      uint32_t ex = *run_total + inc - sum;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { s_pre[4 * lane + i] = ex; ex += c[i]; }
-      __syncwarp();
-      if (lane == 31) *run_total = ex;
-    }
-  };
-  uint32_t v4[4];
-  auto fetch = [&](int p0) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int p = p0 + u * 1024 + tid;
-      v4[u] = 0;
-      if (p < P) v4[u] = a.from_mask ? (uint32_t)mask[p] : __ldg(key + p);
-    }
-  };
-  fetch(0);
-  for (int p0 = 0; p0 < sweep; p0 += 4096) {
-    uint32_t v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = v4[u];
-    if (p0 + 4096 < sweep) fetch(p0 + 4096);              // the next step's values travel meanwhile
-    bool sel[4];
-    if (!a.from_mask) {
-      uint32_t tb[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int p = p0 + u * 1024 + tid;
-        tb[u] = __ballot_sync(0xffffffffu, p < P && v[u] == prefix);
-        if (lane == 0) s_cnt[u * 32 + warp] = __popc(tb[u]);
+      cluster_barrier();
+      uint2 h = make_uint2(0, 0);
+#pragma unroll 1
+      for (int r = 0; r < ctas; ++r) {
+        const uint2 x = *cluster.map_shared_rank(reinterpret_cast<uint2*>(&s_hist[pass][2 * tid]), r);
+        h.x += x.x; h.y += x.y;
       }
+      const uint32_t before = block_scan(h.x + h.y, s_warp[pass & 1]);
+      if (before < k && k <= before + h.x) { s_digit = 2 * tid; s_k = k - before; }
+      if (before + h.x < k && k <= before + h.x + h.y) { s_digit = 2 * tid + 1; s_k = k - before - h.x; }
       __syncthreads();
-      scan_groups(&s_run_tie);
-      __syncthreads();
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int p = p0 + u * 1024 + tid;
-        const uint32_t rank = s_pre[u * 32 + warp] + __popc(tb[u] & ((1u << lane) - 1u));
-        sel[u] = p < P && (v[u] < prefix || (v[u] == prefix && rank < k));
-        if (p < P) mask[p] = sel[u] ? 1 : 0;
-      }
-      __syncthreads();                                    // s_pre is reused below
-    } else {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) sel[u] = (p0 + u * 1024 + tid) < P && v[u] != 0;
+      cutoff |= s_digit << shift;
+      k = s_k;
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint32_t sb = __ballot_sync(0xffffffffu, sel[u]);
-      if (lane == 0) s_cnt[u * 32 + warp] = __popc(sb);
-    }
-    __syncthreads();
-    scan_groups(&s_run_sel);
-    __syncthreads();
-    if (lane == 0) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int tile = (p0 >> 5) + u * 32 + warp;
-        if (tile < ntiles) tp[tile] = (int32_t)s_pre[u * 32 + warp];
-      }
-    }
-    __syncthreads();
   }
+  // ---- pairs below the cutoff and at it, in this CTA and in the CTAs before it
+  uint32_t below = 0, at = 0;
+#pragma unroll 1
+  for (int u = 0, p = p_first; p < p_end; ++u, p += kThreads) {
+    const uint32_t v = key_of(u, p);
+    below += (kFromMask ? v != 0 : v < cutoff) ? 1u : 0u;
+    at += (!kFromMask && v == cutoff) ? 1u : 0u;
+  }
+  below = __reduce_add_sync(0xffffffffu, below);
+  at = __reduce_add_sync(0xffffffffu, at);
+  if (lane == 0 && below) atomicAdd(&s_total[0], below);
+  if (lane == 0 && at) atomicAdd(&s_total[1], at);
+  cluster_barrier();
+  below = at = 0;
+  for (int r = 0; r < rank; ++r) {
+    below += *cluster.map_shared_rank(&s_total[0], r);
+    at += *cluster.map_shared_rank(&s_total[1], r);
+  }
+  // ---- mask and counts in front of every tile, 32 tiles (one per warp) a step.  The first k ties are taken.
+  int32_t* tp = a.tile_prefix + (size_t)unit * a.tile_stride;
+#pragma unroll 1
+  for (int u = 0; u < steps; ++u) {
+    const int p = p_first + u * kThreads;
+    const uint32_t v = key_of(u, p);
+    const bool lt = p < p_end && (kFromMask ? v != 0 : v < cutoff);
+    const bool eq = !kFromMask && p < p_end && v == cutoff;
+    const uint32_t bl = __ballot_sync(0xffffffffu, lt), be = __ballot_sync(0xffffffffu, eq);
+    uint32_t* cnt = s_cnt[u & 1];
+    if (lane == 0) cnt[warp] = __popc(bl) | (__popc(be) << 16);
+    __syncthreads();
+    uint32_t c = cnt[lane];                                // (32 warps, 32 lanes; the sums stay below 2^16)
+    const uint32_t own = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, c, o);
+      if (lane >= o) c += t;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, c, 31), ex = __shfl_sync(0xffffffffu, c - own, warp);
+    const uint32_t tie_before = at + (ex >> 16);
+    if (!kFromMask && p < p_end) mask[p] = (lt || (eq && tie_before + __popc(be & ((1u << lane) - 1u)) < k)) ? 1 : 0;
+    const int tile = t0 + u * kWarps + warp;
+    if (lane == 0 && tile < t1) tp[tile] = (int32_t)(below + (ex & 0xffffu) + min(k, tie_before));
+    below += total & 0xffffu;
+    at += total >> 16;
+  }
+  if (ctas > 1) cluster.sync();                            // no CTA leaves while its shared memory is read
+}
+
+int most_pairs(const RoundTable& t) {
+  int pmax = 0;
+  for (int i = 0; i < t.nseq; ++i) pmax = pmax > t.s[i].P ? pmax : t.s[i].P;
+  return pmax;
+}
+
+// CTAs per unit: one for every 4096 pairs while they all fit the GPU (two per SM).  A cluster's barriers cost about
+// 1.5 us each: 8 units of 16336 pairs 17 us with four CTAs, 28 with eight; 256 units of 16336 pairs 32 us with
+// one, 85 with several waves of clusters of four.
+int cluster_of(const RoundTable& t, int Hkv) {
+  const int pmax = most_pairs(t);
+  int c = 1;
+  while (c < kMaxCluster && c * kPairsPerCta < pmax && (long long)c * 2 * Hkv * t.nseq <= 2 * 148) c *= 2;
+  return c;
+}
+
+template <int kMode>
+cudaError_t launch_select(const StatsTcArgs& sa, const SelectArgs& a, const RoundTable& t, cudaStream_t st) {
+  static KvsPerDeviceOnce configured;
+  cudaError_t e = configured.run([] {
+    return cudaFuncSetAttribute(select_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kKeep * kThreads * (int)sizeof(uint32_t));
+  });
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  const int c = cluster_of(t, a.Hkv);
+  cfg.gridDim = dim3((unsigned)c, (unsigned)a.Hkv, (unsigned)t.nseq);
+  cfg.blockDim = dim3(kThreads);
+  if (kMode != kMask) {
+    int nmax = 0;
+    for (int i = 0; i < t.nseq; ++i) nmax = nmax > t.s[i].n ? nmax : t.s[i].n;
+    const int ntiles = (nmax - t.off + KVS_CTILE - 1) / KVS_CTILE;
+    const int steps = ((ntiles + c - 1) / c + kWarps - 1) / kWarps;
+    cfg.dynamicSmemBytes = (size_t)(steps <= kKeep ? steps : kKeep) * kThreads * sizeof(uint32_t);   // (shorter units keep theirs)
+  }
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)c;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, select_kernel<kMode>, sa, a, t);
 }
 
 }  // namespace
 
-cudaError_t kvs_launch_select(const SelectArgs& a, const RoundTable& t, cudaStream_t st) {
-  dim3 grid(a.Hkv, t.nseq);
-  return kvs_launch_chained(select_pairs_kernel, grid, dim3(1024), 0, st, a, t);
+// The selection kernel adds the partials itself where they are few: up to 4096 pairs of at most two query blocks
+// (8 units of 2000 pairs, 3 partials: 7.9 us against 2.4 + 8.4; of 8192 pairs 27 against 6.6 + 12).  Its few CTAs
+// are slow readers: 8 units of 4000 pairs with 24 partials 33 us against 8 + 11.
+cudaError_t kvs_launch_finalize_select(const StatsTcArgs& sa, const SelectArgs& a, const RoundTable& t, cudaStream_t st,
+                                       int* kernels) {
+  *kernels = 1;
+  const int pmax = most_pairs(t);
+  if (pmax <= 0) return cudaSuccess;
+  if (a.select && pmax <= kFusedPairs && sa.nqblk <= 2) return launch_select<kFused>(sa, a, t, st);
+  cudaError_t e = kvs_launch_chained(finalize_kernel, dim3((pmax + 255) / 256, a.Hkv, t.nseq), dim3(256), 0, st, sa, t);
+  if (e != cudaSuccess || !a.select) return e;
+  *kernels = 2;
+  return launch_select<kScores>(sa, a, t, st);
+}
+
+cudaError_t kvs_launch_mask_prefix(const SelectArgs& a, const RoundTable& t, cudaStream_t st) {
+  return launch_select<kMask>(StatsTcArgs{}, a, t, st);
 }

@@ -18,8 +18,8 @@
 // with |vbar_j - o_q|^2 = |vbar_j|^2 - 2 T_jq / c_j + |o_q|^2.  The probability matrix never
 // leaves the SM.  The row norms |vbar|^2, |vbar_l + vbar_r|^2 and the adjacent-key cosine of
 // every pair come from the attention pass that precedes this kernel (it streams the same rows).
-// Every (query block, statistics group) writes its five sums per pair as a partial; a small
-// kernel adds the partials in a fixed order and forms score and the merge weight of
+// Every (query block, statistics group) writes its five sums per pair as a partial; the
+// selection (kvs_select.cu) adds the partials in a fixed order and forms score and the merge weight of
 // Eq. kstar_final (deterministic, no atomics, no hand-over between warps inside the tile loop).
 // A second instantiation serves the exact weight modes: a supplied loss gradient E (one row per
 // window query) takes the place of the attention output in the T products, and the statistics
@@ -398,52 +398,6 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
   if (threadIdx.x == 0 && misc->abort_flag && a.status_dev) atomicExch(a.status_dev, (int)KVS_ERR_TIMEOUT);
 }
 
-// Sum of the partials of all (query block, statistics group) pairs in a fixed order, then score and
-// left-key weight of each candidate pair.  Weight modes:
-//   0: the sums are norms; w = (N1_l - N12) / (N1_l - 2 N12 + N1_r)                        [Eq. kstar_final]
-//   1: they are the signed sums G11, G22, G12 of g_ij = E^T c_ij; w = (G11 + G12) / (G11 + 2 G12 + G22)
-//                                                                            [Eq. kstar_weight_final_rewrite]
-//   2: as 1 with the coupling dropped, w = G11 / (G11 + G22)                              [Eq. simplified_k]
-// A denominator that is not safely positive gives 1/2; the weight is clipped to [0, 1].
-__global__ void __launch_bounds__(256)
-stats_finalize_kernel(const StatsTcArgs a, const RoundTable tab) {
-  kvs_pdl_launch_dependents();
-  kvs_pdl_wait();
-  const SeqRound sr = tab.s[blockIdx.z];
-  if (sr.n <= 0) return;
-  const int unit = sr.b * a.Hkv + blockIdx.y;
-  const int p = blockIdx.x * 256 + threadIdx.x;
-  if (p >= sr.P) return;
-  const int jl = tab.off + 2 * p;
-  const int nsub = a.nqblk * kGroups;
-  float Al = 0.f, Ar = 0.f, N1l = 0.f, N1r = 0.f, N12 = 0.f;
-  for (int sb = 0; sb < nsub; ++sb) {
-    const size_t i = ((size_t)unit * nsub + sb) * a.pair_stride + p;
-    const float4 v = a.part4[i];
-    Al += v.x; Ar += v.y; N1l += v.z; N1r += v.w;
-    N12 += a.part1[i];
-  }
-  const float cosv = a.pair_norms[(size_t)unit * a.norm_stride + p].w;
-  const float mass = Al + Ar;
-  const float score = (a.score_mode == 0) ? mass * fmaxf(0.f, 1.f - cosv) : mass;
-  float w = 0.5f;
-  if (a.weight_mode == 0) {
-    const float D = N1l - 2.f * N12 + N1r;
-    if (D > 1e-6f * (N1l + N1r) && D < INFINITY) w = fminf(1.f, fmaxf(0.f, (N1l - N12) / D));
-  } else {
-    const float g12 = (a.weight_mode == 2) ? 0.f : N12;
-    const float gamma = N1l + 2.f * g12 + N1r;
-    if (gamma > 1e-6f * (fabsf(N1l) + fabsf(N1r)) && gamma < INFINITY) w = fminf(1.f, fmaxf(0.f, (N1l + g12) / gamma));
-  }
-  const size_t pi = (size_t)unit * a.pair_stride + p;
-  a.score[pi] = fabsf(score);
-  a.w[pi] = w;
-  if (a.N12) a.N12[pi] = N12;
-  if (a.cosv) a.cosv[pi] = cosv;
-  if (a.A) { a.A[(size_t)unit * a.n_max + jl] = Al; a.A[(size_t)unit * a.n_max + jl + 1] = Ar; }
-  if (a.N1) { a.N1[(size_t)unit * a.n_max + jl] = N1l; a.N1[(size_t)unit * a.n_max + jl + 1] = N1r; }
-}
-
 }  // namespace
 
 cudaError_t kvs_launch_stats_tc(const StatsTcArgs& a, const RoundTable& t, const CUtensorMap& tmKp,
@@ -457,13 +411,7 @@ cudaError_t kvs_launch_stats_tc(const StatsTcArgs& a, const RoundTable& t, const
   });
   if (ce != cudaSuccess) return ce;
   dim3 grid(a.nqblk * a.splits, a.Hkv, t.nseq);
-  cudaError_t e = (a.weight_mode == 0)
+  return (a.weight_mode == 0)
       ? kvs_launch_chained(hessian_stats_tc<false>, grid, dim3(kThreads), kSmemBytes, st, a, t, tmKp, tmVp, tmQ, tmOhi, tmOlo)
       : kvs_launch_chained(hessian_stats_tc<true>, grid, dim3(kThreads), kSmemBytes, st, a, t, tmKp, tmVp, tmQ, tmOhi, tmOlo);
-  if (e != cudaSuccess) return e;
-  int pmax = 0;
-  for (int i = 0; i < t.nseq; ++i) pmax = pmax > t.s[i].P ? pmax : t.s[i].P;
-  if (pmax <= 0) return cudaSuccess;
-  dim3 fgrid((pmax + 255) / 256, a.Hkv, t.nseq);
-  return kvs_launch_chained(stats_finalize_kernel, fgrid, dim3(256), 0, st, a, t);
 }

@@ -1,0 +1,47 @@
+"""The selection of a round as integer work: the mask must hold the R smallest (score bits, index) of the scores
+that the same call returns, and the compaction must move every slot accordingly.  Sizes cover the fused and the
+separate finalize, one to eight CTAs per unit, keys that do not fit a CTA's shared memory, and ties at the cutoff."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+# KV heads, slots, keys repeated every `period` slots (0: none; with it most scores occur many times)
+@pytest.mark.parametrize("hkv,n,period,first_round", [
+    (2, 300, 0, 0), (3, 8200, 0, 1), (3, 8400, 64, 0), (8, 20011, 128, 1), (2, 140000, 0, 0), (2, 140000, 512, 1),
+    (160, 66200, 512, 0)])
+def test_mask_is_the_smallest_scores(hkv, n, period, first_round):
+    import torch
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + period)
+    K, V = (torch.empty(1, hkv, n, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    for x in (K, V):
+        rows = torch.randn(hkv, period or n, 128, generator=g, device="cuda").to(torch.bfloat16)
+        x[0] = rows.repeat(1, n // (period or n) + 1, 1)[:, :n]
+    counts = torch.ones(1, hkv, n, dtype=torch.int32, device="cuda")
+    q = torch.randn(1, hkv, 4, 128, generator=g, device="cuda").to(torch.bfloat16)
+    p = kb.make_params(K, V, hkv, 4, causal=False, first_round=first_round)
+    ws = torch.empty(kb.kvs_workspace_size(p, n, 0), dtype=torch.uint8, device="cuda")
+    score, w = (torch.zeros(1, hkv, n // 2, device="cuda") for _ in range(2))
+    mask = torch.zeros(1, hkv, n // 2, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    _, off, P, R = kb.kvs_round_plan(p, n, n - n // 5)[0]
+    kb.kvs_window_stats(p, K, V, counts, q, [n], [n - n // 5], ws, score=score, w=w, mask=mask, status_dev=status)
+    want = torch.zeros_like(mask)
+    order = torch.sort(score[0, :, :P], dim=-1, stable=True).indices[:, :R]
+    want[0].scatter_(1, order, 1)
+    assert torch.equal(mask, want)
+    if period:
+        cut = score[0].gather(1, order[:, -1:])
+        assert int((score[0, :, :P] == cut).sum(1).min()) > 1       # the cutoff is a tie
+    # the same decision through kvs_compact: the map counts the merged pairs before every slot
+    index = torch.zeros(1, hkv, n, dtype=torch.int32, device="cuda")
+    kb.kvs_compact(p, K, V, counts, mask, w, [n], [R], ws, new_index=index, status_dev=status)
+    before = torch.zeros(hkv, n, dtype=torch.int32, device="cuda")
+    before[:, off + 1:off + 2 * P:2] = want[0, :, :P].int()          # the right member of a merged pair moves up by one
+    slots = torch.arange(n, dtype=torch.int32, device="cuda")
+    assert torch.equal(index[0], slots - before.cumsum(1, dtype=torch.int32))
+    assert status.item() == 0
