@@ -519,8 +519,10 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
       int cn0 = 1, cn1 = 1;
       auto fetch_counts = [&](int li) {
         const int j = (t_begin + li) * kTile - shift + ch * 64 + lane;
-        cn0 = (li < my_tiles && j >= 0 && j < n) ? ldg_here(Cb + j) : 1;
-        cn1 = (li < my_tiles && j + 32 < n) ? ldg_here(Cb + j + 32) : 1;
+        // (outside the sequence P' is 0 and any finite count will do; no condition: a predicated load is waited for
+        // where it is issued, which cost 700 cycles a tile)
+        cn0 = ldg_here(Cb + min(max(j, 0), n - 1));
+        cn1 = ldg_here(Cb + min(max(j + 32, 0), n - 1));
       };
       fetch_counts(team);
       for (int li = team; li < my_tiles; li += 2) {
@@ -555,7 +557,12 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
         tmem_ld16(scol, xa);
         // rows of the V tile outside the sequence may hold anything: the team zeroes them
         if (tile_row0 < 0 || tile_row0 + kTile > n) {
-          if (!(alive = warp_wait(&misc->vfull[gi % kVStages], (gi / kVStages) & 1, abort_flag, lane))) { tmem_ld_wait(); continue; }
+          // (the logits run ahead of V by more than its stages: the stage's last use must be over before its barrier's
+          // phase says anything about this tile)
+          static_assert(kVStages == 2, "the tile that used the stage before");
+          if (gi >= 2) alive = warp_wait(&misc->pvdone[(gi - 2) % kSBufs], ((gi - 2) / kSBufs) & 1, abort_flag, lane);
+          if (alive) alive = warp_wait(&misc->vfull[gi % kVStages], (gi / kVStages) & 1, abort_flag, lane);
+          if (!alive) { tmem_ld_wait(); continue; }
           uint8_t* vt = smem + kSmemV + (gi % kVStages) * kOperand;
           for (int it = (threadIdx.x - 64) & 255; it < kTile * 16; it += 256) {
             const int r = it >> 4, c16 = it & 15;
