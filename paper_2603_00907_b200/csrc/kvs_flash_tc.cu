@@ -23,12 +23,13 @@
 // larger by tens of powers of two.  So no tile but the first needs a maximum, and no warp waits for
 // another one.  If a part of l exceeds 2^60 all the same, the CTA walks its range twice more, once for
 // the true maxima and once with them.  (With a running maximum, exchanged between the two warps of a row and
-// between the teams on every tile: 1024 query rows over 131072 slots, 8 heads, 0.85 ms; so: 0.67 ms.)
+// between the teams on every tile: 1024 query rows over 131072 slots, 8 heads, 0.83 ms; so: 0.65 ms, 2 000 cycles a
+// tile of which the tensor core needs 1 536.)
 //
-// Four more warps serve the statistics pass that follows the window attention: tiles are then
+// Eight more warps serve the statistics pass that follows the window attention: tiles are then
 // aligned with the round's candidate pairs, and for every pair they form |vbar_l|^2, |vbar_r|^2,
-// |vbar_l + vbar_r|^2 and the adjacent-key cosine from the staged rows (diagonals of small
-// mma.sync products), so that the statistics kernel does not have to touch the rows for it.
+// |vbar_l + vbar_r|^2 and the adjacent-key cosine from the staged rows, so that the statistics
+// kernel does not have to touch the rows for it.  The query blocks of a KV head share that work.
 #include "kvs_internal.h"
 #include "kvs_sm100.cuh"
 
@@ -43,9 +44,9 @@ constexpr int kKStages = 3, kVStages = 2;
 constexpr int kAhead = 4;                  // tiles requested into L2 ahead of their load
 constexpr int kSmemQ = 0, kSmemK = kOperand, kSmemV = kSmemK + kKStages * kOperand;
 constexpr int kSmemMisc = kSmemV + kVStages * kOperand;
-constexpr int kSoftmaxWarps = 16, kNormWarps = 4;
+constexpr int kSoftmaxWarps = 16, kNormWarps = 8;
 constexpr int kPvWarp = 2 + kSoftmaxWarps + kNormWarps;          // the warp that issues the P V products
-constexpr int kThreads = (kPvWarp + 1) * 32;   // warp 0: TMA, 1: S products, 2-17: softmax, 18-21: pair norms, 22: P V products
+constexpr int kThreads = (kPvWarp + 1) * 32;   // warp 0: TMA, 1: S products, 2-17: softmax, 18-25: pair norms, 26: P V products
 constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: a part of l beyond this asks for another walk
 constexpr int kSBufs = 3;                  // logit / P' buffers in tensor memory
 
@@ -101,52 +102,47 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t saddr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(saddr)
-               : "memory");
-}
-// D(16x8, fp32) += A(16x16, bf16, row major) B(16x8, bf16, column major)
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-      "{%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// For the 8 pairs (rows 2i, 2i+1) of rows [row0, row0 + 16) of one staged operand: |x_l|^2,
-// |x_r|^2 and <x_l, x_r>, delivered to lanes 0-7 (and again to lanes 8-15).  The 16 rows are the
-// A operand and, eight at a time, the B operand of small tensor-core products: the wanted values
-// sit on and next to the diagonal of the 16 x 16 Gram matrix.  Every 8 x 8 fragment is eight
-// consecutive rows, which the 128-byte swizzle spreads over all banks.
-__device__ __forceinline__ void pair_dots8(const uint8_t* tile, int row0, int lane, float& ll, float& rr, float& lr) {
-  const uint32_t base = smem_u32(tile);
-  const int mtx = lane >> 3, rin = lane & 7;                // ldmatrix: this lane feeds row rin of matrix mtx
-  const int row = row0 + (mtx & 1) * 8 + rin;               // matrices 0,2: rows 0-7; 1,3: rows 8-15
-  uint32_t fr[8][4];
+// |x_l|^2, |x_r|^2 and <x_l, x_r> of the 4 * steps pairs (rows 2 i, 2 i + 1) from row row0 (a multiple of 8) of one
+// staged operand, in fp32; lane L gets those of pair pair_of_lane(L), if there is one.  The eight lanes of a
+// quarter warp read the eight 16-byte pieces of half a row: with the 128-byte swizzle no bank conflicts.  Plain FMAs,
+// two channels per instruction, in a loop that stays rolled.  Small mma.sync products (diagonals of Gram
+// matrices) wait for the tensor core behind its own products: 2 400 cycles per operand and tile on four warps,
+// where the softmax needs 2 000.  Unrolled FMAs, 1 300, no longer fit the instruction cache together with the
+// softmax, and both ran at half their speed (clock64).
+__device__ __forceinline__ int pair_of_lane(int lane) { return 4 * ((lane >> 1) & 3) + (lane >> 3); }
+__device__ __forceinline__ void pair_dots(const uint8_t* tile, int row0, int steps, int lane, float& ll, float& rr, float& lr) {
+  const int c = lane & 7, rl0 = row0 + 2 * (lane >> 3);
+  // (the rows of the steps are 8 apart: their swizzle is the same)
+  const uint8_t* pl = tile + rl0 * 128 + ((c ^ (rl0 & 7)) << 4);
+  const uint8_t* pr = tile + (rl0 + 1) * 128 + ((c ^ ((rl0 + 1) & 7)) << 4);
+#pragma unroll 1
+  for (int it = 0; it < steps; ++it, pl += 1024, pr += 1024) {
+    float2 all = make_float2(0.f, 0.f), arr = all, alr = all;
 #pragma unroll
-  for (int kk = 0; kk < 8; ++kk) {
-    const int chunk = 2 * (kk & 3) + (mtx >> 1);            // 16-byte chunk inside the 128-byte row
-    ldmatrix_x4(fr[kk], base + (kk >> 2) * kHalf + row * 128 + ((chunk ^ (row & 7)) << 4));
-  }
-  float d1[4] = {0.f, 0.f, 0.f, 0.f}, d2[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int hf = 0; hf < 2; ++hf) {
+      const uint4 l = *reinterpret_cast<const uint4*>(pl + hf * kHalf), r = *reinterpret_cast<const uint4*>(pr + hf * kHalf);
+      const uint32_t lw[4] = {l.x, l.y, l.z, l.w}, rw[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-  for (int kk = 0; kk < 8; ++kk) {
-    mma16816(d1, fr[kk], fr[kk][0], fr[kk][2]);             // columns = rows 0-7
-    mma16816(d2, fr[kk], fr[kk][1], fr[kk][3]);             // columns = rows 8-15
+      for (int i = 0; i < 4; ++i) {
+        const float2 lf = make_float2(bf16lo(lw[i]), bf16hi(lw[i])), rf = make_float2(bf16lo(rw[i]), bf16hi(rw[i]));
+        all = __ffma2_rn(lf, lf, all);
+        arr = __ffma2_rn(rf, rf, arr);
+        alr = __ffma2_rn(lf, rf, alr);
+      }
+    }
+    float o[3] = {all.x + all.y, arr.x + arr.y, alr.x + alr.y};
+#pragma unroll
+    for (int k = 4; k > 0; k >>= 1)
+#pragma unroll
+      for (int x = 0; x < 3; ++x) o[x] += __shfl_xor_sync(0xffffffffu, o[x], k);
+    if (((lane >> 1) & 3) == it) { ll = o[0]; rr = o[1]; lr = o[2]; }
   }
-  // lane 4 g + t holds rows g and g + 8, columns 2 t and 2 t + 1.  Pair q < 4 (rows 2q, 2q+1, first
-  // product): lane 9 q has <l,l> and <l,r>, lane 9 q + 4 has <r,r>; pair 4 + q the same lanes, in
-  // the lower half of the second product.
-  const int q = lane & 3, srcl = 9 * q, srcr = 9 * q + 4;
-  const bool upper = (lane & 4) != 0;
-  const float ll1 = __shfl_sync(0xffffffffu, d1[0], srcl), ll2 = __shfl_sync(0xffffffffu, d2[2], srcl);
-  const float lr1 = __shfl_sync(0xffffffffu, d1[1], srcl), lr2 = __shfl_sync(0xffffffffu, d2[3], srcl);
-  const float rr1 = __shfl_sync(0xffffffffu, d1[1], srcr), rr2 = __shfl_sync(0xffffffffu, d2[3], srcr);
-  ll = upper ? ll2 : ll1;
-  lr = upper ? lr2 : lr1;
-  rr = upper ? rr2 : rr1;
+}
+// 1 / sqrt(x): the hardware's estimate and a Newton step (the compiler's square root and division took 300 cycles a tile)
+__device__ __forceinline__ float rsqrt_newton(float x) {
+  x = fmaxf(x, 1e-36f);
+  const float y = rsqrtf(x);
+  return fmaf(y * 0.5f, fmaf(-x * y, y, 1.f), y);
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -187,21 +183,22 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     }
     return;
   }
-  // the pair norms of a KV head are shared work: the first query block forms the key cosines, the
-  // second one (the first again, if there is only one) the value norms
-  const bool norm_k = a.pair_norms != nullptr && qblk == 0;
-  const bool norm_v = a.pair_norms != nullptr && qblk == (a.nqblk > 1 ? 1 : 0);
+  // the pair norms of a KV head are shared work of its query blocks: tile t's key cosines belong to block
+  // 2 t mod nqblk, its value norms to block 2 t + 1 mod nqblk
+  const bool norm_k = a.pair_norms != nullptr && ((a.nqblk & 1) || !(qblk & 1));
+  const bool norm_v = a.pair_norms != nullptr && ((a.nqblk & 1) || (qblk & 1));
+  const int norm_arrivals = norm_k && norm_v ? kNormWarps / 2 : kNormWarps;   // per tile and operand
 
   if (threadIdx.x == 0) {
     // the K rows of a stage are free once the logits are formed, the V rows only after P V: two
     // rings, so that the next K tiles are requested a whole softmax earlier than the next V tile
     for (int s = 0; s < kKStages; ++s) {
       mbar_init(&misc->kfull[s], 1);
-      mbar_init(&misc->kfree[s], norm_k ? 1 + kNormWarps : 1);   // MMA commit (+ the pair-norm warps)
+      mbar_init(&misc->kfree[s], norm_k ? 1 + norm_arrivals : 1);   // MMA commit (+ the pair-norm warps)
     }
     for (int s = 0; s < kVStages; ++s) {
       mbar_init(&misc->vfull[s], 1);
-      mbar_init(&misc->vfree[s], norm_v ? 1 + kNormWarps : 1);
+      mbar_init(&misc->vfree[s], norm_v ? 1 + norm_arrivals : 1);
     }
     for (int b = 0; b < kSBufs; ++b) {
       mbar_init(&misc->sfull[b], 1);
@@ -358,75 +355,61 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
       }
     }
   } else if (warp >= 2 + kSoftmaxWarps) {
-    // ================================================================ pair-norm warps (18-21)
+    // ================================================================ pair-norm warps
     if (norm_k || norm_v) {
-      const int nw = warp - (2 + kSoftmaxWarps);                 // rows [32 nw, 32 nw + 32) of every tile
+      // A CTA with both operands to do gives the keys to warps 0-3 and the values to warps 4-7, 32 rows of a tile each;
+      // one with a single operand gives it to all eight, 16 rows each.  (Every warp sees every tile of its operand:
+      // one that skips tiles could take a barrier's phase for an older one.)
+      static_assert(kNormWarps == 8, "the split below");
+      const int nw = warp - (2 + kSoftmaxWarps);
+      const bool both = norm_k && norm_v;
+      const int op = both ? nw >> 2 : (norm_v ? 1 : 0);          // 0: keys, 1: values
+      const int steps = both ? 4 : 2, row0 = both ? 32 * (nw & 3) : 16 * nw;
+      uint64_t* full = op ? misc->vfull : misc->kfull;
+      uint64_t* freed = op ? misc->vfree : misc->kfree;
+      const int stages = op ? kVStages : kKStages;
+      const uint8_t* rows = smem + (op ? kSmemV : kSmemK);
       const int off = tab.off;
       const int32_t* Cn = a.counts + (size_t)unit * a.n_max;
-      const int pl = lane & 15;                                  // lanes 0-15 own the warp's 16 pairs
-      // counts of the next tile's pair travel while the current tile is processed
-      int cl_next = 1, cr_next = 1;
-      if (norm_v) {
-        const int sl = t_begin * kTile - shift + nw * 32 + 2 * pl;
-        if (sl >= off && ((sl - off) >> 1) < sr.P) { cl_next = ldg_here(Cn + sl); cr_next = ldg_here(Cn + sl + 1); }
-      }
+      float* norms = reinterpret_cast<float*>(a.pair_norms + (size_t)unit * a.pair_stride);
+      // left slot of this lane's pair; the counts of a slot (no condition: a predicated load is waited for where it is issued)
+      int slot_l = t_begin * kTile - shift + row0 + 2 * pair_of_lane(lane);
+      const bool has_pair = (lane & 1) == 0 && ((lane >> 1) & 3) < steps;
+      auto count_at = [&](int j) { return ldg_here(Cn + min(max(j, 0), n - 1)); };
+      int cl_next = count_at(slot_l), cr_next = count_at(slot_l + 1);
       bool ok_all = true;
-      for (int li = 0; li < my_tiles; ++li) {
-        const int ks = li % kKStages, kp = (li / kKStages) & 1, vs = li % kVStages, vp = (li / kVStages) & 1;
-        const int slot_l = (t_begin + li) * kTile - shift + nw * 32 + 2 * pl;   // left slot of this lane's pair
+      int st = 0, ph = 0;
+#pragma unroll 1
+      for (int li = 0; li < my_tiles; ++li, slot_l += kTile) {
         const int p = (slot_l - off) >> 1;
-        const bool pair_ok = lane < 16 && slot_l >= off && p < sr.P;
+        const bool mine = (2 * (t_begin + li) + op) % a.nqblk == qblk;
         const int cl = cl_next, cr = cr_next;
-        if (norm_v && li + 1 < my_tiles) {
-          const int sl = slot_l + kTile;
-          cl_next = cr_next = 1;
-          if (sl >= off && ((sl - off) >> 1) < sr.P) { cl_next = ldg_here(Cn + sl); cr_next = ldg_here(Cn + sl + 1); }
-        }
-        float* out = reinterpret_cast<float*>(a.pair_norms + (size_t)unit * a.pair_stride + (pair_ok ? p : 0));
-        const uint8_t* kt = smem + kSmemK + ks * kOperand;
-        const uint8_t* vt = smem + kSmemV + vs * kOperand;
-        int ok = 1;
-        if (norm_k) {
-          if (lane == 0) ok = mbar_wait(&misc->kfull[ks], kp, abort_flag) ? 1 : 0;
-          if (!__shfl_sync(0xffffffffu, ok, 0)) { ok_all = false; break; }
-          float ll[2], rr[2], lr[2];
-          pair_dots8(kt, nw * 32, lane, ll[0], rr[0], lr[0]);
-          pair_dots8(kt, nw * 32 + 16, lane, ll[1], rr[1], lr[1]);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&misc->kfree[ks]);          // the K rows are no longer needed here
-          const bool b = (lane >> 3) & 1;
-          const float kll = b ? ll[1] : ll[0], krr = b ? rr[1] : rr[0], klr = b ? lr[1] : lr[0];
-          if (pair_ok) out[3] = klr / fmaxf(sqrtf(kll) * sqrtf(krr), 1e-30f);
-        }
-        if (norm_v) {
-          if (lane == 0) ok = mbar_wait(&misc->vfull[vs], vp, abort_flag) ? 1 : 0;
-          if (!__shfl_sync(0xffffffffu, ok, 0)) { ok_all = false; break; }
-          float ll[2], rr[2], lr[2];
-          pair_dots8(vt, nw * 32, lane, ll[0], rr[0], lr[0]);
-          pair_dots8(vt, nw * 32 + 16, lane, ll[1], rr[1], lr[1]);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&misc->vfree[vs]);
-          const bool b = (lane >> 3) & 1;
-          const float vll = b ? ll[1] : ll[0], vrr = b ? rr[1] : rr[0], vlr = b ? lr[1] : lr[0];
-          if (pair_ok) {
-            const float icl = 1.f / (float)cl, icr = 1.f / (float)cr;
-            const float r2l = vll * icl * icl, r2r = vrr * icr * icr;
-            out[0] = r2l; out[1] = r2r; out[2] = r2l + r2r + 2.f * vlr * icl * icr;
-          }
+        cl_next = count_at(slot_l + kTile); cr_next = count_at(slot_l + kTile + 1);
+        if (!warp_wait(full + st, ph, abort_flag, lane)) { ok_all = false; break; }
+        float ll = 0.f, rr = 0.f, lr = 0.f;
+        if (mine) pair_dots(rows + st * kOperand, row0, steps, lane, ll, rr, lr);
+        // the rows are no longer needed here.  (The test is always true: it makes the arrival wait for the loads, whose
+        // results the compiler may otherwise collect after it.)
+        __syncwarp();
+        if (lane == 0 && !(ll < -1.f)) mbar_arrive(freed + st);
+        if (++st == stages) { st = 0; ph ^= 1; }
+        if (!mine || !has_pair || slot_l < off || p >= sr.P) continue;
+        if (op) {
+          const float icl = __fdividef(1.f, (float)cl), icr = __fdividef(1.f, (float)cr);   // (small integers)
+          const float r2l = ll * icl * icl, r2r = rr * icr * icr;
+          norms[4 * (size_t)p] = r2l; norms[4 * (size_t)p + 1] = r2r; norms[4 * (size_t)p + 2] = r2l + r2r + 2.f * lr * icl * icr;
+        } else {
+          norms[4 * (size_t)p + 3] = lr * rsqrt_newton(ll) * rsqrt_newton(rr);
         }
       }
+      __syncwarp();
       // further walks: the rows are handed back as they come
       if (lane == 0 && ok_all) {
         const int end = walks() * my_tiles;
         for (int gi = my_tiles; gi < end; ++gi) {
-          if (norm_k) {
-            if (!mbar_wait(&misc->kfull[gi % kKStages], (gi / kKStages) & 1, abort_flag)) break;
-            mbar_arrive(&misc->kfree[gi % kKStages]);
-          }
-          if (norm_v) {
-            if (!mbar_wait(&misc->vfull[gi % kVStages], (gi / kVStages) & 1, abort_flag)) break;
-            mbar_arrive(&misc->vfree[gi % kVStages]);
-          }
+          if (!mbar_wait(full + st, ph, abort_flag)) break;
+          mbar_arrive(freed + st);
+          if (++st == stages) { st = 0; ph ^= 1; }
         }
       }
       __syncwarp();
@@ -553,8 +536,6 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
           warp_arrive(&misc->pready[b][1], lane);
           continue;
         }
-        float xa[16], xb[16];
-        tmem_ld16(scol, xa);
         // rows of the V tile outside the sequence may hold anything: the team zeroes them
         if (tile_row0 < 0 || tile_row0 + kTile > n) {
           // (the logits run ahead of V by more than its stages: the stage's last use must be over before its barrier's
@@ -562,7 +543,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
           static_assert(kVStages == 2, "the tile that used the stage before");
           if (gi >= 2) alive = warp_wait(&misc->pvdone[(gi - 2) % kSBufs], ((gi - 2) / kSBufs) & 1, abort_flag, lane);
           if (alive) alive = warp_wait(&misc->vfull[gi % kVStages], (gi / kVStages) & 1, abort_flag, lane);
-          if (!alive) { tmem_ld_wait(); continue; }
+          if (!alive) continue;
           uint8_t* vt = smem + kSmemV + (gi % kVStages) * kOperand;
           for (int it = (threadIdx.x - 64) & 255; it < kTile * 16; it += 256) {
             const int r = it >> 4, c16 = it & 15;
@@ -571,21 +552,20 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
           }
           fence_proxy_async();                             // the tensor core reads these rows
         }
-        // two halves of 32 slots (one copy of the code, run twice, keeps the roles' code within the instruction cache)
+        // (one copy of the code, run four times: the roles' code has to fit the instruction cache; the other warps cover
+        // the latency of the load)
 #pragma unroll 1
-        for (int hf = 0; hf < 2; ++hf) {
-          const uint32_t col = scol + hf * 32;
+        for (int c = 0; c < 4; ++c) {
+          float x[16];
+          tmem_ld16(scol + c * 16, x);
           tmem_ld_wait();
-          tmem_ld16(col + 16, xb);                         // in flight while the first 16 are worked on
-          mask16(j0 + hf * 32, xa);
-          emit16(col, xa, cnt + hf * 32);
-          tmem_ld_wait();
-          if (hf == 0) tmem_ld16(col + 32, xa);
-          mask16(j0 + hf * 32 + 16, xb);
-          emit16(col + 16, xb, cnt + hf * 32 + 16);
-          tmem_st_wait();
-          tc_fence_before();
-          warp_arrive(&misc->pready[b][hf], lane);
+          mask16(j0 + c * 16, x);
+          emit16(scol + c * 16, x, cnt + c * 16);
+          if (c & 1) {
+            tmem_st_wait();
+            tc_fence_before();
+            warp_arrive(&misc->pready[b][c >> 1], lane);
+          }
         }
       }
       gi_last = (walk + 1) * my_tiles - 1;
