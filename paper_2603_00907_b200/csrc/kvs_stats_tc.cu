@@ -4,11 +4,12 @@
 // bf16 terms, stay in shared memory) and walks a range of tiles of 128 candidate pairs.
 // A 5-D view of the cache, [128, parity, slot/2, head, sequence], lets TMA bring the left
 // members and the right members of the 128 pairs as two separate row tiles, so that TMEM
-// lane p holds everything of pair p.  For each half of 64 queries
+// lane p holds everything of pair p.  For each step of up to 64 queries
 //   S_l = K_l Q^T, S_r = K_r Q^T                    (logits, fp32 in TMEM)
 //   T_l = Vsum_l (O_hi + O_lo)^T, T_r likewise      (value/output inner products)
-// go into one of two TMEM buffers; while the statistics warps reduce one half, the tensor
-// core fills the other.  Two threads (in two warps, each chosen with elect.sync) issue the
+// go into one of two TMEM buffers; while the statistics warps reduce one step, the tensor
+// core fills the other buffer with the next (of the same tile, or of the next tile where a block has
+// no more than 64 queries: 16 x 8 units of 16 K pairs and 64 window rows 233 -> 198 us).  Two threads (in two warps, each chosen with elect.sync) issue the
 // products, one the chains of the left members and one those of the right members: one thread
 // alone measured 2 % slower.  Each statistics thread owns one pair
 // and a share of the queries and reduces, in registers and with no cross-lane traffic,
@@ -25,6 +26,12 @@
 // window query) takes the place of the attention output in the T products, and the statistics
 // warps sum the signed scalars g_ij = E^T c_ij instead of the norms [Section 4.2, text before
 // Eq. h_rank1_unified; Eq. kstar_weight_final_rewrite].
+// What bounds it (256 units of 16 K pairs, 128 queries each, 906 us, 6500 cycles a tile): the special-function
+// pipe needs 5120 cycles a tile (the arithmetic alone, without waits, runs in 5500), the operand reads of
+// the products 4600 of the shared-memory pipe's cycles, and the chip holds 1.6 to 1.7 GHz under this mix.  Tried
+// and slower: operands of the pairs copied to tensor memory (products half as long, 32 queries a step,
+// sixteen statistics warps: +4 %), a team of warps for each buffer (+3 % with sixteen, +8 % with eight), one of the
+// two exponentials by a polynomial on the FMA pipe (+1 to 4 %).
 // Every synchronisation is an mbarrier with a bounded wait, so a warp that gives up can never
 // leave another one stuck.
 #include "kvs_internal.h"
@@ -36,16 +43,14 @@ namespace {
 
 constexpr int kPairs = 128;                // candidate pairs per tile = TMEM lanes
 constexpr int kQB = 128;                   // queries per CTA
-constexpr int kQH = 64;                    // queries per accumulator half
+constexpr int kQH = 64;                    // queries per accumulator buffer, at most
 constexpr int kHalf = 16384;               // bytes of a [128 rows x 64 bf16] swizzled sub-tile
 constexpr int kOperand = 2 * kHalf;        // a [128 x 128] bf16 operand
 constexpr int kSmemQ = 0, kSmemOhi = kOperand, kSmemOlo = 2 * kOperand;
 constexpr int kSmemKl = 3 * kOperand, kSmemKr = 4 * kOperand, kSmemVl = 5 * kOperand, kSmemVr = 6 * kOperand;
 constexpr int kSmemMisc = 7 * kOperand;
-constexpr int kGroups = KVS_STATS_GROUPS;  // statistics groups: a group reduces a share of the queries of every half
+constexpr int kGroups = KVS_STATS_GROUPS;  // statistics groups: a group reduces a share of the queries of every step
 constexpr int kChunk = 8;                  // queries per round of TMEM loads
-constexpr bool kDoubleBuffer = kGroups < 4;   // the next chunk's loads in flight while one chunk is reduced
-constexpr int kChunks = kQH / kChunk;      // chunks of a half, dealt out to the groups as evenly as they go
 constexpr int kStatWarps = 4 * kGroups;
 constexpr int kIssuers = 2;
 constexpr int kFirstStat = 1 + kIssuers;   // warp 0: TMA, warps 1-2: product issuers, then the statistics warps
@@ -123,7 +128,12 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
     return;
   }
   const int my_tiles = t_end - t_begin;
-  const int nh = (min(kQB, a.M - qblk * kQB) > kQH) ? 2 : 1;   // accumulator halves in use
+  // a block of more than 64 queries takes two steps per tile, of half the queries each (to a multiple
+  // of 16: eight sequences of 8 K pairs with blocks of 128 and 96 rows, 140 -> 134 us); a smaller block takes
+  // one.  The steps go to the two accumulator buffers in turn.
+  const int rows = min(kQB, a.M - qblk * kQB);
+  const int nh = rows > kQH ? 2 : 1;
+  const int qn = ((rows + nh - 1) / nh + 15) & ~15;    // queries of a step
 
   // (read from one lane, so that the compiler knows the warp index and all that follows from it
   // -- roles, TMEM and barrier addresses -- to be the same in every lane)
@@ -223,19 +233,20 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
     if (elect_one()) {
       const bool right = warp != 1;
       // descriptors are kept as a constant high word and low words that only need an addition per product
-      constexpr uint32_t idesc = idesc_bf16(kPairs, kQH);
+      const uint32_t idesc = idesc_bf16(kPairs, qn);
       const uint32_t dhi = (uint32_t)(smem_desc_sw128(0, 16, 1024) >> 32);
       auto dlo = [&](int off_bytes) { return (uint32_t)smem_desc_sw128(smem_u32(smem + off_bytes), 16, 1024); };
       const uint32_t q_lo = dlo(kSmemQ), ohi_lo = dlo(kSmemOhi), olo_lo = dlo(kSmemOlo);
       const uint32_t k_lo = dlo(right ? kSmemKr : kSmemKl), v_lo = dlo(right ? kSmemVr : kSmemVl);
       bool ok = mbar_wait(&misc->qfull, 0, abort_flag);
+      uint32_t it = 0;
       for (int li = 0; ok && li < my_tiles; ++li) {
         if (!mbar_wait(&misc->kfull, li & 1, abort_flag)) break;
-        for (int hq = 0; hq < nh; ++hq) {
-          if (!mbar_wait(&misc->tfree[hq], (li & 1) ^ 1, abort_flag)) { ok = false; break; }
+        for (int hq = 0; hq < nh; ++hq, ++it) {
+          if (!mbar_wait(&misc->tfree[it & 1], ((it >> 1) & 1) ^ 1, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t d0 = tmem + hq * 256 + (right ? 64u : 0u);
-          const uint32_t qrow = (uint32_t)(hq * (kQH * 128)) >> 4;   // rows 64.. of the query-side operands
+          const uint32_t d0 = tmem + (it & 1) * 256 + (right ? 64u : 0u);
+          const uint32_t qrow = (uint32_t)(hq * qn * 128) >> 4;   // rows qn.. of the query-side operands
           const uint32_t qh = q_lo + qrow, oh = ohi_lo + qrow, ol = olo_lo + qrow;
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk) {
@@ -253,7 +264,7 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
             if (kk == 0) umma_ss<false>(d0 + 128, v_lo, dhi, ob, dhi, idesc);
             else umma_ss<true>(d0 + 128, v_lo + o, dhi, ob, dhi, idesc);
           }
-          tc_commit(&misc->tfull[hq]);
+          tc_commit(&misc->tfull[it & 1]);
         }
         if (!ok) break;
         tc_commit(&misc->vfree);
@@ -272,21 +283,25 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
     float4* out4 = a.part4 + sub * a.pair_stride;
     float* out1 = a.part1 + sub * a.pair_stride;
     // norms and counts of the next tile's pair travel while the current tile is reduced
-    float4 nrm_next = make_float4(1.f, 1.f, 1.f, 0.f);
-    int cl_next = 1, cr_next = 1;
-    {
-      const int p = t_begin * kPairs + lane_p;
-      if (p < P) { nrm_next = ldg_here(norms + p); cl_next = ldg_here(Cb + off + 2 * p); cr_next = ldg_here(Cb + off + 2 * p + 1); }
-    }
+    // (never predicated: the compiler waits for a predicated load where it stands; a lane past the last
+    // pair reads that pair's values and its sums are not stored)
+    float4 nrm_next;
+    int cl_next, cr_next;
+    auto fetch = [&](int pn) {
+      const int pc = min(pn, P - 1);
+      nrm_next = ldg_here(norms + pc);
+      cl_next = ldg_here(Cb + off + 2 * pc);
+      cr_next = ldg_here(Cb + off + 2 * pc + 1);
+    };
+    fetch(t_begin * kPairs + lane_p);
+    const int nchunk = qn / kChunk;
+    uint32_t it = 0;
     for (int li = 0; li < my_tiles; ++li) {
       const int tile = t_begin + li;
       const int p = tile * kPairs + lane_p;               // candidate pair of this thread
       const float4 nrm = nrm_next;
       const float cl = (float)cl_next, cr = (float)cr_next;
-      if (li + 1 < my_tiles) {
-        const int pn = p + kPairs;
-        if (pn < P) { nrm_next = ldg_here(norms + pn); cl_next = ldg_here(Cb + off + 2 * pn); cr_next = ldg_here(Cb + off + 2 * pn + 1); }
-      }
+      fetch(p + kPairs);
       const float icl = __fdividef(1.f, cl), icr = __fdividef(1.f, cr);   // (counts are small integers)
       const float r2l = nrm.x, r2r = nrm.y, pc = nrm.z;
       const float n2cl = -2.f * cl, n2cr = -2.f * cr, n2il = -2.f * icl, n2ir = -2.f * icr;
@@ -303,34 +318,35 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
       const float2 r2l2 = make_float2(r2l, r2l), r2r2 = make_float2(r2r, r2r), pc2 = make_float2(pc, pc);
       const float2 four2 = make_float2(4.f, 4.f), n4il2 = make_float2(2.f * n2il, 2.f * n2il), n4ir2 = make_float2(2.f * n2ir, 2.f * n2ir);
       bool broken = false;
-      for (int hq = 0; hq < nh; ++hq) {
-        if (!warp_wait(&misc->tfull[hq], li & 1, abort_flag, lane)) { broken = true; break; }
+      for (int hq = 0; hq < nh; ++hq, ++it) {
+        if (!warp_wait(&misc->tfull[it & 1], (it >> 1) & 1, abort_flag, lane)) { broken = true; break; }
         tc_fence_after();
-        const uint32_t col0 = tmem + lane_addr + hq * 256;
-        const float4* qc4 = reinterpret_cast<const float4*>(misc->qconst + hq * (2 * kQH));
-        // chunks [c_begin, c_end) of every half (2 / 3 / 3 of the eight: letting the short share go round
-        // among the groups measured slower; the group that is done early moves on to the next half
-        // and the groups end up staggered, which spreads their serial phases)
-        const int c_begin = (grp * kChunks) / kGroups, c_end = ((grp + 1) * kChunks) / kGroups;
-        // chunks of 8 queries; the loads of the next chunk are in flight while this one is reduced
-        float buf[kDoubleBuffer ? 2 : 1][4][kChunk];
-        auto issue = [&](int c, int b) {
+        const uint32_t col0 = tmem + lane_addr + (it & 1) * 256;
+        const float4* qc4 = reinterpret_cast<const float4*>(misc->qconst + hq * (2 * qn));
+        // chunks [c_begin, c_end) of every step: 2 / 3 / 3 of the eight of 64 queries.  (Letting the short
+        // share go round among the groups measured 1.5 % slower: the group that is done early moves on to
+        // the next step and the groups end up staggered, which spreads their serial phases.)
+        const int c_begin = (grp * nchunk) / kGroups, c_end = ((grp + 1) * nchunk) / kGroups;
+        float buf[4][kChunk];
+        // One chunk's loads at a time: the other warps of the scheduler cover their latency.  (With the next
+        // chunk's loads in flight, 126 registers instead of 96: 2 % slower.)
+#pragma unroll 1
+        for (int c = c_begin; c < c_end; ++c) {
           const uint32_t col = col0 + c * kChunk;
-          tmem_ld8(col, buf[b][0]);
-          tmem_ld8(col + 64, buf[b][1]);
-          tmem_ld8(col + 128, buf[b][2]);
-          tmem_ld8(col + 192, buf[b][3]);
-        };
-        auto reduce = [&](int c, int b) {
+          tmem_ld8(col, buf[0]);
+          tmem_ld8(col + 64, buf[1]);
+          tmem_ld8(col + 128, buf[2]);
+          tmem_ld8(col + 192, buf[3]);
+          tmem_ld_wait();
 #pragma unroll
           for (int i = 0; i < kChunk; i += 2) {
             const float4 cq = qc4[c * (kChunk / 2) + (i >> 1)];           // the two queries' constants (a broadcast read)
             const float2 ncq = make_float2(cq.x, cq.y), hq2 = make_float2(cq.z, cq.w);
-            const float2 el = __ffma2_rn(make_float2(buf[b][0][i], buf[b][0][i + 1]), sc2, ncq);
-            const float2 er = __ffma2_rn(make_float2(buf[b][1][i], buf[b][1][i + 1]), sc2, ncq);
+            const float2 el = __ffma2_rn(make_float2(buf[0][i], buf[0][i + 1]), sc2, ncq);
+            const float2 er = __ffma2_rn(make_float2(buf[1][i], buf[1][i + 1]), sc2, ncq);
             const float2 bl = make_float2(fast_exp2(el.x), fast_exp2(el.y));
             const float2 br = make_float2(fast_exp2(er.x), fast_exp2(er.y));
-            const float2 tl = make_float2(buf[b][2][i], buf[b][2][i + 1]), tr = make_float2(buf[b][3][i], buf[b][3][i + 1]);
+            const float2 tl = make_float2(buf[2][i], buf[2][i + 1]), tr = make_float2(buf[3][i], buf[3][i + 1]);
             sAl = __fadd2_rn(sAl, bl);
             sAr = __fadd2_rn(sAr, br);
             const float2 al = __ffma2_rn(bl, n2cl2, one2), ar = __ffma2_rn(br, n2cr2, one2);   // 1 - 2 alpha
@@ -354,29 +370,9 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
               sN12 = __ffma2_rn(__fmul2_rn(bl, br), make_float2(fast_sqrt(fabsf(d12.x)), fast_sqrt(fabsf(d12.y))), sN12);
             }
           }
-        };
-        if constexpr (kDoubleBuffer) {
-          issue(c_begin, 0);
-          for (int c = c_begin; c < c_end; c += 2) {
-            tmem_ld_wait();
-            if (c + 1 < c_end) issue(c + 1, 1);
-            reduce(c, 0);
-            if (c + 1 < c_end) {
-              tmem_ld_wait();
-              if (c + 2 < c_end) issue(c + 2, 0);
-              reduce(c + 1, 1);
-            }
-          }
-        } else {
-          // (with four warps per scheduler the other warps cover the latency of the loads)
-          for (int c = c_begin; c < c_end; ++c) {
-            issue(c, 0);
-            tmem_ld_wait();
-            reduce(c, 0);
-          }
         }
         tc_fence_before();
-        warp_arrive(&misc->tfree[hq], lane);                               // this half may be overwritten
+        warp_arrive(&misc->tfree[it & 1], lane);                           // the buffer may be overwritten
       }
       if (broken) break;
       // the sums of this (query block, group) for the pair: a later kernel adds the partials in order

@@ -1,0 +1,22 @@
+"""Query blocks of every size class of the statistics kernel: up to 64 rows (one step per tile, the two accumulator
+buffers in turn) and more (two steps of half the rows to a multiple of 16, so that the second ends in padding), with
+one and with several query blocks, and three or more tiles per CTA.  Held to the tolerances of all statistics."""
+import pytest
+
+from paper_2603_00907_b200 import workloads as wl
+from tests import test_gpu_parity as parity
+
+pytestmark = pytest.mark.gpu
+
+
+# window rows per KV head: 1, 16, 24, 64 | 65, 80, 96, 126 | 130, 194, 224
+@pytest.mark.parametrize("group,window", [(1, 1), (2, 8), (3, 8), (4, 16), (5, 13), (5, 16), (4, 24), (7, 18), (5, 26),
+                                          (2, 97), (7, 32)])
+def test_statistics_of_every_block_size(group, window):
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    hkv = 16
+    w = wl.small_case(seed=100 + group * window, batch=1, n_q_heads=group * hkv, n_kv_heads=hkv, window=window,
+                      seq_lens=(8000,), budgets=(7000,))
+    data = wl.make_layer(w)
+    parity._check_round_stats(kb, w, data["K"], data["V"], data["counts"], data["q_win"], list(w.seq_lens), group & 1)
