@@ -174,44 +174,47 @@ struct WsLayout {
   size_t sync_bytes;
 };
 
-// Number of key/pair ranges each (query block, KV head, sequence) item is cut into.  The CTAs run
-// one per SM in waves of 148; a CTA costs its tiles plus about two tile times of set-up and
-// write-back.  The cut k that minimises  waves(items * k) * (ceil(tiles / k) + 2)  is taken (the
-// smaller k when two are within 1 %): 512 items of 256 tiles: k = 2 (7 half-length waves instead
-// of 4 full ones); 64 items of 1024 tiles: k = 9 (576 CTAs in 4 waves of 114 tiles instead of 128
-// CTAs of 512 tiles on 148 SMs); 8 items of 16 tiles: k = 16.  When the CTAs need more than one
-// wave, a range is not made shorter than 16 tiles: the pipeline of a CTA (three logit buffers, two
+// How the tiles of a launch's units are cut into ranges, one CTA each.  The CTAs run one per SM in waves of
+// 148; a CTA costs its tiles plus about two tile times of set-up and write-back.  The cut k of the
+// longest unit that minimises  waves(CTAs) * (ceil(tiles / k) + 2)  is taken (the smaller k when two are
+// within 1 %), with the CTAs counted from every sequence's own length: 512 items of 256 tiles: k = 2 (7
+// half-length waves instead of 4 full ones); 64 items of 1024 tiles: k = 9 (576 CTAs in 4 waves of 114
+// tiles instead of 128 CTAs of 512 tiles on 148 SMs); 8 items of 16 tiles: k = 16; 64 items of 32 to 402
+// tiles: k = 9 where counting all as the longest took 8.  When the CTAs need more than one wave, a
+// range is not made shorter than 16 tiles: the pipeline of a CTA (three logit buffers, two
 // K/V stages) takes a few tiles to fill, which the model's constant does not cover -- 512 items of
 // 20 tiles ran 2.4 % faster uncut (4 waves of 20 tiles) than cut in two (7 waves of 10), while a
 // larger constant instead slowed the long ragged items of the other workloads by up to 6 %.
+struct TileCut {
+  int splits, tiles_per_split;
+  double cost;                      // in tiles
+};
 constexpr int kNumSMs = 148;
 constexpr int kMinRangeTiles = 16;  // (see above)
 constexpr int kMaxTcSplits = 16;    // per item (more only while items * k <= 148); the attention partials are sized for it
 
-int balanced_splits(int items, int ntiles, int* tiles_per_split) {
-  if (items < 1) items = 1;
-  if (ntiles < 1) ntiles = 1;
+// `tiles`: of a unit of every sequence (0: inactive); `mult` CTAs walk each range: heads times query blocks
+TileCut balanced_cut(int mult, const int* tiles, int nseq) {
+  int ntiles = 1;
+  bool same = true;
+  for (int i = 0; i < nseq; ++i) {
+    ntiles = ntiles > tiles[i] ? ntiles : tiles[i];
+    same = same && tiles[i] == tiles[0];
+  }
+  const int items = mult * (nseq > 0 ? nseq : 1);
   int kmax = kNumSMs / items > kMaxTcSplits ? kNumSMs / items : kMaxTcSplits;
   if (kmax > ntiles) kmax = ntiles;
-  int best = 1;
-  double best_cost = 1e30;
+  TileCut best = {1, ntiles, 1e30};
   for (int k = 1; k <= kmax; ++k) {
     const int tps = (ntiles + k - 1) / k;
-    const int ctas = items * ((ntiles + tps - 1) / tps);      // ranges that are not empty
+    int ranges = 0;                                           // that are not empty
+    for (int i = 0; i < (same ? 1 : nseq); ++i) ranges += (tiles[i] + tps - 1) / tps;
+    const int ctas = mult * ranges * (same ? nseq : 1);
     if (k > 1 && tps < kMinRangeTiles && ctas > kNumSMs) continue;
     const double cost = (double)((ctas + kNumSMs - 1) / kNumSMs) * (tps + 2);
-    if (cost < best_cost * 0.99) { best_cost = cost; best = k; }
+    if (cost < best.cost * 0.99) best = {(ntiles + tps - 1) / tps, tps, cost};
   }
-  int tps = (ntiles + best - 1) / best;
-  if (tps < 1) tps = 1;
-  *tiles_per_split = tps;
-  const int s = (ntiles + tps - 1) / tps;
-  return s > 0 ? s : 1;
-}
-
-int tc_splits(int M, int Hkv, int nseq, int ntiles, int* tiles_per_split) {
-  const int nqblk = (M + 127) / 128;
-  return balanced_splits(nqblk * Hkv * nseq, ntiles, tiles_per_split);
+  return best;
 }
 
 // CTAs per cluster, and clusters per (sequence, KV head), of the decode kernel (four warps per CTA, two
@@ -315,16 +318,19 @@ struct Common {
 template <class LaunchFn>
 kvs_status_t enqueue_flash(const kvs_params_t* p, char* ws, const WsLayout& L, cudaStream_t st,
                            const CacheView& view, int Wq, int M, int causal,
-                           const RoundTable& tab, int nmax_slots, const CUtensorMap& tmK,
+                           const RoundTable& tab, const CUtensorMap& tmK,
                            const CUtensorMap& tmV, const CUtensorMap& tmQ, int32_t* status_dev,
                            bool pair_norms, LaunchFn&& launch_fn, int* n_part) {
   FlashTcArgs ta;
   ta.Hkv = p->n_kv_heads; ta.M = M; ta.nqblk = (M + 127) / 128;
   // with pair norms the tiles start at -(off & 1), so that candidate pairs never straddle a tile
-  const int ntiles = (nmax_slots + (pair_norms ? (tab.off & 1) : 0) + 127) / 128;
+  int tiles[KVS_SEQ_CHUNK];
+  for (int i = 0; i < tab.nseq; ++i)
+    tiles[i] = tab.s[i].n > 0 ? (tab.s[i].n + (pair_norms ? (tab.off & 1) : 0) + 127) / 128 : 0;
+  const TileCut cut = balanced_cut(ta.nqblk * ta.Hkv, tiles, tab.nseq);
   ta.pair_norms = pair_norms ? reinterpret_cast<float4*>(ws + L.norms) : nullptr;
   ta.pair_stride = L.pair_stride;
-  ta.splits = tc_splits(M, p->n_kv_heads, tab.nseq, ntiles, &ta.tiles_per_split);
+  ta.splits = cut.splits; ta.tiles_per_split = cut.tiles_per_split;
   ta.Wq = Wq; ta.causal = causal; ta.scale_log2 = p->softmax_scale * 1.4426950408889634f;
   ta.n_max = view.n_max; ta.counts = view.counts;
   ta.part_ml = reinterpret_cast<float2*>(ws + L.part_ml);
@@ -361,14 +367,14 @@ kvs_status_t make_call_tmaps(Common* c, const void* K, const void* V, const void
 // The statistics of one round for the sequences in `tab` (window attention partials,
 // combine, Hessian statistics), and optionally the selection.
 kvs_status_t enqueue_round_stats(const Common& c, const CacheView& view, const void* q_win,
-                                 const RoundTable& tab, int nmax_slots, bool do_select,
+                                 const RoundTable& tab, bool do_select,
                                  float* A, float* N1, float* N12, float* cosv, float* score_out,
                                  float* w_out, uint8_t* mask_out, float* o_out, float* lse_out) {
   const kvs_params_t* p = c.p;
   const float scale_log2 = p->softmax_scale * 1.4426950408889634f;
   int n_part = 0;
   {
-    kvs_status_t fs = enqueue_flash(p, c.ws, c.L, c.st, view, p->window, c.Mw, p->causal, tab, nmax_slots,
+    kvs_status_t fs = enqueue_flash(p, c.ws, c.L, c.st, view, p->window, c.Mw, p->causal, tab,
                                     c.tmK, c.tmV, c.tmQ, c.status_dev, true,
                                     [&](auto&& f) -> kvs_status_t {
                                       CUDA_TRY(launch(KVS_K_FLASH, c.st, f));
@@ -382,7 +388,7 @@ kvs_status_t enqueue_round_stats(const Common& c, const CacheView& view, const v
   ca.part_o = reinterpret_cast<float*>(c.ws + c.L.part_o);
   ca.o_hi = reinterpret_cast<__nv_bfloat16*>(c.ws + c.L.o_hi);
   ca.o_lo = reinterpret_cast<__nv_bfloat16*>(c.ws + c.L.o_lo);
-  ca.qc2 = reinterpret_cast<float2*>(c.ws + c.L.qc2);
+  ca.qc2 = reinterpret_cast<float*>(c.ws + c.L.qc2);
   ca.M_pad = (c.Mw + 127) / 128 * 128;
   ca.out_bf16 = nullptr; ca.lse_out = lse_out; ca.o_out = o_out;
   ca.e = c.weight_mode ? static_cast<const __nv_bfloat16*>(c.e_win) : nullptr;
@@ -390,10 +396,22 @@ kvs_status_t enqueue_round_stats(const Common& c, const CacheView& view, const v
 
   StatsTcArgs ta;
   ta.Hkv = p->n_kv_heads; ta.M = c.Mw; ta.nqblk = (c.Mw + 127) / 128;
-  int pmax = 0;
-  for (int i = 0; i < tab.nseq; ++i) pmax = pmax > tab.s[i].P ? pmax : tab.s[i].P;
-  const int ntiles = (pmax + 127) / 128;               // tiles of 128 candidate pairs
-  ta.splits = balanced_splits(ta.nqblk * ta.Hkv * tab.nseq, ntiles, &ta.tiles_per_split);
+  ta.tiles = 0;
+  int tiles[KVS_SEQ_CHUNK];                            // of 128 candidate pairs
+  for (int i = 0; i < tab.nseq; ++i) {
+    tiles[i] = tab.s[i].n > 0 ? (tab.s[i].P + 127) / 128 : 0;
+    ta.tiles += tiles[i] * ta.Hkv;
+  }
+  const TileCut cut = balanced_cut(ta.nqblk * ta.Hkv, tiles, tab.nseq);
+  ta.splits = cut.splits; ta.tiles_per_split = cut.tiles_per_split;
+  // Equal shares of all tiles instead of ranges, where the ranges leave the last wave or the SMs of short
+  // sequences idle.  A share costs a tile for its set-up, one for a change of unit on the way, and a little of
+  // the kernels after it, whose CTAs then find no idle SM to start on early: where the model gains less
+  // than 15 % the ranges measured the same or better (16 units of 64 tiles, two query blocks: 1048
+  // against 1052 us a pass; 8 units of 1024 tiles 8.49 against 8.6 ms), above it the shares (64 units of 16 to 201
+  // tiles: the kernel 1.39 -> 1.00 ms; 256 units of 10 tiles, two query blocks: a step 573 -> 558 us).
+  const int groups = kvs_stats_groups(ta.nqblk, ta.tiles);
+  if ((ta.tiles + groups - 1) / groups + 3 < 0.85 * cut.cost) ta.splits = 0;
   ta.n_max = view.n_max; ta.pair_stride = c.L.pair_stride;
   ta.scale_log2 = scale_log2; ta.score_mode = p->score_mode; ta.weight_mode = c.weight_mode;
   ta.counts = view.counts; ta.qc2 = ca.qc2; ta.M_pad = ca.M_pad;
@@ -664,15 +682,10 @@ kvs_status_t merge_layer_impl(const kvs_params_t* p, void* K, void* V, int32_t* 
       RoundTable tab;
       tab.nseq = 0;
       tab.off = p->sink + (r & 1);
-      int nmax_slots = 0;
-      for (; b < B && tab.nseq < KVS_SEQ_CHUNK; ++b) {
-        if ((int)plan[b].size() > i) {
-          tab.s[tab.nseq++] = plan[b][i];
-          if (plan[b][i].n > nmax_slots) nmax_slots = plan[b][i].n;
-        }
-      }
+      for (; b < B && tab.nseq < KVS_SEQ_CHUNK; ++b)
+        if ((int)plan[b].size() > i) tab.s[tab.nseq++] = plan[b][i];
       if (tab.nseq == 0) continue;
-      s = enqueue_round_stats(c, view, q_win, tab, nmax_slots, true, nullptr, nullptr, nullptr,
+      s = enqueue_round_stats(c, view, q_win, tab, true, nullptr, nullptr, nullptr,
                               nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
       if (s != KVS_OK) return s;
       CompactArgs ka;
@@ -855,7 +868,7 @@ kvs_status_t kvs_decode_attn(const kvs_params_t* p, const void* q_new, int32_t n
       if (da.splits == 1) continue;
       n_part = da.splits;
     } else {
-      s = enqueue_flash(p, c.ws, c.L, c.st, view, n_new, M, 0, tab, nmax_slots, tmK, tmV, tmQ, status_dev, false,
+      s = enqueue_flash(p, c.ws, c.L, c.st, view, n_new, M, 0, tab, tmK, tmV, tmQ, status_dev, false,
                         [&](auto&& f) -> kvs_status_t {
                           CUDA_TRY(launch(KVS_K_FLASH, c.st, f));
                           return KVS_OK;
@@ -915,12 +928,8 @@ kvs_status_t window_stats_impl(const kvs_params_t* p, const void* K, const void*
     RoundTable tab;
     tab.nseq = 0;
     tab.off = p->sink + (r & 1);
-    int nmax_slots = 0;
-    for (size_t u = k; u < act.size() && tab.nseq < KVS_SEQ_CHUNK; ++u) {
-      tab.s[tab.nseq++] = act[u];
-      if (act[u].n > nmax_slots) nmax_slots = act[u].n;
-    }
-    s = enqueue_round_stats(cc, view, q_win, tab, nmax_slots, mask != nullptr, A, N1, N12, cosv,
+    for (size_t u = k; u < act.size() && tab.nseq < KVS_SEQ_CHUNK; ++u) tab.s[tab.nseq++] = act[u];
+    s = enqueue_round_stats(cc, view, q_win, tab, mask != nullptr, A, N1, N12, cosv,
                             score, w, mask, o_win, lse_win);
     if (s != KVS_OK) return s;
   }

@@ -28,7 +28,11 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
   const int m = blockIdx.x * kCombineRows + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (m >= a.M) {            // padding rows of the per-query constants: alpha = exp2(-inf) = 0
-    if (lane == 0 && a.qc2 && m < a.M_pad) a.qc2[(size_t)unit * a.M_pad + m] = make_float2(-INFINITY, 0.f);
+    if (lane == 0 && a.qc2 && m < a.M_pad) {
+      float* qc = a.qc2 + ((size_t)unit * a.M_pad + m) * 2 - (m & 1);
+      qc[0] = -INFINITY;
+      qc[2] = 0.f;
+    }
     return;
   }
   const size_t base = (size_t)unit * a.splits * a.M + m;
@@ -94,7 +98,11 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
     qconst = eo;
   }
   if (lane == 0) {
-    if (a.qc2) a.qc2[(size_t)unit * a.M_pad + m] = make_float2(-(mstar + log2f(Z)), qconst);
+    if (a.qc2) {
+      float* qc = a.qc2 + ((size_t)unit * a.M_pad + m) * 2 - (m & 1);
+      qc[0] = -(mstar + log2f(Z));
+      qc[2] = qconst;
+    }
     if (a.lse_out) a.lse_out[row] = lse;
   }
   const float v[4] = {od.x, od.y, od.z, od.w};

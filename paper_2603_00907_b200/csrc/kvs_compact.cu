@@ -63,11 +63,6 @@ struct Shared {
 };
 constexpr int kSmemBytes = kStages * kStageBytes + (int)sizeof(Shared);
 
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
 __device__ __forceinline__ void consumer_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 // Wait of all consumer warps on two mbarrier phases; either all 256 threads go on or all leave.

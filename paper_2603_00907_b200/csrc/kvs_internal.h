@@ -72,7 +72,9 @@ struct CombineArgs {
   int32_t M, splits, Hkv;
   const float2* part_ml;
   const float* part_o;
-  float2* qc2;             // [U, M_pad]: (-(max + log2 Z), |o|^2); rows M..M_pad-1 get (-inf, 0) (may be NULL)
+  // [U, M_pad / 2, 4]: (c_2k, c_2k+1, h_2k, h_2k+1) of rows 2k, 2k + 1 with c = -(max + log2 Z), h = |o|^2;
+  // rows M..M_pad-1 get (-inf, 0) (may be NULL)
+  float* qc2;
   int32_t M_pad;           // M rounded up to a multiple of 128 (grid rows when qc2 is written)
   __nv_bfloat16* o_hi;     // [U, M, 128]: o = o_hi + o_lo to ~2^-17 relative (may be NULL)
   __nv_bfloat16* o_lo;
@@ -83,13 +85,16 @@ struct CombineArgs {
 };
 
 struct StatsTcArgs {
-  int32_t Hkv, M, nqblk, splits, tiles_per_split;
+  int32_t Hkv, M, nqblk;
+  int32_t splits, tiles_per_split;        // ranges of a unit's tiles of 128 candidate pairs; 0: equal shares of ...
+  int32_t tiles;                          // ... the tiles of all units of the launch,
+  int32_t tiles_per_group, tiles_extra;   // this many for a group of nqblk CTAs (set by the launcher)
   int32_t n_max, pair_stride;
   float scale_log2;
   int32_t score_mode;
   int32_t weight_mode;     // 0: summed norms (Eq. kstar_final); 1: exact, supplied E; 2: exact without the coupling
   const int32_t* counts;   // [U, n_max]
-  const float2* qc2;       // [U, M_pad]: (-(max + log2 Z), |o|^2), or (-(max + log2 Z), <E, o>) with a supplied E
+  const float* qc2;        // [U, M_pad / 2, 4]: as CombineArgs.qc2; <E, o> in place of |o|^2 with a supplied E
   int32_t M_pad;
   float* score;            // [U, pair_stride]
   float* w;
@@ -135,6 +140,11 @@ struct CompactArgs {
 cudaError_t kvs_launch_combine(const CombineArgs& a, const RoundTable& t, cudaStream_t st);
 // tmKp / tmVp: 5-D pair views [128, parity, slot / 2, head, sequence] of the caches; with
 // weight_mode != 0, tmOhi is the map of the supplied gradient rows E and tmOlo is not used
+// groups of `nqblk` CTAs that share out `tiles` (one CTA per SM)
+inline int kvs_stats_groups(int nqblk, int tiles) {
+  const int fit = 148 / nqblk < tiles ? 148 / nqblk : tiles;
+  return fit > 1 ? fit : 1;
+}
 cudaError_t kvs_launch_stats_tc(const StatsTcArgs& a, const RoundTable& t, const CUtensorMap& tmKp,
                                 const CUtensorMap& tmVp, const CUtensorMap& tmQ, const CUtensorMap& tmOhi,
                                 const CUtensorMap& tmOlo, cudaStream_t st);

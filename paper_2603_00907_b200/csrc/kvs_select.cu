@@ -249,6 +249,8 @@ int cluster_of(const RoundTable& t, int Hkv) {
   return c;
 }
 
+constexpr int kSpreadSmem = 118 * 1024;
+static_assert(kSpreadSmem <= kKeep * kThreads * (int)sizeof(uint32_t), "the kernel is configured for its keys");
 template <int kMode>
 cudaError_t launch_select(const StatsTcArgs& sa, const SelectArgs& a, const RoundTable& t, cudaStream_t st) {
   static KvsPerDeviceOnce configured;
@@ -268,6 +270,11 @@ cudaError_t launch_select(const StatsTcArgs& sa, const SelectArgs& a, const Roun
     const int steps = ((ntiles + c - 1) / c + kWarps - 1) / kWarps;
     cfg.dynamicSmemBytes = (size_t)(steps <= kKeep ? steps : kKeep) * kThreads * sizeof(uint32_t);   // (shorter units keep theirs)
   }
+  // The statistics kernel fills every SM when it walks equal shares: the selection's CTAs then all start on the
+  // few SMs that are done first, where they slow one another (8 units of 1200 pairs: 16 us against 10.8).
+  // Shared memory for one CTA per SM spreads them.
+  if (kMode != kMask && sa.splits == 0 && (long long)c * a.Hkv * t.nseq <= 148 && cfg.dynamicSmemBytes < (size_t)kSpreadSmem)
+    cfg.dynamicSmemBytes = kSpreadSmem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

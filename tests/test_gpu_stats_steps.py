@@ -20,3 +20,16 @@ def test_statistics_of_every_block_size(group, window):
                       seq_lens=(8000,), budgets=(7000,))
     data = wl.make_layer(w)
     parity._check_round_stats(kb, w, data["K"], data["V"], data["counts"], data["q_win"], list(w.seq_lens), group & 1)
+
+
+@pytest.mark.parametrize("group,window,hkv", [(4, 16, 8), (5, 29, 4)])
+def test_shares_that_cross_units(group, window, hkv):
+    """192 units of up to five tiles, and 96 of two query blocks each: the kernel walks equal shares of all tiles, so
+    most CTAs cross from one unit to the next, past a sequence that is done and past units of one ragged tile."""
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    lens = [1300, 1170, 400, 1290, 1301, 700, 1024, 300] * 3
+    w = wl.small_case(seed=7, batch=len(lens), n_q_heads=group * hkv, n_kv_heads=hkv, window=window, seq_lens=tuple(lens),
+                      budgets=tuple(n if i == 4 else n - n // 6 for i, n in enumerate(lens)))
+    data = wl.make_layer(w)
+    parity._check_round_stats(kb, w, data["K"], data["V"], data["counts"], data["q_win"], list(w.seq_lens), 1)
