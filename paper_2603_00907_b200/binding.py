@@ -11,6 +11,8 @@ import math
 import os
 from typing import Dict, List, Optional, Sequence, Tuple
 
+import torch
+
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libkvs.so")
 _lib = None
 
@@ -26,6 +28,20 @@ EXPORTS = ["kvs_version", "kvs_last_error_string", "kvs_launch_count", "kvs_roun
            "kvs_debug_set_wait", "kvs_adjacent_cosine",
            "kvs_workspace_size_per_head", "kvs_merge_layer_per_head", "kvs_decode_attn_per_head",
            "kvs_merge_layer_exact", "kvs_window_stats_exact", "kvs_probe_sfu", "kvs_probe_mma"]
+
+
+# Argument types (p pointer, i/u 32-bit, l 64-bit, z size): declared once, so that a call converts plain Python
+# integers in the foreign-function layer.  (With a ctypes object made for every argument and a Stream object, the
+# host took 11.2 us for a decode call whose kernel takes 7.4; now 7.7 us a call.)
+_CODES = {"p": ctypes.c_void_p, "i": ctypes.c_int32, "u": ctypes.c_uint32, "l": ctypes.c_int64, "z": ctypes.c_size_t}
+_ARGS = {"kvs_round_plan": "piiippppp", "kvs_workspace_size": "piip", "kvs_merge_layer": "pppppppippzpp",
+         "kvs_append_and_merge": "ppppppippp" "ippzpp", "kvs_compact": "ppppppppipppzpp",
+         "kvs_compact_static": "ppppppppipppp", "kvs_decode_attn": "ppipppp" "ipppzpp",
+         "kvs_window_stats": "ppppppp" "i" "pppppppppp" "zpp", "kvs_merge_layer_exact": "ppppppipp" "ippzpp",
+         "kvs_window_stats_exact": "ppppppipp" "i" "pppppppp" "zpp", "kvs_workspace_size_per_head": "piip",
+         "kvs_merge_layer_per_head": "pppppppippzpp", "kvs_decode_attn_per_head": "ppipppp" "ipppzpp",
+         "kvs_adjacent_cosine": "piii" "lll" "ppp", "kvs_debug_set_wait": "uu", "kvs_probe_sfu": "iippp",
+         "kvs_probe_mma": "iiiipp", "kvs_profile_begin": "", "kvs_profile_end": "ipp"}
 
 
 class KvsError(RuntimeError):
@@ -60,12 +76,9 @@ def lib() -> ctypes.CDLL:
         L.kvs_profile_kind_name.restype = ctypes.c_char_p
         L.kvs_profile_kind_name.argtypes = [ctypes.c_int32]
         L.kvs_static_scratch_bytes.restype = ctypes.c_size_t
-        for name in ("kvs_round_plan", "kvs_workspace_size", "kvs_merge_layer", "kvs_compact",
-                     "kvs_decode_attn", "kvs_window_stats", "kvs_profile_begin", "kvs_profile_end",
-                     "kvs_compact_static", "kvs_append_and_merge", "kvs_debug_set_wait", "kvs_adjacent_cosine",
-                     "kvs_workspace_size_per_head", "kvs_merge_layer_per_head", "kvs_decode_attn_per_head",
-                     "kvs_merge_layer_exact", "kvs_window_stats_exact", "kvs_probe_sfu", "kvs_probe_mma"):
+        for name, codes in _ARGS.items():
             getattr(L, name).restype = ctypes.c_int
+            getattr(L, name).argtypes = [_CODES[c] for c in codes]
         _lib = L
     return _lib
 
@@ -75,12 +88,16 @@ def _check(code: int) -> None:
         raise KvsError(code, lib().kvs_last_error_string().decode())
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+def _ptr(t) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
 def _i32(values: Sequence[int]):
-    return (ctypes.c_int32 * len(values))(*[int(v) for v in values])
+    array = ctypes.c_int32 * len(values)
+    try:
+        return array(*values)
+    except TypeError:                  # integers of another kind (NumPy, torch)
+        return array(*[int(v) for v in values])
 
 
 def make_params(K, V, n_q_heads: int, window: int, *, sink: int = 32, recent: Optional[int] = None,
@@ -101,9 +118,9 @@ def make_params(K, V, n_q_heads: int, window: int, *, sink: int = 32, recent: Op
     return p
 
 
-def _stream() -> ctypes.c_void_p:
-    import torch
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    # (the current stream's handle without the Stream object around it: a third of the time)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def kvs_version() -> int:
@@ -137,9 +154,9 @@ def kvs_merge_layer(params: kvs_params_t, K, V, counts, q_win, seq_len: Sequence
     B = params.batch
     new_len = (ctypes.c_int32 * B)()
     _check(lib().kvs_merge_layer(ctypes.byref(params), _ptr(K), _ptr(V), _ptr(counts), _ptr(q_win),
-                                 _i32(seq_len), _i32(budget), ctypes.c_int32(counts.shape[-1]),
+                                 _i32(seq_len), _i32(budget), counts.shape[-1],
                                  new_len, _ptr(workspace),
-                                 ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                 workspace.numel() * workspace.element_size(),
                                  _ptr(status_dev), _stream()))
     return list(new_len)
 
@@ -152,10 +169,10 @@ def kvs_append_and_merge(params: kvs_params_t, K, V, counts, chunk_k, chunk_v, q
     B = params.batch
     new_len = (ctypes.c_int32 * B)()
     _check(lib().kvs_append_and_merge(ctypes.byref(params), _ptr(K), _ptr(V), _ptr(counts), _ptr(chunk_k),
-                                      _ptr(chunk_v), ctypes.c_int32(chunk_k.shape[2]), _ptr(q_win),
-                                      _i32(cur_len), _i32(budget), ctypes.c_int32(counts.shape[-1]),
+                                      _ptr(chunk_v), chunk_k.shape[2], _ptr(q_win),
+                                      _i32(cur_len), _i32(budget), counts.shape[-1],
                                       new_len, _ptr(workspace),
-                                      ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                      workspace.numel() * workspace.element_size(),
                                       _ptr(status_dev), _stream()))
     return list(new_len)
 
@@ -166,9 +183,9 @@ def kvs_compact(params: kvs_params_t, K, V, counts, merge_mask, w_left, seq_len:
     new_len = (ctypes.c_int32 * B)()
     _check(lib().kvs_compact(ctypes.byref(params), _ptr(K), _ptr(V), _ptr(counts), _ptr(merge_mask),
                              _ptr(w_left), _i32(seq_len), _i32(n_merge),
-                             ctypes.c_int32(counts.shape[-1]), new_len, _ptr(new_index),
+                             counts.shape[-1], new_len, _ptr(new_index),
                              _ptr(workspace),
-                             ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                             workspace.numel() * workspace.element_size(),
                              _ptr(status_dev), _stream()))
     return list(new_len)
 
@@ -181,7 +198,7 @@ def kvs_compact_static(params: kvs_params_t, K, V, counts, merge_mask, w_left, s
     new_len = (ctypes.c_int32 * B)()
     _check(lib().kvs_compact_static(ctypes.byref(params), _ptr(K), _ptr(V), _ptr(counts),
                                     _ptr(merge_mask), _ptr(w_left), _i32(seq_len), _i32(n_merge),
-                                    ctypes.c_int32(counts.shape[-1]), new_len, _ptr(new_index),
+                                    counts.shape[-1], new_len, _ptr(new_index),
                                     _ptr(status_dev), _stream()))
     return list(new_len)
 
@@ -193,11 +210,11 @@ def kvs_static_scratch_bytes() -> int:
 def kvs_decode_attn(params: kvs_params_t, q_new, K, V, counts, seq_len: Sequence[int], out,
                     workspace, lse=None, status_dev=None) -> None:
     n_new = q_new.shape[2]
-    _check(lib().kvs_decode_attn(ctypes.byref(params), _ptr(q_new), ctypes.c_int32(n_new), _ptr(K),
+    _check(lib().kvs_decode_attn(ctypes.byref(params), _ptr(q_new), n_new, _ptr(K),
                                  _ptr(V), _ptr(counts), _i32(seq_len),
-                                 ctypes.c_int32(counts.shape[-1]), _ptr(out), _ptr(lse),
+                                 counts.shape[-1], _ptr(out), _ptr(lse),
                                  _ptr(workspace),
-                                 ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                 workspace.numel() * workspace.element_size(),
                                  _ptr(status_dev), _stream()))
 
 
@@ -206,10 +223,10 @@ def kvs_window_stats(params: kvs_params_t, K, V, counts, q_win, seq_len: Sequenc
                      score=None, w=None, mask=None, o_win=None, lse_win=None,
                      status_dev=None) -> None:
     _check(lib().kvs_window_stats(ctypes.byref(params), _ptr(K), _ptr(V), _ptr(counts), _ptr(q_win),
-                                  _i32(seq_len), _i32(budget), ctypes.c_int32(counts.shape[-1]),
+                                  _i32(seq_len), _i32(budget), counts.shape[-1],
                                   _ptr(A), _ptr(N1), _ptr(N12), _ptr(cosv), _ptr(score), _ptr(w),
                                   _ptr(mask), _ptr(o_win), _ptr(lse_win), _ptr(workspace),
-                                  ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                  workspace.numel() * workspace.element_size(),
                                   _ptr(status_dev), _stream()))
 
 
@@ -220,9 +237,9 @@ def kvs_merge_layer_exact(params: kvs_params_t, K, V, counts, q_win, e_win, weig
     B = params.batch
     new_len = (ctypes.c_int32 * B)()
     _check(lib().kvs_merge_layer_exact(ctypes.byref(params), _ptr(K), _ptr(V), _ptr(counts), _ptr(q_win),
-                                       _ptr(e_win), ctypes.c_int32(weight_mode), _i32(seq_len), _i32(budget),
-                                       ctypes.c_int32(counts.shape[-1]), new_len, _ptr(workspace),
-                                       ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                       _ptr(e_win), weight_mode, _i32(seq_len), _i32(budget),
+                                       counts.shape[-1], new_len, _ptr(workspace),
+                                       workspace.numel() * workspace.element_size(),
                                        _ptr(status_dev), _stream()))
     return list(new_len)
 
@@ -231,10 +248,10 @@ def kvs_window_stats_exact(params: kvs_params_t, K, V, counts, q_win, e_win, wei
                            seq_len: Sequence[int], budget: Sequence[int], workspace, *, A=None, g_self=None,
                            g_pair=None, cosv=None, score=None, w=None, mask=None, status_dev=None) -> None:
     _check(lib().kvs_window_stats_exact(ctypes.byref(params), _ptr(K), _ptr(V), _ptr(counts), _ptr(q_win),
-                                        _ptr(e_win), ctypes.c_int32(weight_mode), _i32(seq_len), _i32(budget),
-                                        ctypes.c_int32(counts.shape[-1]), _ptr(A), _ptr(g_self), _ptr(g_pair),
+                                        _ptr(e_win), weight_mode, _i32(seq_len), _i32(budget),
+                                        counts.shape[-1], _ptr(A), _ptr(g_self), _ptr(g_pair),
                                         _ptr(cosv), _ptr(score), _ptr(w), _ptr(mask), _ptr(workspace),
-                                        ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                        workspace.numel() * workspace.element_size(),
                                         _ptr(status_dev), _stream()))
 
 
@@ -251,9 +268,9 @@ def kvs_merge_layer_per_head(params: kvs_params_t, K, V, counts, q_win, seq_len:
     U = params.batch * params.n_kv_heads
     new_len = (ctypes.c_int32 * U)()
     _check(lib().kvs_merge_layer_per_head(ctypes.byref(params), _ptr(K), _ptr(V), _ptr(counts), _ptr(q_win),
-                                          _i32(seq_len), _i32(budget), ctypes.c_int32(counts.shape[-1]),
+                                          _i32(seq_len), _i32(budget), counts.shape[-1],
                                           new_len, _ptr(workspace),
-                                          ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                          workspace.numel() * workspace.element_size(),
                                           _ptr(status_dev), _stream()))
     return list(new_len)
 
@@ -261,40 +278,40 @@ def kvs_merge_layer_per_head(params: kvs_params_t, K, V, counts, q_win, seq_len:
 def kvs_decode_attn_per_head(params: kvs_params_t, q_new, K, V, counts, seq_len: Sequence[int], out,
                              workspace, lse=None, status_dev=None) -> None:
     n_new = q_new.shape[2]
-    _check(lib().kvs_decode_attn_per_head(ctypes.byref(params), _ptr(q_new), ctypes.c_int32(n_new), _ptr(K),
+    _check(lib().kvs_decode_attn_per_head(ctypes.byref(params), _ptr(q_new), n_new, _ptr(K),
                                           _ptr(V), _ptr(counts), _i32(seq_len),
-                                          ctypes.c_int32(counts.shape[-1]), _ptr(out), _ptr(lse),
+                                          counts.shape[-1], _ptr(out), _ptr(lse),
                                           _ptr(workspace),
-                                          ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                          workspace.numel() * workspace.element_size(),
                                           _ptr(status_dev), _stream()))
 
 
 def kvs_adjacent_cosine(x, seq_len: Sequence[int], cos_out) -> None:
     """cos_out[b,h,t] = cosine of rows t and t+1 of the bf16 tensor x [B,H,Nmax,128], t < seq_len[b]-1."""
     B, H, Nmax, _ = x.shape
-    _check(lib().kvs_adjacent_cosine(_ptr(x), ctypes.c_int32(B), ctypes.c_int32(H), ctypes.c_int32(Nmax),
-                                     ctypes.c_int64(x.stride(0)), ctypes.c_int64(x.stride(1)),
-                                     ctypes.c_int64(x.stride(2)), _i32(seq_len), _ptr(cos_out), _stream()))
+    _check(lib().kvs_adjacent_cosine(_ptr(x), B, H, Nmax,
+                                     x.stride(0), x.stride(1),
+                                     x.stride(2), _i32(seq_len), _ptr(cos_out), _stream()))
 
 
 def kvs_debug_set_wait(limit_us: int = 0, withhold: int = 0) -> None:
     """Time limit of the device-side waits (0: the default of one second) and the test hook that
     makes one kind of wait run out (see kvs.h)."""
-    _check(lib().kvs_debug_set_wait(ctypes.c_uint32(limit_us), ctypes.c_uint32(withhold)))
+    _check(lib().kvs_debug_set_wait(limit_us, withhold))
 
 
 def kvs_probe_sfu(blocks: int, iters: int, sink) -> int:
     """Launch the special-function probe on the current stream; returns the operations it executes."""
     ops = ctypes.c_uint64(0)
-    _check(lib().kvs_probe_sfu(ctypes.c_int32(blocks), ctypes.c_int32(iters), _ptr(sink), ctypes.byref(ops), _stream()))
+    _check(lib().kvs_probe_sfu(blocks, iters, _ptr(sink), ctypes.byref(ops), _stream()))
     return int(ops.value)
 
 
 def kvs_probe_mma(blocks: int, n_cols: int, reuse_a: bool, products: int, cycles) -> None:
     """Launch the operand-feed probe on the current stream; `cycles` is a device int64[blocks] that
     receives each CTA's elapsed cycles for its `products` tensor-core products (-1: wait ran out)."""
-    _check(lib().kvs_probe_mma(ctypes.c_int32(blocks), ctypes.c_int32(n_cols), ctypes.c_int32(1 if reuse_a else 0),
-                               ctypes.c_int32(products), _ptr(cycles), _stream()))
+    _check(lib().kvs_probe_mma(blocks, n_cols, 1 if reuse_a else 0,
+                               products, _ptr(cycles), _stream()))
 
 
 def kvs_profile_begin() -> None:
