@@ -367,7 +367,7 @@ kvs_status_t make_call_tmaps(Common* c, const void* K, const void* V, const void
 // The statistics of one round for the sequences in `tab` (window attention partials,
 // combine, Hessian statistics), and optionally the selection.
 kvs_status_t enqueue_round_stats(const Common& c, const CacheView& view, const void* q_win,
-                                 const RoundTable& tab, bool do_select,
+                                 const RoundTable& tab, bool do_select, bool zero_sync,
                                  float* A, float* N1, float* N12, float* cosv, float* score_out,
                                  float* w_out, uint8_t* mask_out, float* o_out, float* lse_out) {
   const kvs_params_t* p = c.p;
@@ -433,6 +433,8 @@ kvs_status_t enqueue_round_stats(const Common& c, const CacheView& view, const v
   se.mask = mask_out ? mask_out : reinterpret_cast<uint8_t*>(c.ws + c.L.mask);
   se.tile_prefix = reinterpret_cast<int32_t*>(c.ws + c.L.tile_prefix);
   se.select = do_select ? 1 : 0;
+  se.zero = reinterpret_cast<uint4*>(c.ws + c.L.sync);
+  se.zero_bytes = zero_sync ? (uint32_t)c.L.sync_bytes : 0;
   int kernels = 1;
   CUDA_TRY(launch(KVS_K_SELECT, c.st, [&] { return kvs_launch_finalize_select(ta, se, tab, c.st, &kernels); }));
   g_launches.fetch_add((uint64_t)kernels - 1, std::memory_order_relaxed);
@@ -542,6 +544,7 @@ kvs_status_t kvs_detail_compact_scratch(const kvs_params_t* p, void* K, void* V,
     se.mask = const_cast<uint8_t*>(merge_mask);
     se.tile_prefix = tile_prefix;
     se.select = 1;
+    se.zero = nullptr; se.zero_bytes = 0;
     CUDA_TRY(launch(KVS_K_MISC, st, [&] { return kvs_launch_mask_prefix(se, tab, st); }));
     CompactArgs ka;
     ka.c = view;
@@ -670,7 +673,7 @@ kvs_status_t merge_layer_impl(const kvs_params_t* p, void* K, void* V, int32_t* 
     }
   }
   if (rounds == 0) return KVS_OK;
-  CUDA_TRY(cudaMemsetAsync(c.ws + c.L.sync, 0, c.L.sync_bytes, c.st));
+  bool first = true;                                     // the first selection zeroes the tickets and flags
   uint32_t* tickets = reinterpret_cast<uint32_t*>(c.ws + c.L.sync);
   uint32_t* flags = tickets + (size_t)KVS_MAX_ROUNDS * c.L.U;
 
@@ -685,9 +688,10 @@ kvs_status_t merge_layer_impl(const kvs_params_t* p, void* K, void* V, int32_t* 
       for (; b < B && tab.nseq < KVS_SEQ_CHUNK; ++b)
         if ((int)plan[b].size() > i) tab.s[tab.nseq++] = plan[b][i];
       if (tab.nseq == 0) continue;
-      s = enqueue_round_stats(c, view, q_win, tab, true, nullptr, nullptr, nullptr,
+      s = enqueue_round_stats(c, view, q_win, tab, true, first, nullptr, nullptr, nullptr,
                               nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
       if (s != KVS_OK) return s;
+      first = false;
       CompactArgs ka;
       ka.c = view;
       ka.pair_stride = c.L.pair_stride; ka.tile_stride = c.L.tile_stride;
@@ -776,7 +780,7 @@ kvs_status_t kvs_compact(const kvs_params_t* p, void* K, void* V, int32_t* count
         if (P < 0) P = 0;
         act.push_back({seq_len[b], P, 0, b});
       }
-  CUDA_TRY(cudaMemsetAsync(c.ws + c.L.sync, 0, c.L.sync_bytes, c.st));
+  bool first = true;
   uint32_t* tickets = reinterpret_cast<uint32_t*>(c.ws + c.L.sync);
   uint32_t* flags = tickets + (size_t)KVS_MAX_ROUNDS * c.L.U;
   const CacheView view = make_view(p, K, V, counts, n_max);
@@ -795,6 +799,9 @@ kvs_status_t kvs_compact(const kvs_params_t* p, void* K, void* V, int32_t* count
     se.mask = const_cast<uint8_t*>(merge_mask);
     se.tile_prefix = reinterpret_cast<int32_t*>(c.ws + c.L.tile_prefix);
     se.select = 1;
+    se.zero = reinterpret_cast<uint4*>(c.ws + c.L.sync);
+    se.zero_bytes = first ? (uint32_t)c.L.sync_bytes : 0;
+    first = false;
     CUDA_TRY(launch(KVS_K_MISC, c.st, [&] { return kvs_launch_mask_prefix(se, tab, c.st); }));
     CompactArgs ka;
     ka.c = view;
@@ -920,7 +927,6 @@ kvs_status_t window_stats_impl(const kvs_params_t* p, const void* K, const void*
   if (act.empty()) return KVS_OK;
   s = make_call_tmaps(&c, K, V, q_win, n_max);
   if (s != KVS_OK) return s;
-  CUDA_TRY(cudaMemsetAsync(c.ws + c.L.sync, 0, c.L.sync_bytes, c.st));
   Common cc = c;
   cc.L.pair_stride = n_max / 2;
   const CacheView view = make_view(p, const_cast<void*>(K), const_cast<void*>(V), const_cast<int32_t*>(counts), n_max);
@@ -929,7 +935,7 @@ kvs_status_t window_stats_impl(const kvs_params_t* p, const void* K, const void*
     tab.nseq = 0;
     tab.off = p->sink + (r & 1);
     for (size_t u = k; u < act.size() && tab.nseq < KVS_SEQ_CHUNK; ++u) tab.s[tab.nseq++] = act[u];
-    s = enqueue_round_stats(cc, view, q_win, tab, mask != nullptr, A, N1, N12, cosv,
+    s = enqueue_round_stats(cc, view, q_win, tab, mask != nullptr, false, A, N1, N12, cosv,
                             score, w, mask, o_win, lse_win);
     if (s != KVS_OK) return s;
   }

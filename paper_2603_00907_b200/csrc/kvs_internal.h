@@ -118,6 +118,11 @@ struct SelectArgs {
   uint8_t* mask;           // [U, pair_stride]
   int32_t* tile_prefix;    // [U, tile_stride]: merged pairs before each compaction tile
   int32_t select;          // 0: scores and weights only
+  // the compaction's tickets and flags, zeroed before the first compaction of a call (zero_bytes 0: not here).
+  // A memset in front of the first kernel cost 2 to 4 us a call (nothing starts early
+  // behind it): a streaming step of one layer 62.3 -> 58.0 us, 128 K slots compacted 368 -> 365 us.
+  uint4* zero;
+  uint32_t zero_bytes;     // a multiple of 16
 };
 
 struct CompactArgs {

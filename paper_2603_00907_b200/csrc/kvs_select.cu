@@ -127,6 +127,10 @@ select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
   if (!kFromMask)
     for (int i = tid; i < 3 * kBins; i += kThreads) (&s_hist[0][0])[i] = 0;
   kvs_pdl_wait();
+  {
+    const uint32_t cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, all = gridDim.x * gridDim.y * gridDim.z;
+    for (uint32_t i = cta * kThreads + tid; i < a.zero_bytes / 16; i += all * kThreads) a.zero[i] = make_uint4(0, 0, 0, 0);
+  }
   const SeqRound sr = tab.s[blockIdx.z];
   const int n = sr.n;
   if (n <= 0) return;                                      // (the whole cluster)
