@@ -35,6 +35,10 @@ constexpr int kStageBytes = 4 * kSub;      // channels 0-63 and 64-127 of K, the
 constexpr int kWarpBytes = kStages * kStageBytes;
 constexpr int kSmemBytes = kWarps * kWarpBytes;
 constexpr float kRescaleGap = 8.f;         // log2 units
+// The stabiliser before any logit.  Finite, so that a block whose logits are all -inf gives weights of 0 (-inf - (-inf)
+// would be NaN), and the lowest value, so that every finite logit moves it.  What has it still at the end is
+// merged like the rest: nothing or zeros are added, and a NaN stays.
+constexpr float kNoMax = -3.402823466e38f;
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                           uint32_t b1) {
@@ -144,7 +148,7 @@ decode_rows_kernel(const DecodeArgs a, const RoundTable tab, const __grid_consta
 #pragma unroll
       for (int i = 0; i < 4; ++i) o[nt][jb][i] = 0.f;
     l[nt][0] = l[nt][1] = 0.f;
-    m_run[nt][0] = m_run[nt][1] = -INFINITY;
+    m_run[nt][0] = m_run[nt][1] = kNoMax;
   }
 
   int stage = 0;
@@ -198,7 +202,7 @@ decode_rows_kernel(const DecodeArgs a, const RoundTable tab, const __grid_consta
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           const float m_new = fmaxf(mn[u], m_run[nt][u]);
-          const float f = m_run[nt][u] > -INFINITY ? fast_exp2(m_run[nt][u] - m_new) : 0.f;
+          const float f = fast_exp2(m_run[nt][u] - m_new);
           l[nt][u] *= f;
 #pragma unroll
           for (int jb = 0; jb < 8; ++jb) { o[nt][jb][u] *= f; o[nt][jb][2 + u] *= f; }
@@ -279,8 +283,7 @@ decode_rows_kernel(const DecodeArgs a, const RoundTable tab, const __grid_consta
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) mx = fmaxf(mx, s_m[w][threadIdx.x]);
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w)
-      if (s_m[w][threadIdx.x] > -INFINITY) sum = fmaf(s_l[w][threadIdx.x], fast_exp2(s_m[w][threadIdx.x] - mx), sum);
+    for (int w = 0; w < kWarps; ++w) sum = fmaf(s_l[w][threadIdx.x], fast_exp2(s_m[w][threadIdx.x] - mx), sum);
     s_cm[threadIdx.x] = mx; s_cl[threadIdx.x] = sum;
   }
   __syncthreads();
@@ -296,7 +299,7 @@ decode_rows_kernel(const DecodeArgs a, const RoundTable tab, const __grid_consta
     for (int u = 0; u < 2; ++u) {
       if (kFour && t >= 2) continue;
       const int row = nt * 8 + 2 * t + u;
-      const float f = m_run[nt][u] > -INFINITY ? fast_exp2(m_run[nt][u] - s_cm[row]) : 0.f;
+      const float f = fast_exp2(m_run[nt][u] - s_cm[row]);
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
@@ -326,9 +329,7 @@ decode_rows_kernel(const DecodeArgs a, const RoundTable tab, const __grid_consta
     float sum = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int r = 0; r < ctas; ++r) {
-      const float mr = *cluster.map_shared_rank(&s_cm[row], r);
-      if (mr == -INFINITY) continue;
-      const float f = fast_exp2(mr - mx);
+      const float f = fast_exp2(*cluster.map_shared_rank(&s_cm[row], r) - mx);
       const float4 v = *cluster.map_shared_rank(reinterpret_cast<float4*>(smem) + i, r);
       sum = fmaf(*cluster.map_shared_rank(&s_cl[row], r), f, sum);
       acc.x = fmaf(v.x, f, acc.x); acc.y = fmaf(v.y, f, acc.y);

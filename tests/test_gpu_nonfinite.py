@@ -1,0 +1,66 @@
+"""Infinite and undefined logits.  A key with an infinite channel gives its slot a logit of -inf, i.e. no weight, wherever
+in a sequence such slots stand; a key with a NaN makes the rows that see it NaN; neither may be lost or spread when
+the parts of a row (blocks, warps, CTAs, key ranges) are merged.  Against the oracle in float64.
+
+Finite outputs are held to what P' in 16 significant bits gives, 2^-17 max |V| < 1e-4 before the bf16 rounding."""
+import numpy as np
+import pytest
+
+from oracle import kvs_oracle as oc
+from paper_2603_00907_b200 import workloads as wl
+from tests import kvs_testlib as tl
+
+pytestmark = pytest.mark.gpu
+
+NEG_INF, NAN = 0xFF80, 0x7FC0
+
+
+def _attend(hq, hkv, t, n, low=(), nan=()):
+    """Decode attention of `t` tokens over n slots whose logits are -inf in the ranges `low` and NaN in `nan`;
+    checked against the oracle for every KV head."""
+    import torch
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    w = wl.small_case(seed=n + t, n_q_heads=hq, n_kv_heads=hkv, window=8, seq_lens=(n,), budgets=(n,), n_decode=t)
+    data = wl.make_layer(w)
+    data["q_new"][..., 0] = 0x3F80                        # 1.0: an infinite key channel 0 decides the logit
+    for lo, hi in low:
+        data["K"][0, :, lo:hi, 0] = NEG_INF
+    for lo, hi in nan:
+        data["K"][0, :, lo:hi, 5] = NAN
+    dev = tl.upload_layer(data)
+    p = kb.make_params(dev["K"], dev["V"], hq, 8)
+    ws = torch.empty(kb.kvs_workspace_size(p, n, t), dtype=torch.uint8, device="cuda")
+    out = torch.zeros((1, hq, t, 128), dtype=torch.bfloat16, device="cuda")
+    lse = torch.zeros((1, hq, t), dtype=torch.float32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    kb.kvs_decode_attn(p, dev["q_new"], dev["K"], dev["V"], dev["counts"], [n], out, ws, lse=lse, status_dev=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    if nan:
+        assert torch.isnan(out).all() and torch.isnan(lse).all()
+        return
+    og, lg, G = tl.bits_of(out), lse.cpu().numpy(), hq // hkv
+    for h in range(hkv):
+        hs = slice(h * G, (h + 1) * G)
+        ref, lse_ref = oc.decode_attention(data["q_new"][0, hs], data["K"][0, h, :n], data["V"][0, h, :n],
+                                           data["counts"][0, h, :n])
+        ok, mx, _, _ = tl.bf16_close(og[0, hs], oc.f64_to_bf16(ref), atol=1e-4)
+        assert ok, (h, mx)
+        assert np.max(np.abs(lg[0, hs] - lse_ref)) < 1e-4
+
+
+# 4, 8 and 16 rows; one CTA, one cluster, several clusters per unit
+FEW_ROWS = [(4, 1, 1, 200), (4, 1, 1, 6000), (8, 1, 1, 640), (2, 1, 7, 6200), (8, 2, 4, 1500)]
+
+
+@pytest.mark.parametrize("hq,hkv,t,n", FEW_ROWS)
+@pytest.mark.parametrize("low", [((0, 16),), ((0, 130),), ((16, 48), (64, 96)), ((3, None),)])
+def test_few_rows_with_slots_of_no_weight(hq, hkv, t, n, low):
+    _attend(hq, hkv, t, n, low=[(lo, n if hi is None else hi) for lo, hi in low])
+
+
+@pytest.mark.parametrize("hq,hkv,t,n", FEW_ROWS)
+@pytest.mark.parametrize("nan", [(0, 16), (16, 32), (128, 200), (7, 8), (0, None)])
+def test_few_rows_that_see_a_nan(hq, hkv, t, n, nan):
+    _attend(hq, hkv, t, n, nan=[(nan[0], n if nan[1] is None else nan[1])])
