@@ -60,7 +60,9 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
       const int cnt = min(32, a.splits - s0);
       float2 own = first;
       if (s0 > 0) own = lane < cnt ? ml[(size_t)(s0 + lane) * a.M] : make_float2(-INFINITY, 0.f);
-      const float f = own.x == -INFINITY ? 0.f : fast_exp2(own.x - mstar);   // 0: an empty range, whose output is not read
+      const float f = own.x == -INFINITY ? 0.f : fast_exp2(own.x - mstar);
+      // an empty range's output is not there to be read; one of weight 0 is (0 times infinity stays NaN)
+      const uint32_t filled = __ballot_sync(0xffffffffu, own.x != -INFINITY);
       Z = fmaf(own.y, f, Z);
       for (int i0 = 0; i0 < cnt; i0 += kBatch) {
         float4 po[kBatch];
@@ -69,7 +71,7 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
         for (int i = 0; i < kBatch; ++i) {
           fi[i] = __shfl_sync(0xffffffffu, f, i0 + i);
           po[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (fi[i] != 0.f) po[i] = *reinterpret_cast<const float4*>(a.part_o + (base + (size_t)(s0 + i0 + i) * a.M) * KVS_D + 4 * lane);
+          if ((filled >> (i0 + i)) & 1u) po[i] = *reinterpret_cast<const float4*>(a.part_o + (base + (size_t)(s0 + i0 + i) * a.M) * KVS_D + 4 * lane);
         }
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {

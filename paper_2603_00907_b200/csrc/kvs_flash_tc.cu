@@ -587,7 +587,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
       tc_fence_after();
       if (part == 0 && m < a.M) {
         const float sum = (misc->part[0][row] + misc->part[1][row]) + (misc->part[2][row] + misc->part[3][row]);
-        a.part_ml[pidx] = make_float2(sum > 0.f ? m_stab : -INFINITY, sum);
+        a.part_ml[pidx] = make_float2(sum == 0.f ? -INFINITY : m_stab, sum);   // (a NaN sum is not an empty range)
       }
       float ov[32];
       tmem_ld32(tmem + lane_addr + kColO + part * 32, ov);

@@ -15,9 +15,9 @@ pytestmark = pytest.mark.gpu
 NEG_INF, NAN = 0xFF80, 0x7FC0
 
 
-def _attend(hq, hkv, t, n, low=(), nan=()):
+def _attend(hq, hkv, t, n, low=(), nan=(), edit=None, every=1):
     """Decode attention of `t` tokens over n slots whose logits are -inf in the ranges `low` and NaN in `nan`;
-    checked against the oracle for every KV head."""
+    checked against the oracle for every KV head (or every `every`-th)."""
     import torch
     from paper_2603_00907_b200 import binding as kb, build
     build.build()
@@ -28,6 +28,8 @@ def _attend(hq, hkv, t, n, low=(), nan=()):
         data["K"][0, :, lo:hi, 0] = NEG_INF
     for lo, hi in nan:
         data["K"][0, :, lo:hi, 5] = NAN
+    if edit:
+        edit(data)
     dev = tl.upload_layer(data)
     p = kb.make_params(dev["K"], dev["V"], hq, 8)
     ws = torch.empty(kb.kvs_workspace_size(p, n, t), dtype=torch.uint8, device="cuda")
@@ -41,13 +43,14 @@ def _attend(hq, hkv, t, n, low=(), nan=()):
         assert torch.isnan(out).all() and torch.isnan(lse).all()
         return
     og, lg, G = tl.bits_of(out), lse.cpu().numpy(), hq // hkv
-    for h in range(hkv):
+    for h in range(0, hkv, every):
         hs = slice(h * G, (h + 1) * G)
         ref, lse_ref = oc.decode_attention(data["q_new"][0, hs], data["K"][0, h, :n], data["V"][0, h, :n],
                                            data["counts"][0, h, :n])
         ok, mx, _, _ = tl.bf16_close(og[0, hs], oc.f64_to_bf16(ref), atol=1e-4)
         assert ok, (h, mx)
         assert np.max(np.abs(lg[0, hs] - lse_ref)) < 1e-4
+    return out
 
 
 # 4, 8 and 16 rows; one CTA, one cluster, several clusters per unit
@@ -64,3 +67,50 @@ def test_few_rows_with_slots_of_no_weight(hq, hkv, t, n, low):
 @pytest.mark.parametrize("nan", [(0, 16), (16, 32), (128, 200), (7, 8), (0, None)])
 def test_few_rows_that_see_a_nan(hq, hkv, t, n, nan):
     _attend(hq, hkv, t, n, nan=[(nan[0], n if nan[1] is None else nan[1])])
+
+
+# more than 16 rows: ranges of one, three, six and 24 tiles of 128 slots; a combine of few rows and of many
+MANY_ROWS = [(2, 2, 20, 700), (64, 64, 24, 700), (90, 90, 40, 700), (80, 80, 40, 3000)]
+
+
+@pytest.mark.parametrize("hq,hkv,t,n", MANY_ROWS)
+@pytest.mark.parametrize("nan", [(300, 301), (0, 128), (640, 700), (0, None)])
+def test_many_rows_that_see_a_nan(hq, hkv, t, n, nan):
+    _attend(hq, hkv, t, n, nan=[(nan[0], n if nan[1] is None else nan[1])])
+
+
+@pytest.mark.parametrize("hq,hkv,t", [(2, 2, 20), (64, 64, 40)])
+def test_an_infinite_value_of_weight_zero(hq, hkv, t):
+    """0 times infinity is NaN, whether the weight was lost inside a key range or between two."""
+    import torch
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    n = 640
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    q, K, V = (torch.randn(1, h, m, 128, generator=g, device="cuda").to(torch.bfloat16) for h, m in ((hq, t), (hkv, n), (hkv, n)))
+    q[..., 0], K[..., 0], K[:, :, 0, 0] = 8.0, 0.0, 400.0   # slot 0 has a logit of 283, the others of about 0
+    V[:, :, -1] = float("inf")
+    counts = torch.ones(1, hkv, n, dtype=torch.int32, device="cuda")
+    p = kb.make_params(K, V, hq, 8)
+    ws = torch.empty(kb.kvs_workspace_size(p, n, t), dtype=torch.uint8, device="cuda")
+    out = torch.zeros_like(q)
+    kb.kvs_decode_attn(p, q, K, V, counts, [n], out, ws)
+    assert torch.isnan(out).all()
+
+
+@pytest.mark.parametrize("hkv,first_round", [(2, 0), (90, 1)])
+def test_window_rows_that_see_a_nan(hkv, first_round):
+    import torch
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    n, W = 700, 24
+    w = wl.small_case(seed=hkv, n_q_heads=hkv, n_kv_heads=hkv, window=W, seq_lens=(n,), budgets=(500,))
+    data = wl.make_layer(w)
+    data["K"][0, :, 300, 5] = NAN
+    dev = tl.upload_layer(data)
+    p = kb.make_params(dev["K"], dev["V"], hkv, W, first_round=first_round)
+    ws = torch.empty(kb.kvs_workspace_size(p, n, 0), dtype=torch.uint8, device="cuda")
+    o, lse = torch.zeros(1, hkv, W, 128, device="cuda"), torch.zeros(1, hkv, W, device="cuda")
+    kb.kvs_window_stats(p, dev["K"], dev["V"], dev["counts"], dev["q_win"], [n], [500], ws, o_win=o, lse_win=lse)
+    assert torch.isnan(o).all() and torch.isnan(lse).all()
