@@ -21,8 +21,8 @@
 // The stabiliser m of a row is the row's maximum over the CTA's FIRST tile and stays: fp32 sums and
 // bf16 terms are floating point, so a later logit that is larger costs no precision until it is
 // larger by tens of powers of two.  So no tile but the first needs a maximum, and no warp waits for
-// another one.  If a part of l exceeds 2^60 all the same, the CTA walks its range twice more, once for
-// the true maxima and once with them.  (With a running maximum, exchanged between the two warps of a row and
+// another one.  If a part of l exceeds 2^60 all the same, or the first tile has nothing but logits of -inf
+// for a row, the CTA walks its range twice more, once for the true maxima and once with them.  (With a running maximum, exchanged between the two warps of a row and
 // between the teams on every tile: 1024 query rows over 131072 slots, 8 heads, 0.83 ms; so: 0.65 ms, 2 000 cycles a
 // tile of which the tensor core needs 1 536.)
 //
@@ -441,13 +441,14 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
       for (int i = 0; i < 16; ++i) mx[i & 1] = fmaxf(mx[i & 1], x[i]);
       return fmaxf(mx[0], mx[1]);
     };
-    // the row's maximum from its four parts (all softmax threads together); a row without a visible slot has none
-    auto set_stab = [&](float mine) {
+    // the row's maximum from its four parts (all softmax threads together); false if it has no finite logit
+    auto set_stab = [&](float mine) -> bool {
       misc->part[part][row] = mine;
       softmax_barrier();
       const float mx = fmaxf(fmaxf(misc->part[0][row], misc->part[1][row]), fmaxf(misc->part[2][row], misc->part[3][row]));
       m_stab = mx > -INFINITY ? mx * a.scale_log2 : 0.f;
       softmax_barrier();                                   // (the parts are written again later)
+      return mx > -INFINITY;
     };
     // P' = exp2(scaled logit - m) of 16 slots as hi + lo bf16, two slots per 32-bit column, over the 8 (hi) and
     // 8 (lo) columns in place of the logits.  The hi term is the value cut to bf16 (a byte permute, no
@@ -492,7 +493,9 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
         mx = fmaxf(max16(xa), max16(xb));
         tc_fence_before();
       }
-      set_stab(mx);
+      // A row that sees slots in the first tile, but no logit above -inf, has nothing to go by: its later logits may be
+      // of any size, so the range is walked again.  (One that sees none there sees none in this range.)
+      if (!set_stab(mx) && alive && max(0, t_begin * kTile - shift) <= last_vis) misc->again = 1;
     }
     int gi_last = 0;
     for (int walk = 0, n_walks = 1; walk < n_walks; ++walk) {
