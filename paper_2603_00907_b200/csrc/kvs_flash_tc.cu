@@ -48,6 +48,10 @@ constexpr int kSoftmaxWarps = 16, kNormWarps = 8;
 constexpr int kPvWarp = 2 + kSoftmaxWarps + kNormWarps;          // the warp that issues the P V products
 constexpr int kThreads = (kPvWarp + 1) * 32;   // warp 0: TMA, 1: S products, 2-17: softmax, 18-25: pair norms, 26: P V products
 constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: a part of l beyond this asks for another walk
+// From here on a logit (log2 units) is scaled and rounded before the stabiliser, which was rounded the same way, is
+// subtracted.  One fused multiply-add leaves the product unrounded: two equal logits of 2^24 then differ from
+// the stabiliser by up to half a unit, of 1e30 by far more than an exponent holds.
+constexpr float kFarLogit = 1048576.f;     // 2^20
 constexpr int kSBufs = 3;                  // logit / P' buffers in tensor memory
 
 struct Misc {
@@ -428,6 +432,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     float* cnt = misc->cnt[warp - 2];
     bool alive = true;
     float m_stab = 0.f, l = 0.f;             // the stabiliser (log2 units) and this thread's part of l
+    bool far = false;                        // a row of the warp has one beyond kFarLogit
     // masks the logits of 16 slots from j0 on
     auto mask16 = [&](int j0, float* x) {
       if (j0 >= 0 && j0 + 15 <= last_free) return;
@@ -447,6 +452,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
       softmax_barrier();
       const float mx = fmaxf(fmaxf(misc->part[0][row], misc->part[1][row]), fmaxf(misc->part[2][row], misc->part[3][row]));
       m_stab = mx > -INFINITY ? mx * a.scale_log2 : 0.f;
+      far = __any_sync(0xffffffffu, fabsf(m_stab) > kFarLogit) != 0;
       softmax_barrier();                                   // (the parts are written again later)
       return mx > -INFINITY;
     };
@@ -456,7 +462,12 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     // Two slots per instruction: the softmax warps are short of issue slots.
     float2 ls[2];
     auto emit16 = [&](uint32_t col, float* x, const float* cnt16) {
-      const float2 sc2 = make_float2(a.scale_log2, a.scale_log2), nm2 = make_float2(-m_stab, -m_stab);
+      if (far) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] *= a.scale_log2;
+      }
+      const float sc = far ? 1.f : a.scale_log2;
+      const float2 sc2 = make_float2(sc, sc), nm2 = make_float2(-m_stab, -m_stab);
       uint32_t hi[8], lo[8];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {

@@ -95,6 +95,16 @@ def test_many_rows_with_slots_of_no_weight(hq, hkv, t, n, low, far):
     _attend(hq, hkv, t, n, low=low, edit=_rest_far_below(low[-1][1]) if far else None, every=39)
 
 
+@pytest.mark.parametrize("hq,hkv,t,n", [FEW_ROWS[1], FEW_ROWS[4]] + MANY_ROWS[:3])
+@pytest.mark.parametrize("value", [3e9, -3e9, -1e20, 1e30, -3.38e38])
+def test_equal_logits_of_any_size(hq, hkv, t, n, value):
+    """Every slot has the same logit, up to bf16's lowest value times the scale: equal weights."""
+    def edit(data):
+        data["K"][:] = 0
+        data["K"][..., 0] = wl.f32_to_bf16_bits(np.float32([value]))[0]
+    _attend(hq, hkv, t, n, edit=edit, every=39)
+
+
 @pytest.mark.parametrize("hq,hkv,t", [(2, 2, 20), (64, 64, 40)])
 def test_an_infinite_value_of_weight_zero(hq, hkv, t):
     """0 times infinity is NaN, whether the weight was lost inside a key range or between two."""
