@@ -1,6 +1,7 @@
 """Query blocks of every size class of the statistics kernel: up to 64 rows (one step per tile, the two accumulator
 buffers in turn) and more (two steps of half the rows to a multiple of 16, so that the second ends in padding), with
 one and with several query blocks, and three or more tiles per CTA.  Held to the tolerances of all statistics."""
+import numpy as np
 import pytest
 
 from paper_2603_00907_b200 import workloads as wl
@@ -33,3 +34,41 @@ def test_shares_that_cross_units(group, window, hkv):
                       budgets=tuple(n if i == 4 else n - n // 6 for i, n in enumerate(lens)))
     data = wl.make_layer(w)
     parity._check_round_stats(kb, w, data["K"], data["V"], data["counts"], data["q_win"], list(w.seq_lens), 1)
+
+
+@pytest.mark.parametrize("seed", [1, 2])
+def test_values_around_a_mean(seed):
+    """|vbar - o|^2 is a small difference of terms of about |mean|^2 = 128 here, and <vbar, o> comes from sixteen
+    additions into an accumulator that is cut to 24 bits each time.  With the hi and lo terms of o in turn the partial
+    sums grow evenly and the cuts add up to 8 * 2^-24 of the result, with all lo terms last to 12 * 2^-24: the error
+    of N1 and N12 measured 0.96e-5 and 2.1e-5 of their norm in the first order, 1.4e-5 and 2.9e-5 in the second,
+    in that proportion.  The bounds lie between."""
+    import torch
+    from oracle import kvs_oracle as oc
+    from paper_2603_00907_b200 import binding as kb, build
+    from tests import kvs_testlib as tl
+    build.build()
+    hq, hkv, n, W = 32, 8, 1024, 32
+    w = wl.small_case(seed=60 + seed, n_q_heads=hq, n_kv_heads=hkv, window=W, seq_lens=(n,), budgets=(340,))
+    data = wl.make_layer(w)
+    rng = np.random.default_rng(seed)
+    c = 1 + rng.exponential(12.0, size=(1, hkv, n)).astype(np.int32)
+    mean = rng.standard_normal((1, hkv, 1, 128))
+    values = rng.standard_normal((1, hkv, n, 128)) * np.sqrt(c)[..., None] + mean * c[..., None]
+    data["counts"][:], data["V"] = c, wl.f32_to_bf16_bits(values.astype(np.float32))
+    dev = tl.upload_layer(data)
+    p = kb.make_params(dev["K"], dev["V"], hq, W)
+    ws = torch.empty(kb.kvs_workspace_size(p, n, 0), dtype=torch.uint8, device="cuda")
+    N1, N12 = torch.zeros(1, hkv, n, device="cuda"), torch.zeros(1, hkv, n // 2, device="cuda")
+    kb.kvs_window_stats(p, dev["K"], dev["V"], dev["counts"], dev["q_win"], [n], [340], ws, N1=N1, N12=N12)
+    err, ref = np.zeros(2), np.zeros(2)
+    for h in range(hkv):
+        st = oc.round_stats(data["K"][0, h], data["V"][0, h], c[0, h], data["q_win"][0, 4 * h:4 * h + 4], 340, 0,
+                            **parity._oracle_kwargs(w))
+        off, P = st["off"], st["P"]
+        for i, (got, want) in enumerate(((N1[0, h, off:off + 2 * P], st["N1"][off:off + 2 * P]),
+                                         (N12[0, h, :P], st["N12"][:P]))):
+            err[i] += np.sum((got.cpu().numpy() - want) ** 2)
+            ref[i] += np.sum(want ** 2)
+    rel = np.sqrt(err / ref)
+    assert rel[0] < 1.15e-5 and rel[1] < 2.4e-5, rel
