@@ -142,11 +142,11 @@ __device__ __forceinline__ void pair_dots(const uint8_t* tile, int row0, int ste
     if (((lane >> 1) & 3) == it) { ll = o[0]; rr = o[1]; lr = o[2]; }
   }
 }
-// 1 / sqrt(x): the hardware's estimate and a Newton step (the compiler's square root and division took 300 cycles a tile)
+// 1 / sqrt(x) of a sum of squares: the hardware's estimate and a Newton step (the compiler's square root and division took
+// 300 cycles a tile).  0 gives a large finite number, and the step is left out where it is not defined (infinity).
 __device__ __forceinline__ float rsqrt_newton(float x) {
-  x = fmaxf(x, 1e-36f);
-  const float y = rsqrtf(x);
-  return fmaf(y * 0.5f, fmaf(-x * y, y, 1.f), y);
+  const float y = fminf(rsqrtf(x), 1e38f);
+  return fmaf(y * 0.5f, fmaxf(fmaf(-x * y, y, 1.f), -1.f), y);
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -403,7 +403,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
           const float r2l = ll * icl * icl, r2r = rr * icr * icr;
           norms[4 * (size_t)p] = r2l; norms[4 * (size_t)p + 1] = r2r; norms[4 * (size_t)p + 2] = r2l + r2r + 2.f * lr * icl * icr;
         } else {
-          norms[4 * (size_t)p + 3] = lr * rsqrt_newton(ll) * rsqrt_newton(rr);
+          norms[4 * (size_t)p + 3] = lr * fminf(rsqrt_newton(ll) * rsqrt_newton(rr), 1e30f);
         }
       }
       __syncwarp();

@@ -72,3 +72,17 @@ def test_values_around_a_mean(seed):
             ref[i] += np.sum(want ** 2)
     rel = np.sqrt(err / ref)
     assert rel[0] < 1.15e-5 and rel[1] < 2.4e-5, rel
+
+
+@pytest.mark.parametrize("scale", [3e-18, 2e-20, 0.0])
+def test_cosine_of_short_keys(scale):
+    """Every second key is `scale` times as long: the cosine with its neighbour does not depend on it until the product
+    of the lengths is below 1e-30, where it is 0 (in float64 as in float32)."""
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    w = wl.small_case(seed=77, window=8, seq_lens=(700,), budgets=(500,))
+    data = wl.make_layer(w)
+    keys = (data["K"].astype(np.uint32) << 16).view(np.float32)
+    keys[:, :, ::2] *= np.float32(scale)
+    data["K"] = wl.f32_to_bf16_bits(keys)
+    parity._check_round_stats(kb, w, data["K"], data["V"], data["counts"], data["q_win"], [700], 0)
