@@ -39,6 +39,9 @@ constexpr float kRescaleGap = 8.f;         // log2 units
 // would be NaN), and the lowest value, so that every finite logit moves it.  What has it still at the end is
 // merged like the rest: nothing or zeros are added, and a NaN stays.
 constexpr float kNoMax = -3.402823466e38f;
+// The stabiliser is put a little above the maximum.  At the maximum P' would be exactly 1, its lo term 0, and 0 times an
+// infinite value NaN: one row in sixteen that sees an infinite value had its block's maximum there.
+constexpr float kAbove = 0.01f;
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                           uint32_t b1) {
@@ -201,7 +204,7 @@ decode_rows_kernel(const DecodeArgs a, const RoundTable tab, const __grid_consta
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const float m_new = fmaxf(mn[u], m_run[nt][u]);
+          const float m_new = fmaxf(mn[u] + kAbove, m_run[nt][u]);
           const float f = fast_exp2(m_run[nt][u] - m_new);
           l[nt][u] *= f;
 #pragma unroll

@@ -80,6 +80,25 @@ def test_many_rows_that_see_a_nan(hq, hkv, t, n, nan):
     _attend(hq, hkv, t, n, nan=[(nan[0], n if nan[1] is None else nan[1])])
 
 
+@pytest.mark.parametrize("hq,hkv,t,n", FEW_ROWS)
+@pytest.mark.parametrize("slot", [0, 5, 130])
+def test_few_rows_whose_largest_weight_has_an_infinite_value(hq, hkv, t, n, slot):
+    import torch
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    q, K, V = (torch.randn(1, h, m, 128, generator=g, device="cuda").to(torch.bfloat16) for h, m in ((hq, t), (hkv, n), (hkv, n)))
+    q[..., 0], K[..., 0], K[:, :, slot, 0] = 8.0, 0.0, 20.0   # a logit of 14 against 0 +- 1
+    V[:, :, slot] = float("inf")
+    counts = torch.ones(1, hkv, n, dtype=torch.int32, device="cuda")
+    p = kb.make_params(K, V, hq, 8)
+    ws = torch.empty(kb.kvs_workspace_size(p, n, t), dtype=torch.uint8, device="cuda")
+    out = torch.zeros_like(q)
+    kb.kvs_decode_attn(p, q, K, V, counts, [n], out, ws)
+    assert (out == float("inf")).all()
+
+
 def _rest_far_below(lo):
     """Keys from slot lo on with logits of about -265 (e to that power is no float)."""
     def edit(data):
@@ -93,6 +112,15 @@ def _rest_far_below(lo):
 def test_many_rows_with_slots_of_no_weight(hq, hkv, t, n, low, far):
     """The first tiles of a range may have no weight at all, and the first logits after them any size."""
     _attend(hq, hkv, t, n, low=low, edit=_rest_far_below(low[-1][1]) if far else None, every=39)
+
+
+@pytest.mark.parametrize("hq,hkv,t,n", [FEW_ROWS[1], FEW_ROWS[4]] + MANY_ROWS)
+@pytest.mark.parametrize("lo,hi", [(0, 128), (140, 400)])
+def test_slots_of_the_lowest_value(hq, hkv, t, n, lo, hi):
+    """Logits of about -3e37, as far below the others as a float goes: no weight."""
+    def edit(data):
+        data["K"][0, :, lo:hi, 0] = 0xFF7F
+    _attend(hq, hkv, t, n, edit=edit, every=39)
 
 
 @pytest.mark.parametrize("hq,hkv,t,n", [FEW_ROWS[1], FEW_ROWS[4]] + MANY_ROWS[:3])
