@@ -58,3 +58,27 @@ def test_decode_of_few_rows(hq, hkv, t, lens, token_major):
             ok, mx, _, _ = tl.bf16_close(og[b, hs], oc.f64_to_bf16(ref), atol=1e-4)
             assert ok, (b, h, mx)
             assert np.max(np.abs(lg[b, hs] - lse_ref)) < 1e-4
+
+
+@pytest.mark.parametrize("hq,hkv,t,n", [(4, 1, 1, 40000), (16, 2, 2, 20011), (8, 2, 4, 9000)])
+def test_stages_are_refilled_behind_their_use(hq, hkv, t, n):
+    """Every warp fills its ring dozens of times: thirty passes over changing neighbours in the stream give the same bits,
+    and those of the oracle's rounding for one head."""
+    import torch
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    w = wl.small_case(seed=n, n_q_heads=hq, n_kv_heads=hkv, window=8, seq_lens=(n,), budgets=(n,), n_decode=t)
+    data = wl.make_layer(w)
+    dev = tl.upload_layer(data)
+    p = kb.make_params(dev["K"], dev["V"], hq, 8)
+    ws = torch.empty(kb.kvs_workspace_size(p, n, t), dtype=torch.uint8, device="cuda")
+    outs = []
+    for _ in range(30):
+        out = torch.zeros((1, hq, t, 128), dtype=torch.bfloat16, device="cuda")
+        kb.kvs_decode_attn(p, dev["q_new"], dev["K"], dev["V"], dev["counts"], [n], out, ws)
+        outs.append(out)
+    assert all(torch.equal(o, outs[0]) for o in outs)
+    G = hq // hkv
+    ref, _ = oc.decode_attention(data["q_new"][0, :G], data["K"][0, 0], data["V"][0, 0], data["counts"][0, 0])
+    ok, mx, _, _ = tl.bf16_close(tl.bits_of(outs[0])[0, :G], oc.f64_to_bf16(ref), atol=1e-4)
+    assert ok, mx
