@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
   constexpr bool kFromMask = kMode == kMask;
   extern __shared__ uint32_t s_key[];
-  __shared__ uint32_t s_hist[3][kBins];
+  __shared__ alignas(8) uint32_t s_hist[3][kBins];       // (read as pairs of bins)
   __shared__ uint32_t s_warp[2][kWarps], s_digit, s_k, s_total[2], s_cnt[2][kWarps];
   kvs_pdl_launch_dependents();
   cg::cluster_group cluster = cg::this_cluster();

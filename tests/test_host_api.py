@@ -149,3 +149,19 @@ def test_variant_entry_points_reject_bad_arguments_before_any_cuda_call(lib):
     assert pm(1, 64, 0, 12, x, None) == 1           # not a multiple of 8
     assert pm(0, 64, 0, 64, x, None) == 1
     assert pm(1, 64, 0, 64, None, None) == 1
+
+
+def test_shared_arrays_read_as_wider_words_declare_that_alignment():
+    """A __shared__ array has the alignment of its element type, whatever the compiler places in front of it."""
+    csrc = os.path.join(ROOT, "paper_2603_00907_b200", "csrc")
+    size = {"uint2": 8, "float2": 8, "uint4": 16, "float4": 16}
+    seen = 0
+    for name in sorted(os.listdir(csrc)):
+        if not name.endswith((".cu", ".cuh")):
+            continue
+        text = open(os.path.join(csrc, name)).read()
+        for kind, var in re.findall(r"reinterpret_cast<(?:const )?(uint2|uint4|float2|float4)\*>\(&?(s_\w+)", text):
+            declared = re.search(r"__shared__ alignas\((\d+)\)[^;]*\b%s\[" % var, text)
+            assert declared and int(declared.group(1)) >= size[kind], (name, var, kind)
+            seen += 1
+    assert seen
