@@ -85,9 +85,14 @@ decode_rows_kernel(const DecodeArgs a, const RoundTable tab, const __grid_consta
   __shared__ float s_m[kWarps][kRows], s_l[kWarps][kRows];
   __shared__ float s_cm[kRows], s_cl[kRows];             // of the CTA: maximum and sum
   kvs_pdl_launch_dependents();
+  if (sm100::smem_u32(smem) & 1023u) {                    // the swizzled tiles need a 1024-byte aligned base (the same in every CTA)
+    kvs_pdl_wait();
+    if (threadIdx.x == 0 && a.status_dev) atomicExch(a.status_dev, (int)KVS_ERR_CUDA);
+    return;
+  }
   if (threadIdx.x == 0) {
     for (int i = 0; i < kWarps * kStages; ++i) sm100::mbar_init(&s_full[0][i], 1);
-    s_ctl[0] = (sm100::smem_u32(smem) & 1023u) ? 1 : 0;   // (the swizzled tiles need a 1024-byte aligned base)
+    s_ctl[0] = 0;
     s_ctl[1] = (int)a.wait_us;
     sm100::mbar_fence_init();
   }
@@ -128,7 +133,6 @@ decode_rows_kernel(const DecodeArgs a, const RoundTable tab, const __grid_consta
     }
     copy_commit();                                       // (empty groups at the end keep the count right)
   };
-  if (ctl[0]) b = b_end;                                 // (a misplaced ring: report it and leave)
   if (lane == 0) { sm100::prefetch_tmap(&tmK); sm100::prefetch_tmap(&tmV); }
   for (int s = 0; s < kStages; ++s) request(b + s * b_step, s);
   // query rows as B fragments: lane 4 g + t holds row g of each tile
