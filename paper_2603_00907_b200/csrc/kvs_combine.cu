@@ -61,7 +61,8 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
       float2 own = first;
       if (s0 > 0) own = lane < cnt ? ml[(size_t)(s0 + lane) * a.M] : make_float2(-INFINITY, 0.f);
       const float f = own.x == -INFINITY ? 0.f : fast_exp2(own.x - mstar);
-      // an empty range's output is not there to be read; one of weight 0 is (0 times infinity stays NaN)
+      // An empty range has left no output: what stands there is read and dropped (a condition on a load is waited for
+      // before it).  One of weight 0 counts: 0 times infinity stays NaN.
       const uint32_t filled = __ballot_sync(0xffffffffu, own.x != -INFINITY);
       Z = fmaf(own.y, f, Z);
       for (int i0 = 0; i0 < cnt; i0 += kBatch) {
@@ -70,11 +71,11 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
           fi[i] = __shfl_sync(0xffffffffu, f, i0 + i);
-          po[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if ((filled >> (i0 + i)) & 1u) po[i] = *reinterpret_cast<const float4*>(a.part_o + (base + (size_t)(s0 + i0 + i) * a.M) * KVS_D + 4 * lane);
+          po[i] = *reinterpret_cast<const float4*>(a.part_o + (base + (size_t)min(s0 + i0 + i, a.splits - 1) * a.M) * KVS_D + 4 * lane);
         }
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
+          if (!((filled >> (i0 + i)) & 1u)) po[i] = make_float4(0.f, 0.f, 0.f, 0.f);
           acc.x = fmaf(po[i].x, fi[i], acc.x); acc.y = fmaf(po[i].y, fi[i], acc.y);
           acc.z = fmaf(po[i].z, fi[i], acc.z); acc.w = fmaf(po[i].w, fi[i], acc.w);
         }
@@ -129,11 +130,20 @@ combine_partials(const CombineArgs a, const RoundTable tab) {
 
 }  // namespace
 
+// Shared memory that the kernel does not use, so that two CTAs of the batched form fit an SM and not three.  They are
+// launched while the attention still runs, onto the SMs that it leaves idle, and three to an SM slow one another
+// (16 units of 80 rows: a call of the statistics 28.1 us, with two 24.6; a streaming step 65.5 and 59.7).
+constexpr int kTwoPerSM = 90 * 1024;
+
 cudaError_t kvs_launch_combine(const CombineArgs& a, const RoundTable& t, cudaStream_t st) {
+  static KvsPerDeviceOnce configured;
+  cudaError_t e = configured.run([] {
+    return cudaFuncSetAttribute(combine_partials<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTwoPerSM);
+  });
+  if (e != cudaSuccess) return e;
   const int rows = a.qc2 ? a.M_pad : a.M;
   dim3 grid((rows + kCombineRows - 1) / kCombineRows, a.Hkv, t.nseq);
-  // (two CTAs per SM: one wave at the registers of a batch)
-  if ((long long)grid.x * grid.y * grid.z <= 2 * 148)
-    return kvs_launch_chained(combine_partials<8>, grid, dim3(kCombineRows * 32), 0, st, a, t);
+  if ((long long)grid.x * grid.y * grid.z <= 2 * 148)      // one wave
+    return kvs_launch_chained(combine_partials<8>, grid, dim3(kCombineRows * 32), kTwoPerSM, st, a, t);
   return kvs_launch_chained(combine_partials<1>, grid, dim3(kCombineRows * 32), 0, st, a, t);
 }
