@@ -217,18 +217,56 @@ TileCut balanced_cut(int mult, const int* tiles, int nseq) {
   return best;
 }
 
+// What a decode call walks: (sequence, KV head) units, and the 16-slot blocks of the longest and of all of them.
+struct DecodeWork {
+  int units, longest;
+  long long blocks;
+};
+DecodeWork decode_work(const int32_t* seq_len, int nseq, int Hkv) {
+  DecodeWork w = {0, 0, 0};
+  for (int b = 0; b < nseq; ++b) {
+    if (seq_len[b] <= 0) continue;
+    const int n = (seq_len[b] + KVS_DECODE_BLOCK - 1) / KVS_DECODE_BLOCK;
+    w.units += Hkv;
+    w.blocks += (long long)n * Hkv;
+    w.longest = w.longest > n ? w.longest : n;
+  }
+  return w;
+}
+
+// Whether a call of M rows per KV head takes the kernel for few rows (kvs_decode.cu), else the tensor-core tiles.  Nine to
+// sixteen rows cost that kernel 0.9 us a block of a warp (up to eight 0.66), and its partials and their combine 6 us:
+// up to 24 units with more than eleven blocks a warp in one cluster of eight on average, but not so long that
+// several clusters a unit pay, are faster in tiles.  8 heads, 16 rows, tiles against this kernel: 3000 slots 12.0 and
+// 11.7 us, 6000: 13.9 and 17.3, 12000: 17.5 and 22.3, 16384: 20.1 both, 32768: 36.6 and 31.1; 16 heads of
+// 8192: 19.0 and 27.2, of 16384: 35.0 and 38, of 32768: 58 and 53; 24 of 8192: 24.5 and 26.0; 32 of 8192: 34 and 28.
+bool decode_in_few_rows(int M, const DecodeWork& w) {
+  if (M > KVS_DECODE_ROWS) return false;
+  return !(M > 8 && w.units <= 24 && w.blocks > 352LL * w.units && w.longest < 1024 && w.blocks <= 16384);
+}
+
 // CTAs per cluster, and clusters per (sequence, KV head), of the decode kernel (four warps per CTA, two
-// CTAs per SM).  The cluster grows to eight CTAs while the grid stays within 512: one sequence of 2048
-// slots, 8 heads: 7.3 us with eight, 9.8 with four, 25 with one; 256 units of 512-8192 slots: 91 us with
-// two, 109 with eight (the waits for a cluster's slowest CTA; sixteen took 9 us for 300 slots against 4.8).
-// A unit gets more clusters, and a combine kernel, only where SMs are idle and a warp keeps six blocks
-// (about 2 us of the combine against 0.66 us a block): 8 units of 16384 slots 27.4 -> 18.7 us with four.
-int decode_cluster(int units, int nmax_slots, int max_splits, int* splits) {
-  const int nblocks = (nmax_slots + KVS_DECODE_BLOCK - 1) / KVS_DECODE_BLOCK;
+// CTAs per SM).  The cluster grows to eight CTAs while the grid stays in one wave of 296: one sequence of 2048
+// slots, 8 heads: 7.3 us with eight, 9.8 with four, 25 with one; 64 units of 2048 slots 12.2 us with four, 18.6 with eight.
+// Beyond one wave, up to 512 CTAs,
+//   * for ragged batches, whose longest unit would be the last: 64 units of 4096-32768 slots 122 us with eight, 136 with
+//     four; 256 of 512-8192 91 us with two, 109 with eight (for the waits for a cluster's slowest CTA), and
+//   * for long units whose grid gets near 512 (1.7 waves): 256 units of 8192 slots 159 us with two, 175 with one; of 3000
+//     slots 73 and 70; 128 of 12000 122 us with four, 130 with two; but 96 of 8192 75 and 70 (384 CTAs).
+// (Sixteen took 9 us for 300 slots against 4.8.)  A unit gets more clusters, and a combine kernel, only where SMs are idle and a
+// warp keeps six blocks (about 2 us of the combine against 0.66 us a block): 8 units of 16384 slots 27.4 -> 18.7 us with four.
+int decode_cluster(const DecodeWork& w, int max_splits, int* splits) {
+  const bool ragged = 5LL * w.longest * w.units > 6 * w.blocks;   // the longest 1.2 times the average
   int c = 1;
-  while (c < 8 && units * c * 2 <= 512 && c * 4 < nblocks) c *= 2;
+  while (c < 8 && c * 4 < w.longest) {
+    const int grid = 2 * c * w.units;
+    const bool one_wave = grid <= 2 * kNumSMs;
+    const bool full = c < 4 && grid > 3 * kNumSMs && w.longest >= 2 * c * 4 * 40;
+    if (!one_wave && (grid > 512 || !(ragged || full))) break;
+    c *= 2;
+  }
   int s = 1;
-  while (units * c * s * 2 <= 2 * kNumSMs && nblocks >= c * 4 * s * 2 * 6 && 2 * s <= max_splits) s *= 2;
+  while (w.units * c * s * 2 <= 2 * kNumSMs && w.longest >= c * 4 * s * 2 * 6 && 2 * s <= max_splits) s *= 2;
   *splits = s;
   return c;
 }
@@ -834,7 +872,7 @@ kvs_status_t kvs_decode_attn(const kvs_params_t* p, const void* q_new, int32_t n
   const int B = p->batch;
   const int M = c.G * n_new;
   const CacheView view = make_view(p, const_cast<void*>(K), const_cast<void*>(V), const_cast<int32_t*>(counts), n_max);
-  const bool few_rows = M <= KVS_DECODE_ROWS;
+  const bool few_rows = decode_in_few_rows(M, decode_work(seq_len, B, p->n_kv_heads));
   CUtensorMap tmK, tmV, tmQ;
   {
     const uint64_t kd[4] = {KVS_D, (uint64_t)n_max, (uint64_t)p->n_kv_heads, (uint64_t)p->batch};
@@ -850,11 +888,9 @@ kvs_status_t kvs_decode_attn(const kvs_params_t* p, const void* q_new, int32_t n
   for (int b0 = 0; b0 < B; b0 += KVS_SEQ_CHUNK) {
     RoundTable tab;
     tab.nseq = 0; tab.off = 0;
-    int nmax_slots = 0;
     for (int b = b0; b < B && b < b0 + KVS_SEQ_CHUNK; ++b) {
       if (seq_len[b] <= 0) continue;
       tab.s[tab.nseq++] = {seq_len[b], 0, 0, b};
-      if (seq_len[b] > nmax_slots) nmax_slots = seq_len[b];
     }
     if (tab.nseq == 0) continue;
     int n_part = 0;
@@ -870,7 +906,8 @@ kvs_status_t kvs_decode_attn(const kvs_params_t* p, const void* q_new, int32_t n
       da.out = static_cast<__nv_bfloat16*>(out); da.lse = lse;
       da.part_ml = reinterpret_cast<float2*>(c.ws + c.L.part_ml);
       da.part_o = reinterpret_cast<float*>(c.ws + c.L.part_o);
-      const int ctas = decode_cluster(p->n_kv_heads * tab.nseq, nmax_slots, splits_bound(M, p->n_kv_heads), &da.splits);
+      const int ctas = decode_cluster(decode_work(seq_len + b0, std::min(KVS_SEQ_CHUNK, B - b0), p->n_kv_heads),
+                                      splits_bound(M, p->n_kv_heads), &da.splits);
       CUDA_TRY(launch(KVS_K_FLASH, c.st, [&] { return kvs_launch_decode_rows(da, tab, tmK, tmV, ctas, c.st); }));
       if (da.splits == 1) continue;
       n_part = da.splits;

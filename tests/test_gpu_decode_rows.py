@@ -19,7 +19,12 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("hq,hkv,t,lens,token_major", [
     (1, 1, 1, (1,), False), (4, 1, 1, (15, 16, 17), False), (5, 1, 1, (63, 64, 65, 129), True),
     (4, 2, 4, (511, 513, 200), False), (3, 1, 3, (2049, 0, 33), True), (8, 1, 1, (1025,), False),
-    (4, 1, 1, (3500,), False), (2, 1, 7, (6200, 40), True), (16, 8, 1, tuple(range(17, 17 + 70)), False)])
+    (4, 1, 1, (3500,), False), (2, 1, 7, (6200, 40), True), (16, 8, 1, tuple(range(17, 17 + 70)), False),
+    # nine and sixteen rows on both sides of the lengths that go to the tensor-core tiles
+    (9, 1, 1, (5632,), False), (9, 1, 1, (5633,), True), (4, 1, 4, (5700, 5650), False), (16, 1, 1, (16369,), False),
+    # units for clusters of four, two and one CTA in one wave of the GPU, and a ragged batch beyond it
+    (24, 24, 1, (700, 640), True), (72, 24, 3, (333, 300, 301, 320, 310), False), (48, 48, 2, (90, 129, 128, 127), False),
+    (40, 40, 1, (5200, 40, 33, 70), False)])
 def test_decode_of_few_rows(hq, hkv, t, lens, token_major):
     import torch
     from paper_2603_00907_b200 import binding as kb, build

@@ -54,7 +54,7 @@ def _attend(hq, hkv, t, n, low=(), nan=(), edit=None, every=1):
 
 
 # 4, 8 and 16 rows; one CTA, one cluster, several clusters per unit
-FEW_ROWS = [(4, 1, 1, 200), (4, 1, 1, 6000), (8, 1, 1, 640), (2, 1, 7, 6200), (8, 2, 4, 1500)]
+FEW_ROWS = [(4, 1, 1, 200), (4, 1, 1, 6000), (8, 1, 1, 640), (1, 1, 7, 6200), (8, 2, 4, 1500)]
 
 
 @pytest.mark.parametrize("hq,hkv,t,n", FEW_ROWS)
