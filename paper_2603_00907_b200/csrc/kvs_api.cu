@@ -246,8 +246,10 @@ bool decode_in_few_rows(int M, const DecodeWork& w) {
 }
 
 // CTAs per cluster, and clusters per (sequence, KV head), of the decode kernel (four warps per CTA, two
-// CTAs per SM).  The cluster grows to eight CTAs while the grid stays in one wave of 296: one sequence of 2048
-// slots, 8 heads: 7.3 us with eight, 9.8 with four, 25 with one; 64 units of 2048 slots 12.2 us with four, 18.6 with eight.
+// CTAs per SM): as many as there are blocks for and as run in one wave, up to eight.  (With the last
+// cluster that fits, 56 of five CTAs, some still start late: 20.5 us for 3000 slots, 15.6 with four.)  One sequence of 2048
+// slots, 8 heads: 7.3 us with eight, 9.8 with four, 25 with one; 64 units of 2048 slots 12.2 us with four, 18.6 with eight;
+// 80 of 3000 24.4 us with three, 28.4 with two, 32.7 with four.
 // Beyond one wave, up to 512 CTAs,
 //   * for ragged batches, whose longest unit would be the last: 64 units of 4096-32768 slots 122 us with eight, 136 with
 //     four; 256 of 512-8192 91 us with two, 109 with eight (for the waits for a cluster's slowest CTA), and
@@ -257,13 +259,14 @@ bool decode_in_few_rows(int M, const DecodeWork& w) {
 // warp keeps six blocks (about 2 us of the combine against 0.66 us a block): 8 units of 16384 slots 27.4 -> 18.7 us with four.
 int decode_cluster(const DecodeWork& w, int max_splits, int* splits) {
   const bool ragged = 5LL * w.longest * w.units > 6 * w.blocks;   // the longest 1.2 times the average
+  const int* fit = w.units > 32 ? kvs_decode_resident_clusters() : nullptr;   // (up to 32 clusters of eight always fit)
   int c = 1;
-  while (c < 8 && c * 4 < w.longest) {
-    const int grid = 2 * c * w.units;
-    const bool one_wave = grid <= 2 * kNumSMs;
-    const bool full = c < 4 && grid > 3 * kNumSMs && w.longest >= 2 * c * 4 * 40;
-    if (!one_wave && (grid > 512 || !(ragged || full))) break;
-    c *= 2;
+  for (int k = 2; k <= KVS_DECODE_CLUSTER && (k - 1) * 4 < w.longest; ++k)
+    if (!fit || w.units + (k > 2) <= fit[k]) c = k;
+  for (int k = 2 * c < KVS_DECODE_CLUSTER ? 2 * c : KVS_DECODE_CLUSTER; c < k && c * 4 < w.longest && k * w.units <= 512;
+       k = 2 * c < KVS_DECODE_CLUSTER ? 2 * c : KVS_DECODE_CLUSTER) {
+    if (!ragged && !(c < 4 && k * w.units > 3 * kNumSMs && w.longest >= k * 4 * 40)) break;
+    c = k;
   }
   int s = 1;
   while (w.units * c * s * 2 <= 2 * kNumSMs && w.longest >= c * 4 * s * 2 * 6 && 2 * s <= max_splits) s *= 2;

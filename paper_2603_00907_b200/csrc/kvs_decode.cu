@@ -20,6 +20,8 @@
 // 16 rows 135 -> 90 us.  Loads straight into registers reached 4.9-5.5 TB/s, lane-private cp.async 4.9.
 #include <cooperative_groups.h>
 
+#include <mutex>
+
 #include "kvs_internal.h"
 #include "kvs_sm100.cuh"
 
@@ -363,12 +365,17 @@ decode_rows_kernel(const DecodeArgs a, const RoundTable tab, const __grid_consta
 }
 
 template <int kTiles, bool kFour>
-cudaError_t launch_rows(const DecodeArgs& a, const RoundTable& t, const CUtensorMap& tmK, const CUtensorMap& tmV, int ctas,
-                        cudaStream_t st) {
+cudaError_t configure_rows() {
   static KvsPerDeviceOnce configured;
-  cudaError_t e = configured.run([] {
+  return configured.run([] {
     return cudaFuncSetAttribute(decode_rows_kernel<kTiles, kFour>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   });
+}
+
+template <int kTiles, bool kFour>
+cudaError_t launch_rows(const DecodeArgs& a, const RoundTable& t, const CUtensorMap& tmK, const CUtensorMap& tmV, int ctas,
+                        cudaStream_t st) {
+  cudaError_t e = configure_rows<kTiles, kFour>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(ctas * a.splits), (unsigned)a.Hkv, (unsigned)t.nseq);
@@ -388,6 +395,43 @@ cudaError_t launch_rows(const DecodeArgs& a, const RoundTable& t, const CUtensor
 }
 
 }  // namespace
+
+// Clusters of 1 to 8 CTAs that are resident at once (entry k: of k CTAs): two CTAs fit an SM, but a cluster has to find its
+// place in one group of SMs, and the groups are not all of one size (one B200: 296, 148, 93, 71, 56, 45, 37 and 33
+// clusters).  Asked once per device for the kernel of the most rows; all of them are bound by shared memory.
+const int* kvs_decode_resident_clusters() {
+  struct Table { std::atomic<int> known; int n[KVS_DECODE_CLUSTER + 1]; };
+  static Table tables[64] = {};
+  static std::mutex mutex;
+  static const int unknown[KVS_DECODE_CLUSTER + 1] = {0, 256, 128, 85, 64, 51, 42, 36, 32};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return unknown;
+  Table& t = tables[dev];
+  if (t.known.load(std::memory_order_acquire)) return t.n;
+  std::lock_guard<std::mutex> lock(mutex);
+  for (int k = 1; k <= KVS_DECODE_CLUSTER; ++k) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)k);
+    cfg.blockDim = dim3(kWarps * 32);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)k;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (configure_rows<2, false>() != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, decode_rows_kernel<2, false>, &cfg) != cudaSuccess || n < 1) {
+      cudaGetLastError();                                  // (the launch itself reports what is wrong)
+      return unknown;
+    }
+    t.n[k] = n;
+  }
+  t.known.store(1, std::memory_order_release);
+  return t.n;
+}
 
 cudaError_t kvs_launch_decode_rows(const DecodeArgs& a, const RoundTable& t, const CUtensorMap& tmK,
                                    const CUtensorMap& tmV, int ctas, cudaStream_t st) {

@@ -159,6 +159,7 @@ cudaError_t kvs_launch_flash_tc(const FlashTcArgs& a, const RoundTable& t, const
 // a (unit, split); with one split the output is final, with more every cluster leaves a partial.
 #define KVS_DECODE_ROWS 16
 #define KVS_DECODE_BLOCK 16        // slots of one box of its K and V tensor maps
+#define KVS_DECODE_CLUSTER 8       // CTAs of a cluster, at most
 struct DecodeArgs {
   const int32_t* counts;   // [U, n_max]
   int32_t n_max, Hkv, M, splits;
@@ -172,6 +173,7 @@ struct DecodeArgs {
   uint32_t wait_us;        // time limit of one device-side wait, microseconds
   uint32_t debug_stall;    // test hook: bit 0 = no tiles are requested
 };
+const int* kvs_decode_resident_clusters();    // entry k: clusters of k CTAs that run at once
 cudaError_t kvs_launch_decode_rows(const DecodeArgs& a, const RoundTable& t, const CUtensorMap& tmK,
                                    const CUtensorMap& tmV, int ctas, cudaStream_t st);
 // Chunk of fresh tokens appended after the slots in use (table entry n = slots in use).

@@ -22,7 +22,8 @@ pytestmark = pytest.mark.gpu
     (4, 1, 1, (3500,), False), (2, 1, 7, (6200, 40), True), (16, 8, 1, tuple(range(17, 17 + 70)), False),
     # nine and sixteen rows on both sides of the lengths that go to the tensor-core tiles
     (9, 1, 1, (5632,), False), (9, 1, 1, (5633,), True), (4, 1, 4, (5700, 5650), False), (16, 1, 1, (16369,), False),
-    # units for clusters of four, two and one CTA in one wave of the GPU, and a ragged batch beyond it
+    # units for clusters of seven to one CTA in one wave of the GPU, and a ragged batch beyond it
+    (36, 36, 1, (900,), False), (40, 20, 2, (800, 790), False), (50, 50, 3, (700,), False), (45, 45, 1, (600, 577), False),
     (24, 24, 1, (700, 640), True), (72, 24, 3, (333, 300, 301, 320, 310), False), (48, 48, 2, (90, 129, 128, 127), False),
     (40, 40, 1, (5200, 40, 33, 70), False)])
 def test_decode_of_few_rows(hq, hkv, t, lens, token_major):
