@@ -251,8 +251,9 @@ bool decode_in_few_rows(int M, const DecodeWork& w) {
 // slots, 8 heads: 7.3 us with eight, 9.8 with four, 25 with one; 64 units of 2048 slots 12.2 us with four, 18.6 with eight;
 // 80 of 3000 24.4 us with three, 28.4 with two, 32.7 with four.
 // Beyond one wave, up to 512 CTAs,
-//   * for ragged batches, whose longest unit would be the last: 64 units of 4096-32768 slots 122 us with eight, 136 with
-//     four; 256 of 512-8192 91 us with two, 109 with eight (for the waits for a cluster's slowest CTA), and
+//   * for ragged batches, whose longest unit would be the last, if its warps keep six blocks: 64 units of 4096-32768 slots
+//     122 us with eight, 136 with four; 168 of 299-1198 21.2 us with two, 26.5 with one; 72 of 124-498 10.6 us with three,
+//     11.8 with six; 256 of 512-8192 91 us with two, 109 with eight (for the waits for a cluster's slowest CTA), and
 //   * for long units whose grid gets near 512 (1.7 waves): 256 units of 8192 slots 159 us with two, 175 with one; of 3000
 //     slots 73 and 70; 128 of 12000 122 us with four, 130 with two; but 96 of 8192 75 and 70 (384 CTAs).
 // (Sixteen took 9 us for 300 slots against 4.8.)  A unit gets more clusters, and a combine kernel, only where SMs are idle and a
@@ -265,7 +266,7 @@ int decode_cluster(const DecodeWork& w, int max_splits, int* splits) {
     if (!fit || w.units + (k > 2) <= fit[k]) c = k;
   for (int k = 2 * c < KVS_DECODE_CLUSTER ? 2 * c : KVS_DECODE_CLUSTER; c < k && c * 4 < w.longest && k * w.units <= 512;
        k = 2 * c < KVS_DECODE_CLUSTER ? 2 * c : KVS_DECODE_CLUSTER) {
-    if (!ragged && !(c < 4 && k * w.units > 3 * kNumSMs && w.longest >= k * 4 * 40)) break;
+    if (w.longest < k * 4 * (ragged ? 6 : 40) || !(ragged || (c < 4 && k * w.units > 3 * kNumSMs))) break;
     c = k;
   }
   int s = 1;
