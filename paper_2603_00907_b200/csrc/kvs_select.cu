@@ -29,7 +29,6 @@ constexpr int kKeep = 32;                  // keys of a thread held in shared me
 constexpr int kBins = 2048;
 constexpr int kMaxCluster = 8;
 constexpr int kPairsPerCta = 4096;         // (see cluster_of)
-constexpr int kFusedPairs = 4096;          // (see kvs_launch_finalize_select)
 
 // Sum of the partials of all (query block, statistics group) pairs in a fixed order, then score and
 // left-key weight of candidate pair p.  Weight modes:
@@ -292,17 +291,26 @@ cudaError_t launch_select(const StatsTcArgs& sa, const SelectArgs& a, const Roun
   return cudaLaunchKernelEx(&cfg, select_kernel<kMode>, sa, a, t);
 }
 
+// Whether the selection kernel adds the partials itself: where they are few (at most two query blocks), and
+//   * a unit has up to 1024 pairs: 8 units of 350 30.3 us a call against 31.1 with a kernel of its own, 32 of 700 40.4 and 43.8;
+//   * there are up to 16 units of up to 3072 pairs, or up to 44000 pairs in all: 16 of 2000 42.5 us and 46.3, 8 of 3000 42.3
+//     and 44.5, 24 of 1760 51.1 and 55.4;
+//   * the units are enough for the GPU: 128 of 2000 175 us and 186.
+// Between them its few CTAs are slow readers: 24 units of 3000 pairs 74 us against 64, 32 of 2000 67 and 61, 64 of 4000
+// 195 and 183, 16 of 4000 63 and 61.
+bool fused_finalize(const StatsTcArgs& sa, const SelectArgs& a, int units, int pmax) {
+  if (!a.select || sa.nqblk > 2 || pmax > 4096) return false;
+  return pmax <= 1024 || units >= 128 || (pmax <= 3072 && (units <= 16 || pmax * units <= 44000));
+}
+
 }  // namespace
 
-// The selection kernel adds the partials itself where they are few: up to 4096 pairs of at most two query blocks
-// (8 units of 2000 pairs, 3 partials: 7.9 us against 2.4 + 8.4; of 8192 pairs 27 against 6.6 + 12).  Its few CTAs
-// are slow readers: 8 units of 4000 pairs with 24 partials 33 us against 8 + 11.
 cudaError_t kvs_launch_finalize_select(const StatsTcArgs& sa, const SelectArgs& a, const RoundTable& t, cudaStream_t st,
                                        int* kernels) {
   *kernels = 1;
   const int pmax = most_pairs(t);
   if (pmax <= 0) return cudaSuccess;
-  if (a.select && pmax <= kFusedPairs && sa.nqblk <= 2) return launch_select<kFused>(sa, a, t, st);
+  if (fused_finalize(sa, a, a.Hkv * t.nseq, pmax)) return launch_select<kFused>(sa, a, t, st);
   cudaError_t e = kvs_launch_chained(finalize_kernel, dim3((pmax + 255) / 256, a.Hkv, t.nseq), dim3(256), 0, st, sa, t);
   if (e != cudaSuccess || !a.select) return e;
   *kernels = 2;

@@ -10,7 +10,11 @@ pytestmark = pytest.mark.gpu
 # KV heads, slots, keys repeated every `period` slots (0: none; with it most scores occur many times)
 @pytest.mark.parametrize("hkv,n,period,first_round", [
     (2, 300, 0, 0), (3, 8200, 0, 1), (3, 8400, 64, 0), (8, 20011, 128, 1), (2, 140000, 0, 0), (2, 140000, 512, 1),
-    (160, 66200, 512, 0)])
+    (160, 66200, 512, 0),
+    # both sides of the lines between one kernel and two (1024 pairs; 3072 with up to 16 units or 44000 in all; 4096 from
+    # 128 units on)
+    (50, 2084, 0, 0), (50, 2086, 32, 0), (17, 5212, 0, 0), (17, 5214, 32, 1), (16, 6181, 64, 1), (16, 6184, 0, 1),
+    (128, 8228, 64, 0), (128, 8230, 0, 0)])
 def test_mask_is_the_smallest_scores(hkv, n, period, first_round):
     import torch
     from paper_2603_00907_b200 import binding as kb, build
