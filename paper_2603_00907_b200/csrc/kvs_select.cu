@@ -28,7 +28,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kKeep = 32;                  // keys of a thread held in shared memory (with more, all are read again)
 constexpr int kBins = 2048;
 constexpr int kMaxCluster = 8;
-constexpr int kPairsPerCta = 4096;         // (see cluster_of)
+constexpr int kPairsPerCta = 4096, kMaskPairsPerCta = 3072;   // (see cluster_of)
 
 // Sum of the partials of all (query block, statistics group) pairs in a fixed order, then score and
 // left-key weight of candidate pair p.  Weight modes:
@@ -244,11 +244,13 @@ int most_pairs(const RoundTable& t) {
 
 // CTAs per unit: one for every 4096 pairs while they all fit the GPU (two per SM).  A cluster's barriers cost about
 // 1.5 us each: 8 units of 16336 pairs 17 us with four CTAs, 28 with eight; 256 units of 16336 pairs 32 us with
-// one, 85 with several waves of clusters of four.
-int cluster_of(const RoundTable& t, int Hkv) {
+// one, 85 with several waves of clusters of four.  The counts of a given mask have one such barrier and take a CTA for
+// 3072 pairs: a compaction of 4 units of 7200 pairs 22.1 us, with half as many 24.0; of 8 units of 16336 63.2 and 64.4;
+// but of 32 units of 2180 74.4 with two CTAs and 70.8 with one.
+int cluster_of(const RoundTable& t, int Hkv, int pairs_per_cta) {
   const int pmax = most_pairs(t);
   int c = 1;
-  while (c < kMaxCluster && c * kPairsPerCta < pmax && (long long)c * 2 * Hkv * t.nseq <= 2 * 148) c *= 2;
+  while (c < kMaxCluster && c * pairs_per_cta < pmax && (long long)c * 2 * Hkv * t.nseq <= 2 * 148) c *= 2;
   return c;
 }
 
@@ -263,7 +265,7 @@ cudaError_t launch_select(const StatsTcArgs& sa, const SelectArgs& a, const Roun
   });
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  const int c = cluster_of(t, a.Hkv);
+  const int c = cluster_of(t, a.Hkv, kMode == kMask ? kMaskPairsPerCta : kPairsPerCta);
   cfg.gridDim = dim3((unsigned)c, (unsigned)a.Hkv, (unsigned)t.nseq);
   cfg.blockDim = dim3(kThreads);
   if (kMode != kMask) {
