@@ -45,8 +45,10 @@ constexpr int kAhead = 4;                  // tiles requested into L2 ahead of t
 constexpr int kSmemQ = 0, kSmemK = kOperand, kSmemV = kSmemK + kKStages * kOperand;
 constexpr int kSmemMisc = kSmemV + kVStages * kOperand;
 constexpr int kSoftmaxWarps = 16, kNormWarps = 8;
-constexpr int kPvWarp = 2 + kSoftmaxWarps + kNormWarps;          // the warp that issues the P V products
-constexpr int kThreads = (kPvWarp + 1) * 32;   // warp 0: TMA, 1: S products, 2-17: softmax, 18-25: pair norms, 26: P V products
+// Warp 0: TMA, 1: S products, 2-17: softmax, 18-25: pair norms (in calls that form them), the last: P V products.  Decode
+// calls are launched without the norm warps: 408 units of three tiles 36.2 -> @@ us.
+template <bool kNorms> constexpr int kPvWarp = 2 + kSoftmaxWarps + (kNorms ? kNormWarps : 0);
+template <bool kNorms> constexpr int kThreads = (kPvWarp<kNorms> + 1) * 32;
 constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: a part of l beyond this asks for another walk
 // From here on a logit (log2 units) is scaled and rounded before the stabiliser, which was rounded the same way, is
 // subtracted.  One fused multiply-add leaves the product unrounded: two equal logits of 2^24 then differ from
@@ -60,7 +62,7 @@ struct Misc {
   int abort_flag, wait_us;                 // (adjacent: the bounded waits read both through one pointer)
   int again;                               // the range is walked again with true maxima
   alignas(16) float cnt[kSoftmaxWarps][64];   // per warp: the counts of its 64 slots (read as float4)
-  float part[4][kTile];                    // the four parts (team x column half) of every row's maximum, then of its sum
+  float part_max[4][kTile], part_sum[4][kTile];   // the four parts (team x column half) of every row's maximum and sum
 };
 constexpr int kSmemBytes = kSmemMisc + (int)sizeof(Misc);
 static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
@@ -149,7 +151,8 @@ __device__ __forceinline__ float rsqrt_newton(float x) {
   return fmaf(y * 0.5f, fmaxf(fmaf(-x * y, y, 1.f), -1.f), y);
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool kNorms>
+__global__ void __launch_bounds__(kThreads<kNorms>, 1)
 flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmQ) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -166,7 +169,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
   // -- roles, TMEM and barrier addresses -- to be the same in every lane)
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   // with pair norms, tile t covers slots [128 t - shift, 128 t - shift + 128): aligned with the pairs
-  const int shift = a.pair_norms ? (tab.off & 1) : 0;
+  const int shift = kNorms ? (tab.off & 1) : 0;
   const int ntiles = (n + shift + kTile - 1) / kTile;
   const int t_begin = min(ntiles, split * a.tiles_per_split);
   const int t_end = min(ntiles, t_begin + a.tiles_per_split);
@@ -189,8 +192,8 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
   }
   // the pair norms of a KV head are shared work of its query blocks: tile t's key cosines belong to block
   // 2 t mod nqblk, its value norms to block 2 t + 1 mod nqblk
-  const bool norm_k = a.pair_norms != nullptr && ((a.nqblk & 1) || !(qblk & 1));
-  const bool norm_v = a.pair_norms != nullptr && ((a.nqblk & 1) || (qblk & 1));
+  const bool norm_k = kNorms && ((a.nqblk & 1) || !(qblk & 1));
+  const bool norm_v = kNorms && ((a.nqblk & 1) || (qblk & 1));
   const int norm_arrivals = norm_k && norm_v ? kNormWarps / 2 : kNormWarps;   // per tile and operand
 
   if (threadIdx.x == 0) {
@@ -228,9 +231,11 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
   volatile int* abort_flag = &misc->abort_flag;
   // test hook: the producer requests no K tile, so that the waits on them run out
   const bool withhold_k = (a.debug_stall & 1u) != 0;
-  // Every role walks the range once and then asks whether it is walked twice more (`again`).  Stages, buffers
-  // and phases go by the tile's number over all walks, gi = walk * my_tiles + li.
+  // Every role walks the range once and then asks whether it is walked twice more (`again`; a range of one tile has
+  // its true maxima from the start).  Stages, buffers and phases go by the tile's number over all walks,
+  // gi = walk * my_tiles + li.
   auto walks = [&]() -> int {
+    if (my_tiles == 1) return 1;
     if (!mbar_wait(&misc->verdict, 0, abort_flag)) return 1;
     return *(volatile int*)&misc->again ? 3 : 1;
   };
@@ -318,7 +323,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
         if (gi == my_tiles - 1) end = walks() * my_tiles;
       }
     }
-  } else if (warp == kPvWarp) {
+  } else if (warp == kPvWarp<kNorms>) {
     // ================================================================ issuer of the P V products
     if (elect_one()) {
       constexpr uint32_t idesc_o = idesc_bf16(128, 128, false, true);    // P' (K-major) x V tile (MN-major)
@@ -448,12 +453,11 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     };
     // the row's maximum from its four parts (all softmax threads together); false if it has no finite logit
     auto set_stab = [&](float mine) -> bool {
-      misc->part[part][row] = mine;
+      misc->part_max[part][row] = mine;                    // (read for the last time before the barrier of the verdict)
       softmax_barrier();
-      const float mx = fmaxf(fmaxf(misc->part[0][row], misc->part[1][row]), fmaxf(misc->part[2][row], misc->part[3][row]));
+      const float mx = fmaxf(fmaxf(misc->part_max[0][row], misc->part_max[1][row]), fmaxf(misc->part_max[2][row], misc->part_max[3][row]));
       m_stab = mx > -INFINITY ? mx * a.scale_log2 : 0.f;
       far = __any_sync(0xffffffffu, fabsf(m_stab) > kFarLogit) != 0;
-      softmax_barrier();                                   // (the parts are written again later)
       return mx > -INFINITY;
     };
     // P' = exp2(scaled logit - m) of 16 slots as hi + lo bf16, two slots per 32-bit column, over the 8 (hi) and
@@ -585,7 +589,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
       gi_last = (walk + 1) * my_tiles - 1;
       if (walk == 1) set_stab(mx);
       l = (ls[0].x + ls[0].y) + (ls[1].x + ls[1].y);
-      if (walk == 0) {
+      if (walk == 0 && my_tiles > 1) {
         if (__any_sync(0xffffffffu, !(l < kSumLimit)) && lane == 0) misc->again = 1;
         warp_arrive(&misc->verdict, lane);
         softmax_barrier();
@@ -594,13 +598,13 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     }
     // ---- the partial of this key range: the four parts of a row's sum are added, and each thread writes 32
     //      channels of the row of O
-    misc->part[part][row] = l;
+    misc->part_sum[part][row] = l;
     softmax_barrier();
     const size_t pidx = ((size_t)unit * a.splits + split) * a.M + m;
     if (alive && warp_wait(&misc->pvdone[gi_last % kSBufs], (gi_last / kSBufs) & 1, abort_flag, lane)) {
       tc_fence_after();
       if (part == 0 && m < a.M) {
-        const float sum = (misc->part[0][row] + misc->part[1][row]) + (misc->part[2][row] + misc->part[3][row]);
+        const float sum = (misc->part_sum[0][row] + misc->part_sum[1][row]) + (misc->part_sum[2][row] + misc->part_sum[3][row]);
         a.part_ml[pidx] = make_float2(sum == 0.f ? -INFINITY : m_stab, sum);   // (a NaN sum is not an empty range)
       }
       float ov[32];
@@ -630,9 +634,15 @@ cudaError_t kvs_launch_flash_tc(const FlashTcArgs& a, const RoundTable& t, const
                                 const CUtensorMap& tmV, const CUtensorMap& tmQ, cudaStream_t st) {
   static KvsPerDeviceOnce configured;
   cudaError_t ce = configured.run([] {
-    return cudaFuncSetAttribute(flash_partial_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    for (auto k : {flash_partial_tc<false>, flash_partial_tc<true>}) {
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
   });
   if (ce != cudaSuccess) return ce;
   dim3 grid(a.nqblk * a.splits, a.Hkv, t.nseq);
-  return kvs_launch_chained(flash_partial_tc, grid, dim3(kThreads), kSmemBytes, st, a, t, tmK, tmV, tmQ);
+  const bool norms = a.pair_norms != nullptr;
+  return kvs_launch_chained(norms ? flash_partial_tc<true> : flash_partial_tc<false>, grid,
+                            dim3(norms ? kThreads<true> : kThreads<false>), kSmemBytes, st, a, t, tmK, tmV, tmQ);
 }
