@@ -59,6 +59,83 @@ def test_attention_wait_runs_out_then_the_next_call_is_clean(kb):
         assert ok, mx
 
 
+def test_tile_attention_wait_runs_out_then_the_next_call_is_clean(kb):
+    """As above with 32 rows per KV head, which take the tensor-core tiles (up to 16 rows have a kernel of their own)."""
+    import torch
+    w = tp._small(seed=44, batch=1, n_q_heads=8, n_kv_heads=2, window=8, seq_lens=(600,), budgets=(600,), n_decode=8)
+    data = wl.make_layer(w)
+    dev, p, ws = tp._setup(kb, w, data)
+    out = torch.zeros((1, w.n_q_heads, 8, 128), dtype=torch.bfloat16, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    kb.kvs_debug_set_wait(LIMIT_US, 1)
+    try:
+        kb.kvs_decode_attn(p, dev["q_new"], dev["K"], dev["V"], dev["counts"], [600], out, ws, status_dev=status)
+        torch.cuda.synchronize()
+    finally:
+        kb.kvs_debug_set_wait(0, 0)
+    assert status.item() == KVS_ERR_TIMEOUT
+    status.zero_()
+    kb.kvs_decode_attn(p, dev["q_new"], dev["K"], dev["V"], dev["counts"], [600], out, ws, status_dev=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    G = w.group
+    for h in range(w.n_kv_heads):
+        ref, _ = oc.decode_attention(data["q_new"][0, h * G:(h + 1) * G], data["K"][0, h, :600], data["V"][0, h, :600],
+                                     data["counts"][0, h, :600])
+        ok, mx, _, _ = tl.bf16_close(tl.bits_of(out)[0, h * G:(h + 1) * G], oc.f64_to_bf16(ref))
+        assert ok, mx
+
+
+@pytest.mark.parametrize("window", [8, 40])
+def test_window_attention_wait_runs_out_then_the_next_call_is_clean(kb, window):
+    """The attention of the window pass, whose pair-norm warps wait for the same tiles: one query block, and two that share
+    the norms."""
+    import torch
+    w = tp._small(seed=45, batch=1, n_q_heads=8, n_kv_heads=2, window=window, seq_lens=(900,), budgets=(300,))
+    data = wl.make_layer(w)
+    dev, p, ws = tp._setup(kb, w, data)
+    score = torch.zeros((1, 2, w.n_max // 2), dtype=torch.float32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    kb.kvs_debug_set_wait(LIMIT_US, 1)
+    try:
+        kb.kvs_window_stats(p, dev["K"], dev["V"], dev["counts"], dev["q_win"], [900], [300], ws, score=score,
+                            status_dev=status)
+        torch.cuda.synchronize()
+    finally:
+        kb.kvs_debug_set_wait(0, 0)
+    assert status.item() == KVS_ERR_TIMEOUT
+    tp._check_round_stats(kb, w, data["K"], data["V"], data["counts"], data["q_win"], [900], 0)
+
+
+def test_statistics_wait_runs_out_in_equal_shares_too(kb):
+    """A ragged batch of 192 units, whose tiles the statistics kernel deals out in equal shares."""
+    import torch
+    lens = [1300, 1170, 400, 1290, 1301, 700, 1024, 300] * 3
+    w = wl.small_case(seed=46, batch=len(lens), n_q_heads=32, n_kv_heads=8, window=16, seq_lens=tuple(lens),
+                      budgets=tuple(n - n // 6 for n in lens))
+    data = wl.make_layer(w)
+    dev, p, ws = tp._setup(kb, w, data)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def score():
+        out = torch.zeros((len(lens), 8, w.n_max // 2), dtype=torch.float32, device="cuda")
+        kb.kvs_window_stats(p, dev["K"], dev["V"], dev["counts"], dev["q_win"], lens, list(w.budgets), ws, score=out,
+                            status_dev=status)
+        torch.cuda.synchronize()
+        return out
+
+    before = score()
+    assert status.item() == 0
+    kb.kvs_debug_set_wait(LIMIT_US, 2)
+    try:
+        score()
+    finally:
+        kb.kvs_debug_set_wait(0, 0)
+    assert status.item() == KVS_ERR_TIMEOUT
+    status.zero_()
+    assert torch.equal(score(), before) and status.item() == 0
+
+
 def test_statistics_wait_runs_out_then_the_next_call_is_clean(kb):
     import torch
     w = tp._small(seed=42, batch=1, n_q_heads=8, n_kv_heads=2, window=8, seq_lens=(900,), budgets=(300,))

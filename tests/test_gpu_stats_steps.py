@@ -36,6 +36,44 @@ def test_shares_that_cross_units(group, window, hkv):
     parity._check_round_stats(kb, w, data["K"], data["V"], data["counts"], data["q_win"], list(w.seq_lens), 1)
 
 
+@pytest.mark.parametrize("mode", [1, 2])
+def test_shares_that_cross_units_with_a_supplied_gradient(mode):
+    """The same batch in the exact weight modes: two query operands instead of three are replaced from unit to unit.  Units
+    at both ends of the walk and of a sequence, a short one, and one of two ragged tiles, against the oracle."""
+    import torch
+    from oracle import kvs_oracle as oc
+    from paper_2603_00907_b200 import binding as kb, build
+    from tests import kvs_testlib as tl
+    build.build()
+    lens = [1300, 1170, 400, 1290, 1301, 700, 1024, 300] * 3
+    hkv, G, W = 8, 4, 16
+    w = wl.small_case(seed=8, batch=len(lens), n_q_heads=G * hkv, n_kv_heads=hkv, window=W, seq_lens=tuple(lens),
+                      budgets=tuple(n - n // 6 for n in lens))
+    data = wl.make_layer(w)
+    rng = np.random.default_rng(8)
+    data["counts"][:] = rng.integers(1, 4, size=data["counts"].shape)
+    E = wl.f32_to_bf16_bits(rng.standard_normal(data["q_win"].shape).astype(np.float32))
+    dev, p, ws = parity._setup(kb, w, data)
+    B, n_max = w.batch, w.n_max
+    A, gs = (torch.zeros(B, hkv, n_max, device="cuda") for _ in range(2))
+    gp = torch.zeros(B, hkv, n_max // 2, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    kb.kvs_window_stats_exact(p, dev["K"], dev["V"], dev["counts"], dev["q_win"], tl.to_dev_bf16(E), mode, lens,
+                              list(w.budgets), ws, A=A, g_self=gs, g_pair=gp, status_dev=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    for b, h in ((0, 0), (0, 7), (1, 0), (2, 3), (7, 7), (11, 4), (15, 0), (23, 7)):
+        n, hs = lens[b], slice(h * G, (h + 1) * G)
+        st = oc.round_stats(data["K"][b, h, :n], data["V"][b, h, :n], data["counts"][b, h, :n].astype(np.int64),
+                            data["q_win"][b, hs], w.budgets[b], 0, weight_mode=mode, E_bits=E[b, hs], **parity._oracle_kwargs(w))
+        off, P, ab = st["off"], st["P"], st["Gabs"]
+        ok, _, plain = tl.rel_close(A[b, h, off:off + 2 * P].cpu().numpy(), st["A"][off:off + 2 * P])
+        assert ok, (b, h, plain)
+        g = gs[b, h, off:off + 2 * P].cpu().numpy()
+        for got, want, size in ((g[::2], st["G11"], ab[0]), (g[1::2], st["G22"], ab[1]), (gp[b, h, :P].cpu().numpy(), st["G12"], ab[2])):
+            assert np.all(np.abs(got - want) <= tl.STAT_RTOL * size + 1e-37), (b, h)
+
+
 @pytest.mark.parametrize("seed", [1, 2])
 def test_values_around_a_mean(seed):
     """|vbar - o|^2 is a small difference of terms of about |mean|^2 = 128 here, and <vbar, o> comes from sixteen
