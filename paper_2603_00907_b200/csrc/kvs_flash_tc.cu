@@ -46,7 +46,7 @@ constexpr int kSmemQ = 0, kSmemK = kOperand, kSmemV = kSmemK + kKStages * kOpera
 constexpr int kSmemMisc = kSmemV + kVStages * kOperand;
 constexpr int kSoftmaxWarps = 16, kNormWarps = 8;
 // Warp 0: TMA, 1: S products, 2-17: softmax, 18-25: pair norms (in calls that form them), the last: P V products.  Decode
-// calls are launched without the norm warps: 408 units of three tiles 36.2 -> @@ us.
+// calls are launched without the norm warps: 408 units of three tiles 35.9 -> 34.7 us.
 template <bool kNorms> constexpr int kPvWarp = 2 + kSoftmaxWarps + (kNorms ? kNormWarps : 0);
 template <bool kNorms> constexpr int kThreads = (kPvWarp<kNorms> + 1) * 32;
 constexpr float kSumLimit = 1.152921504606847e18f;   // 2^60: a part of l beyond this asks for another walk
@@ -436,7 +436,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     const int part = team * 2 + ch;
     float* cnt = misc->cnt[warp - 2];
     bool alive = true;
-    float m_stab = 0.f, l = 0.f;             // the stabiliser (log2 units) and this thread's part of l
+    float m_stab = 0.f;                      // the stabiliser (log2 units)
     bool far = false;                        // a row of the warp has one beyond kFarLogit
     // masks the logits of 16 slots from j0 on
     auto mask16 = [&](int j0, float* x) {
@@ -588,18 +588,18 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
       }
       gi_last = (walk + 1) * my_tiles - 1;
       if (walk == 1) set_stab(mx);
-      l = (ls[0].x + ls[0].y) + (ls[1].x + ls[1].y);
+      if (walk == 1) continue;
+      const float l = (ls[0].x + ls[0].y) + (ls[1].x + ls[1].y);   // this thread's part of l
+      misc->part_sum[part][row] = l;                       // (of the first walk, if there are more: not read)
       if (walk == 0 && my_tiles > 1) {
         if (__any_sync(0xffffffffu, !(l < kSumLimit)) && lane == 0) misc->again = 1;
         warp_arrive(&misc->verdict, lane);
-        softmax_barrier();
-        if (*(volatile int*)&misc->again) n_walks = 3;     // (the same for all softmax threads)
       }
+      softmax_barrier();
+      if (walk == 0 && my_tiles > 1 && *(volatile int*)&misc->again) n_walks = 3;   // (the same for all softmax threads)
     }
     // ---- the partial of this key range: the four parts of a row's sum are added, and each thread writes 32
     //      channels of the row of O
-    misc->part_sum[part][row] = l;
-    softmax_barrier();
     const size_t pidx = ((size_t)unit * a.splits + split) * a.M + m;
     if (alive && warp_wait(&misc->pvdone[gi_last % kSBufs], (gi_last / kSBufs) & 1, abort_flag, lane)) {
       tc_fence_after();
