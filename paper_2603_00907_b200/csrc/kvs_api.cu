@@ -170,7 +170,7 @@ size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct WsLayout {
   size_t part_ml, part_o, qc2, norms, o_hi, o_lo, score, w, mask, tile_prefix, part4, part1, sync, total;
-  int splits_max, M_max, pair_stride, tile_stride, counter_stride, nqblk_w, U;
+  int M_max, pair_stride, tile_stride, nqblk_w, U;
   size_t sync_bytes;
 };
 
@@ -294,7 +294,6 @@ WsLayout make_layout(const kvs_params_t* p, int n_max, int max_new) {
   const int sw = splits_bound(Mw, p->n_kv_heads), sd = max_new > 0 ? splits_bound(Md, p->n_kv_heads) : 0;
   const size_t rows_w = (size_t)sw * Mw, rows_d = (size_t)sd * Md;
   const size_t part_rows = rows_w > rows_d ? rows_w : rows_d;
-  L.splits_max = sw > sd ? sw : sd;
   L.U = p->batch * p->n_kv_heads;
   L.pair_stride = n_max / 2 + 1;
   L.tile_stride = n_max / KVS_CTILE + 2;
@@ -310,16 +309,13 @@ WsLayout make_layout(const kvs_params_t* p, int n_max, int max_new) {
   L.o_hi = o;    o += align_up((size_t)L.U * L.M_max * KVS_D * sizeof(__nv_bfloat16));
   L.o_lo = o;    o += align_up((size_t)L.U * L.M_max * KVS_D * sizeof(__nv_bfloat16));
   L.nqblk_w = (Mw + 127) / 128;
-  L.counter_stride = n_max / 128 + 2;
   // partial sums of every (query block, statistics group): five floats per candidate pair
   const size_t nsub = (size_t)L.nqblk_w * KVS_STATS_GROUPS;
   L.part4 = o;   o += align_up((size_t)L.U * nsub * L.pair_stride * sizeof(float4));
   L.part1 = o;   o += align_up((size_t)L.U * nsub * L.pair_stride * sizeof(float));
-  // tickets [KVS_MAX_ROUNDS][U], flags [U][tile_stride], tile counters [U][counter_stride];
-  // zeroed once per call
+  // tickets [KVS_MAX_ROUNDS][U], flags [U][tile_stride]; zeroed once per call
   L.sync = o;
-  L.sync_bytes = align_up(((size_t)KVS_MAX_ROUNDS * L.U + (size_t)L.U * L.tile_stride +
-                           (size_t)L.U * L.counter_stride) * sizeof(uint32_t));
+  L.sync_bytes = align_up(((size_t)KVS_MAX_ROUNDS * L.U + (size_t)L.U * L.tile_stride) * sizeof(uint32_t));
   o += L.sync_bytes;
   L.total = o;
   return L;

@@ -165,3 +165,16 @@ def test_shared_arrays_read_as_wider_words_declare_that_alignment():
             assert declared and int(declared.group(1)) >= size[kind], (name, var, kind)
             seen += 1
     assert seen
+
+
+def test_workspace_holds_no_more_than_its_parts(lib):
+    """The tickets and flags, which the first selection of every call zeroes, are all there is beside the arrays."""
+    p = _params(batch=3)
+    n, new, U, G = 4096, 4, 24, 4
+    up = lambda x: (x + 255) & ~255
+    Mw, pairs, tiles = G * 32, n // 2 + 1, n // 64 + 2
+    splits = max(148 // 8, 16, -(-2 * 148 // 8))
+    rows = splits * Mw
+    parts = [U * rows * 8, U * rows * 512, U * 128 * 8, U * pairs * 16, U * pairs * 4, U * pairs * 4, U * pairs, U * tiles * 4,
+             U * Mw * 256, U * Mw * 256, U * 3 * pairs * 16, U * 3 * pairs * 4, (64 * U + U * tiles) * 4]
+    assert kb.kvs_workspace_size(p, n, new) == sum(up(x) for x in parts)
