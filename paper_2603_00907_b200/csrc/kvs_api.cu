@@ -181,8 +181,8 @@ struct WsLayout {
 // half-length waves instead of 4 full ones); 64 items of 1024 tiles: k = 9 (576 CTAs in 4 waves of 114
 // tiles instead of 128 CTAs of 512 tiles on 148 SMs); 8 items of 16 tiles: k = 16; 64 items of 32 to 402
 // tiles: k = 9 where counting all as the longest took 8.  When the CTAs need more than one wave, a
-// range is not made shorter than 16 tiles: the pipeline of a CTA (three logit buffers, two
-// K/V stages) takes a few tiles to fill, which the model's constant does not cover -- 512 items of
+// range is not made shorter than 16 tiles: the pipeline of a CTA (three logit buffers, three K and two
+// V stages) takes a few tiles to fill, which the model's constant does not cover -- 512 items of
 // 20 tiles ran 2.4 % faster uncut (4 waves of 20 tiles) than cut in two (7 waves of 10), while a
 // larger constant instead slowed the long ragged items of the other workloads by up to 6 %.
 struct TileCut {
@@ -742,7 +742,6 @@ kvs_status_t merge_layer_impl(const kvs_params_t* p, void* K, void* V, int32_t* 
       ka.new_index = nullptr;
       ka.status_dev = status_dev;
       ka.wait_us = g_wait_us.load(); ka.debug_stall = g_debug_stall.load();
-    ka.wait_us = g_wait_us.load(); ka.debug_stall = g_debug_stall.load();
       CUDA_TRY(launch(KVS_K_COMPACT, c.st, [&] { return kvs_launch_compact(ka, tab, c.st); }));
     }
   }

@@ -1,7 +1,7 @@
 // Attention partials on the tensor cores (tcgen05 + TMEM + TMA), queries on TMEM lanes.
 //
 // One CTA owns a block of 128 query rows (Q is staged once in shared memory) and a contiguous range
-// of 128-slot tiles.  K and V tiles travel in two separate two-stage TMA rings; per tile one
+// of 128-slot tiles.  K tiles travel in a three-stage TMA ring and V tiles in one of two stages; per tile one
 // thread issues
 //   S[q, slot] = Q K_tile^T                         (fp32 in TMEM, three buffers: the logits run two tiles
 //                                                    ahead of the P V products, so that a softmax team that
@@ -12,7 +12,7 @@
 // P' = exp(s - m), split into two bf16 terms, and stores them back into the very columns the
 // logits came from (16 logits make 8 columns of hi and 8 of lo terms), keeping its part of
 // l = sum_j c_j exp(s_j - m): the count bias ln c_j of a merged slot is just the factor c_j in
-// that sum.  The issuing thread then runs
+// that sum.  Another issuing thread then runs
 //   O[q, :] += (P'_hi + P'_lo) Vsum_tile            (P' from tensor memory, V as the MN-major operand)
 // with the one O accumulating in TMEM across all tiles [Eq. attn_def_vec with merged slots:
 // o = sum_j alpha_j Vsum_j / c_j].  At the end the CTA writes (stabiliser, sum, O) as the partial
@@ -397,8 +397,9 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
         if (!warp_wait(full + st, ph, abort_flag, lane)) { ok_all = false; break; }
         float ll = 0.f, rr = 0.f, lr = 0.f;
         if (mine) pair_dots(rows + st * kOperand, row0, steps, lane, ll, rr, lr);
-        // the rows are no longer needed here.  (The test is always true: it makes the arrival wait for the loads, whose
-        // results the compiler may otherwise collect after it.)
+        // the rows are no longer needed here.  (The test is always true: it makes the arrival wait for the loads' results.
+        // The barrier of the warp and the arrival order the loads already; this way their data are in registers, too,
+        // as in every other place of these kernels where a stage is handed back to the TMA.)
         __syncwarp();
         if (lane == 0 && !(ll < -1.f)) mbar_arrive(freed + st);
         if (++st == stages) { st = 0; ph ^= 1; }

@@ -143,13 +143,13 @@ struct CompactArgs {
 // ----------------------------------------------------------------------------- launchers
 // Each returns the cudaError_t of its launch.  `nseq_units` = table.nseq * Hkv.
 cudaError_t kvs_launch_combine(const CombineArgs& a, const RoundTable& t, cudaStream_t st);
-// tmKp / tmVp: 5-D pair views [128, parity, slot / 2, head, sequence] of the caches; with
-// weight_mode != 0, tmOhi is the map of the supplied gradient rows E and tmOlo is not used
 // groups of `nqblk` CTAs that share out `tiles` (one CTA per SM)
 inline int kvs_stats_groups(int nqblk, int tiles) {
   const int fit = 148 / nqblk < tiles ? 148 / nqblk : tiles;
   return fit > 1 ? fit : 1;
 }
+// tmKp / tmVp: 5-D pair views [128, parity, slot / 2, head, sequence] of the caches; with
+// weight_mode != 0, tmOhi is the map of the supplied gradient rows E and tmOlo is not used
 cudaError_t kvs_launch_stats_tc(const StatsTcArgs& a, const RoundTable& t, const CUtensorMap& tmKp,
                                 const CUtensorMap& tmVp, const CUtensorMap& tmQ, const CUtensorMap& tmOhi,
                                 const CUtensorMap& tmOlo, cudaStream_t st);
