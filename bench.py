@@ -107,15 +107,15 @@ class ClockSampler(threading.Thread):
                 "reasons": sorted(reasons), "samples": len(sm), "scope": scope}
 
 
-# DRAM traffic of each kernel kind as a multiple of its algorithmic bytes, from the ncu captures
-# summarised under profiles/ (dram__bytes_read.sum + dram__bytes_write.sum of rounds 0 and 1 of a
-# 10-layer case, whose inputs exceed L2; traffic grows with the units processed, so the ratio
-# carries over to a full launch).  Each entry names the kernel source it was taken on: once that
-# file changes, the figure is stale and `traffic` is reported as null.
+# DRAM traffic of each kernel kind as a multiple of its algorithmic bytes, from the ncu capture
+# summarised in profiles/large_kernels_2x32k.md (dram__bytes_read.sum + dram__bytes_write.sum of one
+# round of two sequences of 32 K slots, whose inputs exceed L2; traffic grows with the units
+# processed, so the ratio carries over to a full launch).  Each entry names the kernel source it was
+# taken on: once that file changes, the figure is stale and `traffic` is reported as null.
 NCU_TRAFFIC = {
-    "hessian_stats": (1.12, "kvs_stats_tc.cu", "2daefb055af8f342"),
-    "attn_partials": (1.08, "kvs_flash_tc.cu", "1e5de049a90cbae9"),
-    "merge_compact": (0.98, "kvs_compact.cu", "4da4e4dd3c26a8df"),
+    "hessian_stats": (1.11, "kvs_stats_tc.cu", "5565af8be512ae8a"),
+    "attn_partials": (1.05, "kvs_flash_tc.cu", "b9f292f6f3f403de"),
+    "merge_compact": (0.90, "kvs_compact.cu", "3624b502768ce023"),
 }
 
 
