@@ -1,6 +1,8 @@
 """The attention kernel's stabiliser is the maximum over a CTA's first tile of 128 slots.  Rows whose later logits
 are larger by a little, by almost and by more than the range of an exponent of a part of the sum allows (2^60: the
 CTA then walks its slots again with the true maxima), and rows whose first tiles are negligible, against the oracle.
+The first test has few units, whose slots are cut into ranges of one tile each (each with its own stabiliser); the others
+have so many that a CTA walks eight or nine tiles.
 
 P' carries 16 significant bits and is at most 2^60 times the first tile's largest: the relative error of an
 output stays 2^-17 max |V / c|, below 1e-4 here, plus the fp32 error of a logit of up to 320 (2^-24 * 320 = 2e-5,
