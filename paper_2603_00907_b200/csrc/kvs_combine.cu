@@ -15,7 +15,9 @@ constexpr int kCombineRows = 8;
 // kBatch: partial outputs of a row that are requested together.  With few rows the kernel is a chain of L2
 // round trips, and shorter with eight (1024 rows of 9-37 ranges: 8.5-10 -> 5.3 us); with many rows it is
 // bound by bytes in flight, and the registers of a batch cost occupancy (8192 rows of 8 ranges: 9 us one by one,
-// 15 us in eights; 65536 rows of 2: 24 and 75 us).
+// 15 us in eights; 65536 rows of 2: 24 and 75 us).  Between them four (58 registers: four CTAs to an SM): 16 units of 189 rows
+// and 2 to 7 ranges 14.6 us a call, one by one 18.3, in eights 15.6; 16 units of 224 rows 83.9, 88.4 and 84.6; 32
+// units of 256 rows 85.6, 84.8 and 88.9.
 template <int kBatch>
 __global__ void __launch_bounds__(kCombineRows * 32)
 combine_partials(const CombineArgs a, const RoundTable tab) {
@@ -145,5 +147,7 @@ cudaError_t kvs_launch_combine(const CombineArgs& a, const RoundTable& t, cudaSt
   dim3 grid((rows + kCombineRows - 1) / kCombineRows, a.Hkv, t.nseq);
   if ((long long)grid.x * grid.y * grid.z <= 2 * 148)      // one wave
     return kvs_launch_chained(combine_partials<8>, grid, dim3(kCombineRows * 32), kTwoPerSM, st, a, t);
+  if ((long long)grid.x * grid.y * grid.z <= 4 * 148)
+    return kvs_launch_chained(combine_partials<4>, grid, dim3(kCombineRows * 32), 0, st, a, t);
   return kvs_launch_chained(combine_partials<1>, grid, dim3(kCombineRows * 32), 0, st, a, t);
 }
