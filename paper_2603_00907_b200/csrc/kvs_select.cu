@@ -4,17 +4,20 @@
 // (32 candidate pairs each), a thread one pair of every 1024.  The cluster
 //   1. adds the statistics kernel's partial sums of every pair in a fixed order and forms the pair's
 //      score and left-key weight (for long rounds a kernel of its own does that, see below),
-//   2. finds the bit pattern of the R-th smallest score by a radix select in three passes of 11, 11
-//      and 10 bits (scores are non-negative floats: their bit patterns order like unsigned integers);
-//      every CTA counts its own keys in shared memory and adds up the cluster's histograms,
+//   2. finds the bit pattern of the R-th smallest score (scores are non-negative floats: their bit patterns order
+//      like unsigned integers).  A pass counts the keys of an interval in 4096 bins and goes on with the bin
+//      that holds the R-th; two passes are the rule, since it ends when a bin is taken as a whole,
 //   3. writes the mask (ties at the cutoff are taken in index order) and, for every compaction tile,
 //      the number of merged pairs that precede it.
-// The keys stay in shared memory from the first step to the last.  Latency bound: barriers, L2 round trips
-// and instruction fetches -- every instruction runs a few times only, so the loops are kept rolled (keys
-// in registers and unrolled loops took 2.5 k cycles a pass).
-// Measured, statistics' finalize + selection of a round, one CTA per unit and four passes -> this:
-// 8 units of 2000 pairs 11.0 -> 7.9 us, of 16336 pairs 36.5 -> 24 us; 64 units of 2.5-32 k pairs 42 -> 27 us;
-// 8 units of 65 k pairs and 24 partials a pair 73 -> 47 us.  The counts of a given mask (65 k pairs): 18 -> 7.5 us.
+// A warp owns consecutive tiles, so that the counts in front of a tile need one barrier a launch.
+// The keys stay in shared memory from the first step to the last.  Latency bound: barriers (of a cluster 1.1 k cycles
+// each), L2 round trips and issue slots, of which an instruction of all 1024 threads takes eight on every scheduler.
+// Measured, clock64 from the wait for the kernel before to the end, three passes of 11, 11 and 10 bits with all counts
+// read from the other CTAs and a barrier for every 1024 pairs -> this: 8 units of 2000 pairs 14.7 -> 11.0 k cycles, of
+// 4096 16.2 -> 10.4, of 16336 23.9 -> 13.7, of 65 k 41.8 -> 20.4 k.  With the finalize kernel, us by events: 8 units of 16336
+// pairs 28.0 -> 17.9, 13 rounds of 8 units from 65 k pairs on 557 -> 428.
+// (Listing the keys of the first pass's bin and ranking them by comparison in place of the second pass: 140 keys
+// 3.7 k cycles, 480 keys 18 k.)
 #include <cooperative_groups.h>
 
 #include "kvs_internal.h"
@@ -26,7 +29,8 @@ namespace {
 constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int kKeep = 32;                  // keys of a thread held in shared memory (with more, all are read again)
-constexpr int kBins = 2048;
+constexpr int kBinBits = 12, kBins = 1 << kBinBits;   // of a pass
+static_assert(kBins == 4 * kThreads, "a thread sums four bins");
 constexpr int kMaxCluster = 8;
 constexpr int kPairsPerCta = 4096, kMaskPairsPerCta = 3072;   // (see cluster_of)
 
@@ -37,12 +41,12 @@ constexpr int kPairsPerCta = 4096, kMaskPairsPerCta = 3072;   // (see cluster_of
 //                                                                            [Eq. kstar_weight_final_rewrite]
 //   2: as 1 with the coupling dropped, w = G11 / (G11 + G22)                              [Eq. simplified_k]
 // A denominator that is not safely positive gives 1/2; the weight is clipped to [0, 1].
-__device__ __forceinline__ float finalize_pair(const StatsTcArgs& a, int unit, int off, int p) {
-  const int jl = off + 2 * p;
+struct PairSums { float Al, Ar, N1l, N1r, N12, cosv; };
+__device__ __forceinline__ PairSums pair_sums(const StatsTcArgs& a, int unit, int p) {
   const int nsub = a.nqblk * KVS_STATS_GROUPS;
   const float4* p4 = a.part4 + (size_t)unit * nsub * a.pair_stride + p;
   const float* p1 = a.part1 + (size_t)unit * nsub * a.pair_stride + p;
-  float Al = 0.f, Ar = 0.f, N1l = 0.f, N1r = 0.f, N12 = 0.f;
+  PairSums s = {0.f, 0.f, 0.f, 0.f, 0.f, a.pair_norms[(size_t)unit * a.norm_stride + p].w};
   for (int sb = 0; sb < nsub; sb += KVS_STATS_GROUPS) {
     float4 v[KVS_STATS_GROUPS];
     float x[KVS_STATS_GROUPS];
@@ -52,49 +56,42 @@ __device__ __forceinline__ float finalize_pair(const StatsTcArgs& a, int unit, i
       x[i] = p1[(size_t)(sb + i) * a.pair_stride];
     }
 #pragma unroll
-    for (int i = 0; i < KVS_STATS_GROUPS; ++i) { Al += v[i].x; Ar += v[i].y; N1l += v[i].z; N1r += v[i].w; N12 += x[i]; }
+    for (int i = 0; i < KVS_STATS_GROUPS; ++i) { s.Al += v[i].x; s.Ar += v[i].y; s.N1l += v[i].z; s.N1r += v[i].w; s.N12 += x[i]; }
   }
-  const float cosv = a.pair_norms[(size_t)unit * a.norm_stride + p].w;
-  const float mass = Al + Ar;
-  const float score = (a.score_mode == 0) ? mass * fmaxf(0.f, 1.f - cosv) : mass;
+  return s;
+}
+__device__ __forceinline__ float finish_pair(const StatsTcArgs& a, int unit, int off, int p, const PairSums& s) {
+  const int jl = off + 2 * p;
+  const float mass = s.Al + s.Ar;
+  const float score = (a.score_mode == 0) ? mass * fmaxf(0.f, 1.f - s.cosv) : mass;
   float w = 0.5f;
   if (a.weight_mode == 0) {
-    const float D = N1l - 2.f * N12 + N1r;
-    if (D > 1e-6f * (N1l + N1r) && D < INFINITY) w = fminf(1.f, fmaxf(0.f, (N1l - N12) / D));
+    const float D = s.N1l - 2.f * s.N12 + s.N1r;
+    if (D > 1e-6f * (s.N1l + s.N1r) && D < INFINITY) w = fminf(1.f, fmaxf(0.f, (s.N1l - s.N12) / D));
   } else {
-    const float g12 = (a.weight_mode == 2) ? 0.f : N12;
-    const float gamma = N1l + 2.f * g12 + N1r;
-    if (gamma > 1e-6f * (fabsf(N1l) + fabsf(N1r)) && gamma < INFINITY) w = fminf(1.f, fmaxf(0.f, (N1l + g12) / gamma));
+    const float g12 = (a.weight_mode == 2) ? 0.f : s.N12;
+    const float gamma = s.N1l + 2.f * g12 + s.N1r;
+    if (gamma > 1e-6f * (fabsf(s.N1l) + fabsf(s.N1r)) && gamma < INFINITY) w = fminf(1.f, fmaxf(0.f, (s.N1l + g12) / gamma));
   }
   const size_t pi = (size_t)unit * a.pair_stride + p;
   a.score[pi] = fabsf(score);
   a.w[pi] = w;
-  if (a.N12) a.N12[pi] = N12;
-  if (a.cosv) a.cosv[pi] = cosv;
-  if (a.A) { a.A[(size_t)unit * a.n_max + jl] = Al; a.A[(size_t)unit * a.n_max + jl + 1] = Ar; }
-  if (a.N1) { a.N1[(size_t)unit * a.n_max + jl] = N1l; a.N1[(size_t)unit * a.n_max + jl + 1] = N1r; }
+  if (a.N12) a.N12[pi] = s.N12;
+  if (a.cosv) a.cosv[pi] = s.cosv;
+  if (a.A) { a.A[(size_t)unit * a.n_max + jl] = s.Al; a.A[(size_t)unit * a.n_max + jl + 1] = s.Ar; }
+  if (a.N1) { a.N1[(size_t)unit * a.n_max + jl] = s.N1l; a.N1[(size_t)unit * a.n_max + jl + 1] = s.N1r; }
   return fabsf(score);
 }
 
-// Exclusive prefix of `v` over the threads of the CTA (one barrier; `s_warp` is free again after the next one).
-__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* s_warp) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t inc = v;
+// Inclusive prefix over the lanes of the warp.
+__device__ __forceinline__ uint32_t warp_scan(uint32_t v) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
+    const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
   }
-  if (lane == 31) s_warp[warp] = inc;
-  __syncthreads();
-  uint32_t w = s_warp[lane];                               // (32 warps, 32 lanes)
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, w, o);
-    if (lane >= o) w += t;
-  }
-  const uint32_t before = warp ? __shfl_sync(0xffffffffu, w, warp - 1) : 0u;
-  return before + inc - v;
+  return v;
 }
 
 // Step 1 alone, over the whole GPU: one thread per pair.
@@ -105,26 +102,35 @@ finalize_kernel(const StatsTcArgs a, const RoundTable tab) {
   const SeqRound sr = tab.s[blockIdx.z];
   const int p = blockIdx.x * 256 + threadIdx.x;
   if (sr.n <= 0 || p >= sr.P) return;
-  finalize_pair(a, sr.b * a.Hkv + blockIdx.y, tab.off, p);
+  const int unit = sr.b * a.Hkv + blockIdx.y;
+  finish_pair(a, unit, tab.off, p, pair_sums(a, unit, p));
 }
 
+// The digit of the first pass: 64 bins to an octave of the score from 2^-56 to 2^8; what lies outside joins the first
+// or the last bin.  (It grows with the score, and the bins are so narrow that few scores share the cutoff's.)
+constexpr int kFirstBin = (127 - 56) << 6;
+__device__ __forceinline__ int first_digit(uint32_t v) { return min(max((int)(v >> 17) - kFirstBin, 0), kBins - 1); }
+
 // kFused: step 1 too; kScores: the scores are in memory; kMask: the mask is an input (kvs_compact) and only
-// the counts of step 3 are formed.
-enum { kFused = 0, kScores = 1, kMask = 2 };
-template <int kMode>
-__global__ void __launch_bounds__(kThreads, 2)
+// the counts of step 3 are formed.  kFusedFew: as kFused, with the registers of a whole SM to a CTA and two pairs a thread in flight
+// (8 units of 2000 pairs: the first step 6700 -> 4700 cycles, most of which the partials' 150 KB take to get to one SM).
+// kCluster: more than one CTA to a unit; with the scores in memory one CTA to an SM, too: at the 32 registers of two, the
+// passes spilled (8 units of 16336 pairs: 21.7 k cycles against 13.7 k).
+enum { kFused = 0, kScores = 1, kMask = 2, kFusedFew = 3 };
+template <int kMode, bool kCluster>
+__global__ void __launch_bounds__(kThreads, kMode == kFusedFew || (kMode == kScores && kCluster) ? 1 : 2)
 select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
   constexpr bool kFromMask = kMode == kMask;
   extern __shared__ uint32_t s_key[];
-  __shared__ alignas(8) uint32_t s_hist[3][kBins];       // (read as pairs of bins)
-  __shared__ uint32_t s_warp[2][kWarps], s_digit, s_k, s_total[2], s_cnt[2][kWarps];
+  // two passes' counts in turn: a CTA still reads those of one pass when another one counts for the next
+  __shared__ alignas(16) uint32_t s_hist[kFromMask ? 1 : 2][kFromMask ? 4 : kBins];
+  __shared__ uint32_t s_coarse[2][kWarps], s_pick[3], s_below[kWarps], s_at[kWarps];
   kvs_pdl_launch_dependents();
   cg::cluster_group cluster = cg::this_cluster();
-  const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int ctas = kCluster ? (int)cluster.num_blocks() : 1, rank = kCluster ? (int)cluster.block_rank() : 0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < 2) s_total[tid] = 0;
   if (!kFromMask)
-    for (int i = tid; i < 3 * kBins; i += kThreads) (&s_hist[0][0])[i] = 0;
+    for (int i = tid; i < 2 * kBins; i += kThreads) (&s_hist[0][0])[i] = 0;
   kvs_pdl_wait();
   {
     const uint32_t cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, all = gridDim.x * gridDim.y * gridDim.z;
@@ -135,105 +141,157 @@ select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
   if (n <= 0) return;                                      // (the whole cluster)
   const int unit = sr.b * a.Hkv + blockIdx.y;
   const int P = sr.P;
-  // this CTA's compaction tiles and pairs
+  // this CTA's compaction tiles, and this warp's: `steps` of them, one pair of each to a lane
   const int ntiles = max(0, n - tab.off + KVS_CTILE - 1) / KVS_CTILE;
   const int per_cta = (ntiles + ctas - 1) / ctas;
   const int t0 = min(ntiles, rank * per_cta), t1 = min(ntiles, t0 + per_cta);
-  const int steps = (t1 - t0 + kWarps - 1) / kWarps;       // of 32 tiles = 1024 pairs
+  const int steps = (t1 - t0 + kWarps - 1) / kWarps;
+  const int tile0 = t0 + warp * steps;
   const int p_end = min(P, 32 * t1);
-  const int p_first = 32 * t0 + tid;
+  const int p_first = 32 * tile0 + lane;
   uint8_t* mask = a.mask + (size_t)unit * a.pair_stride;
   const uint32_t* score = reinterpret_cast<const uint32_t*>(sa.score) + (size_t)unit * a.pair_stride;
 
-  if (!kFromMask) {
+  if (kMode == kFused) {
 #pragma unroll 1
-    for (int u = 0, p = p_first; p < p_end; ++u, p += kThreads) {
-      const uint32_t x = kMode == kFused ? __float_as_uint(finalize_pair(sa, unit, tab.off, p)) : score[p];
-      if (steps <= kKeep) s_key[u * kThreads + tid] = x;
+    for (int u = 0, p = p_first; u < steps && p < p_end; ++u, p += 32) {
+      const float x = finish_pair(sa, unit, tab.off, p, pair_sums(sa, unit, p));
+      if (steps <= kKeep) s_key[u * kThreads + tid] = __float_as_uint(x);
     }
+  } else if (kMode == kFusedFew) {
+#pragma unroll 1
+    for (int u = 0, p = p_first; u < steps && p < p_end; u += 2, p += 64) {
+      const bool two = u + 1 < steps && p + 32 < p_end;
+      const PairSums x = pair_sums(sa, unit, p), y = pair_sums(sa, unit, two ? p + 32 : p);
+      const float sx = finish_pair(sa, unit, tab.off, p, x);
+      const float sy = two ? finish_pair(sa, unit, tab.off, p + 32, y) : 0.f;
+      if (steps <= kKeep) {
+        s_key[u * kThreads + tid] = __float_as_uint(sx);
+        if (two) s_key[(u + 1) * kThreads + tid] = __float_as_uint(sy);
+      }
+    }
+  } else if (kMode == kScores && steps <= kKeep) {
+#pragma unroll 4
+    for (int u = 0; u < steps; ++u) s_key[u * kThreads + tid] = p_first + 32 * u < p_end ? score[p_first + 32 * u] : 0u;
   }
-  // the keys of this CTA (every thread reads only what it has written itself)
-  const uint32_t* keys = steps <= kKeep ? s_key + tid : score + p_first;
-  auto key_of = [&](int u, int p) -> uint32_t {
+  // the key of a step (every thread reads only what it has written itself)
+  auto key_of = [&](int u) -> uint32_t {
+    const int p = p_first + 32 * u;
     if (p >= p_end) return 0u;
-    return kFromMask ? (uint32_t)mask[p] : keys[(size_t)u * kThreads];
+    return kFromMask ? (uint32_t)mask[p] : steps <= kKeep ? s_key[u * kThreads + tid] : score[p];
   };
-  auto cluster_barrier = [&] { if (ctas > 1) cluster.sync(); else __syncthreads(); };
+  auto cluster_barrier = [&] { if (kCluster) cluster.sync(); else __syncthreads(); };
+  auto of_rank = [&](auto* x, int r) { return kCluster ? *cluster.map_shared_rank(x, r) : *x; };
 
-  // ---- cutoff: bit pattern of the R-th smallest score; k of its ties are taken
+  // ---- cutoff: bit pattern of the R-th smallest score; k of its ties are taken.  Every pass cuts the interval
+  //      [lo, lo + width) that holds it into up to 4096 bins, until the interval is one pattern or is taken as a whole.
   uint32_t cutoff = 0, k = kFromMask ? 0u : (uint32_t)sr.R;
-  __syncthreads();
   if (!kFromMask) {
+    uint32_t lo = 0, width = 0x80000000u;
+    __syncthreads();
 #pragma unroll 1
-    for (int pass = 0; pass < 3; ++pass) {
-      const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
-      const int bits = pass == 2 ? 10 : 11;
-#pragma unroll 1
-      for (int u = 0, p = p_first; p < p_end; ++u, p += kThreads) {
-        const uint32_t v = key_of(u, p);
-        if (pass == 0 || ((v ^ cutoff) >> (shift + bits)) == 0) atomicAdd(&s_hist[pass][(v >> shift) & ((1u << bits) - 1u)], 1u);
+    for (int pass = 0;; ++pass) {
+      uint32_t* hist = s_hist[pass & 1];
+      if (pass >= 2) {
+        for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
+        __syncthreads();
       }
-      cluster_barrier();
-      uint2 h = make_uint2(0, 0);
-#pragma unroll 1
-      for (int r = 0; r < ctas; ++r) {
-        const uint2 x = *cluster.map_shared_rank(reinterpret_cast<uint2*>(&s_hist[pass][2 * tid]), r);
-        h.x += x.x; h.y += x.y;
+      const int shift = max(0, 32 - __clz((int)(width - 1)) - kBinBits);
+#pragma unroll 2
+      for (int u = 0; u < steps; ++u) {
+        const uint32_t v = key_of(u);
+        if (p_first + 32 * u < p_end && v - lo < width) atomicAdd(&hist[pass == 0 ? (uint32_t)first_digit(v) : (v - lo) >> shift], 1u);
       }
-      const uint32_t before = block_scan(h.x + h.y, s_warp[pass & 1]);
-      if (before < k && k <= before + h.x) { s_digit = 2 * tid; s_k = k - before; }
-      if (before + h.x < k && k <= before + h.x + h.y) { s_digit = 2 * tid + 1; s_k = k - before - h.x; }
       __syncthreads();
-      cutoff |= s_digit << shift;
-      k = s_k;
+      // The 128 bins that hold the k-th key are found from the sums of 128, its bin from their counts: little is read of the
+      // other CTAs' shared memory (all counts of three CTAs: 1400 cycles, of seven 2700), and one warp does it (all of
+      // them, redundantly, took 1000 cycles a pass more: with 1024 threads an instruction is eight issue slots).
+      uint32_t* coarse = s_coarse[pass & 1];
+      const uint4 mine = reinterpret_cast<const uint4*>(s_hist[pass & 1])[tid];
+      const uint32_t of_mine = __reduce_add_sync(0xffffffffu, mine.x + mine.y + mine.z + mine.w);
+      if (lane == 0) coarse[warp] = of_mine;
+      cluster_barrier();
+      if (warp == 0) {
+        uint32_t sum = 0;
+#pragma unroll 4
+        for (int r = 0; r < ctas; ++r) sum += of_rank(&coarse[lane], r);
+        const uint32_t upto = warp_scan(sum);
+        const int hit = (__ffs((int)__ballot_sync(0xffffffffu, upto >= k)) - 1) & 31;
+        uint32_t before = __shfl_sync(0xffffffffu, upto - sum, hit);
+        uint32_t h[4] = {0, 0, 0, 0};
+#pragma unroll 4
+        for (int r = 0; r < ctas; ++r) {
+          const uint4 x = of_rank(reinterpret_cast<uint4*>(s_hist[pass & 1]) + 32 * hit + lane, r);
+          h[0] += x.x; h[1] += x.y; h[2] += x.z; h[3] += x.w;
+        }
+        const uint32_t own = (h[0] + h[1]) + (h[2] + h[3]);
+        before += warp_scan(own) - own;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (before < k && k <= before + h[i]) { s_pick[0] = 4 * (32 * hit + lane) + i; s_pick[1] = k - before; s_pick[2] = h[i]; }
+          before += h[i];
+        }
+      }
+      __syncthreads();
+      const uint32_t bin = s_pick[0], in_bin = s_pick[2];
+      k = s_pick[1];
+      if (pass == 0) {
+        lo = bin == 0 ? 0u : (bin + kFirstBin) << 17;
+        width = (bin == kBins - 1 ? 0x80000000u : (bin + kFirstBin + 1) << 17) - lo;
+      } else {
+        width = min(1u << shift, width - (bin << shift));
+        lo += bin << shift;
+      }
+      if (in_bin == k) { cutoff = lo + width; k = 0; break; }
+      if (width == 1) { cutoff = lo; break; }
     }
   }
-  // ---- pairs below the cutoff and at it, in this CTA and in the CTAs before it
-  uint32_t below = 0, at = 0;
-#pragma unroll 1
-  for (int u = 0, p = p_first; p < p_end; ++u, p += kThreads) {
-    const uint32_t v = key_of(u, p);
-    below += (kFromMask ? v != 0 : v < cutoff) ? 1u : 0u;
-    at += (!kFromMask && v == cutoff) ? 1u : 0u;
+  // ---- pairs below the cutoff and at it, in this warp ...
+  uint32_t below = 0, at = 0, kept = 0;
+#pragma unroll 4
+  for (int u = 0; u < steps; ++u) {
+    const uint32_t v = key_of(u);
+    const bool in = p_first + 32 * u < p_end;
+    const uint32_t c = __popc(__ballot_sync(0xffffffffu, in && (kFromMask ? v != 0 : v < cutoff)));
+    below += c;
+    if (kFromMask && lane == (u & 31)) kept = c;
+    if (!kFromMask && k != 0) at += __popc(__ballot_sync(0xffffffffu, in && v == cutoff));
+  }
+  if (lane == 0) { s_below[warp] = below; s_at[warp] = at; }
+  cluster_barrier();
+  // ... and in front of it
+  below = lane < warp ? s_below[lane] : 0u;
+  at = lane < warp ? s_at[lane] : 0u;
+  for (int r = 0; r < rank; ++r) {
+    below += of_rank(&s_below[lane], r);
+    if (!kFromMask) at += of_rank(&s_at[lane], r);
   }
   below = __reduce_add_sync(0xffffffffu, below);
-  at = __reduce_add_sync(0xffffffffu, at);
-  if (lane == 0 && below) atomicAdd(&s_total[0], below);
-  if (lane == 0 && at) atomicAdd(&s_total[1], at);
-  cluster_barrier();
-  below = at = 0;
-  for (int r = 0; r < rank; ++r) {
-    below += *cluster.map_shared_rank(&s_total[0], r);
-    at += *cluster.map_shared_rank(&s_total[1], r);
-  }
-  // ---- mask and counts in front of every tile, 32 tiles (one per warp) a step.  The first k ties are taken.
+  if (!kFromMask) at = __reduce_add_sync(0xffffffffu, at);
+  // ---- mask and counts in front of every tile.  The first k ties are taken.
   int32_t* tp = a.tile_prefix + (size_t)unit * a.tile_stride;
-#pragma unroll 1
-  for (int u = 0; u < steps; ++u) {
-    const int p = p_first + u * kThreads;
-    const uint32_t v = key_of(u, p);
-    const bool lt = p < p_end && (kFromMask ? v != 0 : v < cutoff);
-    const bool eq = !kFromMask && p < p_end && v == cutoff;
-    const uint32_t bl = __ballot_sync(0xffffffffu, lt), be = __ballot_sync(0xffffffffu, eq);
-    uint32_t* cnt = s_cnt[u & 1];
-    if (lane == 0) cnt[warp] = __popc(bl) | (__popc(be) << 16);
-    __syncthreads();
-    uint32_t c = cnt[lane];                                // (32 warps, 32 lanes; the sums stay below 2^16)
-    const uint32_t own = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, c, o);
-      if (lane >= o) c += t;
+  if (kFromMask && steps <= 32) {
+    const uint32_t upto = warp_scan(kept);
+    if (lane < steps && tile0 + lane < t1) tp[tile0 + lane] = (int32_t)(below + upto - kept);
+  } else {
+#pragma unroll 2
+    for (int u = 0; u < steps; ++u) {
+      const int p = p_first + 32 * u;
+      const uint32_t v = key_of(u);
+      const bool in = p < p_end;
+      const bool lt = in && (kFromMask ? v != 0 : v < cutoff);
+      bool taken = lt;
+      if (lane == 0 && tile0 + u < t1) tp[tile0 + u] = (int32_t)(below + min(k, at));
+      below += __popc(__ballot_sync(0xffffffffu, lt));
+      if (!kFromMask && k != 0) {                          // (mostly the interval was taken as a whole, and there are no ties)
+        const uint32_t be = __ballot_sync(0xffffffffu, in && v == cutoff);
+        taken = lt || (in && v == cutoff && at + __popc(be & ((1u << lane) - 1u)) < k);
+        at += __popc(be);
+      }
+      if (!kFromMask && in) mask[p] = taken ? 1 : 0;
     }
-    const uint32_t total = __shfl_sync(0xffffffffu, c, 31), ex = __shfl_sync(0xffffffffu, c - own, warp);
-    const uint32_t tie_before = at + (ex >> 16);
-    if (!kFromMask && p < p_end) mask[p] = (lt || (eq && tie_before + __popc(be & ((1u << lane) - 1u)) < k)) ? 1 : 0;
-    const int tile = t0 + u * kWarps + warp;
-    if (lane == 0 && tile < t1) tp[tile] = (int32_t)(below + (ex & 0xffffu) + min(k, tie_before));
-    below += total & 0xffffu;
-    at += total >> 16;
   }
-  if (ctas > 1) cluster.sync();                            // no CTA leaves while its shared memory is read
+  if (kCluster) cluster.sync();                            // no CTA leaves while its shared memory is read
 }
 
 int most_pairs(const RoundTable& t) {
@@ -242,30 +300,30 @@ int most_pairs(const RoundTable& t) {
   return pmax;
 }
 
-// CTAs per unit: one for every 4096 pairs while they all fit the GPU (two per SM).  A cluster's barriers cost about
-// 1.5 us each: 8 units of 16336 pairs 17 us with four CTAs, 28 with eight; 256 units of 16336 pairs 32 us with
-// one, 85 with several waves of clusters of four.  The counts of a given mask have one such barrier and take a CTA for
+// CTAs per unit: one for every 4096 pairs while they all fit the GPU, one per SM (6144 and 8192: a call of the statistics of 8
+// units of 16336 pairs 132.0 and 134.0 us, with 4096 132.3; nine rounds of 8 units from 16 k pairs on 148, 152 and
+// 144 us in the selections; 256 units of 16336 pairs 32 us with one, 85 with several waves of clusters of
+// four).  The counts of a given mask need few registers: two per SM, a CTA for
 // 3072 pairs: a compaction of 4 units of 7200 pairs 22.1 us, with half as many 24.0; of 8 units of 16336 63.2 and 64.4;
 // but of 32 units of 2180 74.4 with two CTAs and 70.8 with one.
-int cluster_of(const RoundTable& t, int Hkv, int pairs_per_cta) {
+int cluster_of(const RoundTable& t, int Hkv, int pairs_per_cta, int fit) {
   const int pmax = most_pairs(t);
   int c = 1;
-  while (c < kMaxCluster && c * pairs_per_cta < pmax && (long long)c * 2 * Hkv * t.nseq <= 2 * 148) c *= 2;
+  while (c < kMaxCluster && c * pairs_per_cta < pmax && (long long)c * 2 * Hkv * t.nseq <= fit) c *= 2;
   return c;
 }
 
 constexpr int kSpreadSmem = 118 * 1024;
 static_assert(kSpreadSmem <= kKeep * kThreads * (int)sizeof(uint32_t), "the kernel is configured for its keys");
-template <int kMode>
-cudaError_t launch_select(const StatsTcArgs& sa, const SelectArgs& a, const RoundTable& t, cudaStream_t st) {
+template <int kMode, bool kCluster>
+cudaError_t launch_select(const StatsTcArgs& sa, const SelectArgs& a, const RoundTable& t, int c, cudaStream_t st) {
   static KvsPerDeviceOnce configured;
   cudaError_t e = configured.run([] {
-    return cudaFuncSetAttribute(select_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(select_kernel<kMode, kCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 kKeep * kThreads * (int)sizeof(uint32_t));
   });
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  const int c = cluster_of(t, a.Hkv, kMode == kMask ? kMaskPairsPerCta : kPairsPerCta);
   cfg.gridDim = dim3((unsigned)c, (unsigned)a.Hkv, (unsigned)t.nseq);
   cfg.blockDim = dim3(kThreads);
   if (kMode != kMask) {
@@ -289,8 +347,8 @@ cudaError_t launch_select(const StatsTcArgs& sa, const SelectArgs& a, const Roun
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, select_kernel<kMode>, sa, a, t);
+  cfg.numAttrs = kCluster ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, select_kernel<kMode, kCluster>, sa, a, t);
 }
 
 // Whether the selection kernel adds the partials itself: where they are few (at most two query blocks), and
@@ -312,13 +370,17 @@ cudaError_t kvs_launch_finalize_select(const StatsTcArgs& sa, const SelectArgs& 
   *kernels = 1;
   const int pmax = most_pairs(t);
   if (pmax <= 0) return cudaSuccess;
-  if (fused_finalize(sa, a, a.Hkv * t.nseq, pmax)) return launch_select<kFused>(sa, a, t, st);
+  const int units = a.Hkv * t.nseq;
+  if (fused_finalize(sa, a, units, pmax))                  // (at most 4096 pairs a unit: one CTA)
+    return units <= 148 ? launch_select<kFusedFew, false>(sa, a, t, 1, st) : launch_select<kFused, false>(sa, a, t, 1, st);
   cudaError_t e = kvs_launch_chained(finalize_kernel, dim3((pmax + 255) / 256, a.Hkv, t.nseq), dim3(256), 0, st, sa, t);
   if (e != cudaSuccess || !a.select) return e;
   *kernels = 2;
-  return launch_select<kScores>(sa, a, t, st);
+  const int c = cluster_of(t, a.Hkv, kPairsPerCta, 148);
+  return c > 1 ? launch_select<kScores, true>(sa, a, t, c, st) : launch_select<kScores, false>(sa, a, t, c, st);
 }
 
 cudaError_t kvs_launch_mask_prefix(const SelectArgs& a, const RoundTable& t, cudaStream_t st) {
-  return launch_select<kMask>(StatsTcArgs{}, a, t, st);
+  const int c = cluster_of(t, a.Hkv, kMaskPairsPerCta, 2 * 148);
+  return c > 1 ? launch_select<kMask, true>(StatsTcArgs{}, a, t, c, st) : launch_select<kMask, false>(StatsTcArgs{}, a, t, c, st);
 }

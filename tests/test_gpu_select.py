@@ -49,3 +49,41 @@ def test_mask_is_the_smallest_scores(hkv, n, period, first_round):
     slots = torch.arange(n, dtype=torch.int32, device="cuda")
     assert torch.equal(index[0], slots - before.cumsum(1, dtype=torch.int32))
     assert status.item() == 0
+
+
+# KV heads, slots, period of the keys, factor of the queries.  Large queries leave most slots with masses far below 2^-56
+# or of 0; a period of 2 gives all pairs one score, fewer and more of them than are ranked directly; the last cases
+# walk more than 32 steps a CTA.
+@pytest.mark.parametrize("hkv,n,period,factor", [
+    (2, 300, 2, 1), (2, 2200, 2, 1), (3, 2200, 0, 30), (8, 2084, 0, 4), (3, 8400, 16, 1), (8, 40001, 0, 30), (8, 40001, 2, 1),
+    (2, 140000, 64, 1), (160, 66200, 0, 30), (160, 66200, 2, 1)])
+def test_a_pass_takes_the_smallest_scores(hkv, n, period, factor):
+    import torch
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + period + factor)
+    K, V = (torch.empty(1, hkv, n, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    for x in (K, V):
+        rows = torch.randn(hkv, period or n, 128, generator=g, device="cuda").to(torch.bfloat16)
+        x[0] = rows.repeat(1, n // (period or n) + 1, 1)[:, :n]
+    counts = torch.ones(1, hkv, n, dtype=torch.int32, device="cuda")
+    q = (factor * torch.randn(1, hkv, 4, 128, generator=g, device="cuda")).to(torch.bfloat16)
+    p = kb.make_params(K, V, hkv, 4, causal=False)
+    ws = torch.empty(kb.kvs_workspace_size(p, n, 0), dtype=torch.uint8, device="cuda")
+    score, w = (torch.zeros(1, hkv, n // 2, device="cuda") for _ in range(2))
+    mask = torch.zeros(1, hkv, n // 2, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    _, off, P, R = kb.kvs_round_plan(p, n, n - n // 5)[0]
+    kb.kvs_window_stats(p, K, V, counts, q, [n], [n - n // 5], ws, score=score, w=w, mask=mask, status_dev=status)
+    want = torch.zeros_like(mask)
+    want[0].scatter_(1, torch.sort(score[0, :, :P], dim=-1, stable=True).indices[:, :R], 1)
+    assert torch.equal(mask, want)
+    # one round of a pass makes the same decision and counts its tiles alike
+    K2, V2, counts2 = K.clone(), V.clone(), counts.clone()
+    kb.kvs_compact(p, K2, V2, counts2, mask, w, [n], [R], ws, status_dev=status)
+    assert kb.kvs_merge_layer(p, K, V, counts, q, [n], [n - R], ws, status_dev=status) == [n - R]
+    for x, y in ((K, K2), (V, V2), (counts, counts2)):
+        assert torch.equal(x[:, :, :n - R].view(torch.int16 if x is not counts else torch.int32),
+                           y[:, :, :n - R].view(torch.int16 if x is not counts else torch.int32))
+    assert status.item() == 0
