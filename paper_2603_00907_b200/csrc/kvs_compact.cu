@@ -12,9 +12,9 @@
 // publish "tile loaded", wait (bounded) until every earlier tile whose source rows they are
 // about to overwrite has loaded too, and store the surviving rows at
 //   new slot = old slot - (merged pairs before it).
-// Tickets make the wait safe: a tile only waits for tiles with smaller tickets, whose owners
-// are running and handle their own tiles in ticket order, so the smallest unpublished tile
-// never waits.
+// Tickets make the wait safe: a tile only waits for tiles of its unit with smaller tickets, which were taken before its own.
+// Every CTA handles its tiles, of one unit or of several, in the order in which it took them, so
+// that of all tiles not yet published the one taken first never waits.
 #include "kvs_internal.h"
 #include "kvs_sm100.cuh"
 
@@ -51,7 +51,7 @@ struct TileMeta {
   int32_t tile;                  // -1: no more tiles
   int32_t E0;                    // merged pairs before the tile
   uint32_t selbits;              // bit i: pair i of the tile is merged
-  int32_t pad;
+  int32_t seq, h;                // the tile's unit: entry of the launch table, KV head
   float w[32];
   int32_t cnt[KVS_CTILE];
 };
@@ -79,9 +79,10 @@ __device__ __forceinline__ bool consumer_wait(uint64_t* b0, uint64_t* b1, uint32
 // Persistent CTAs per unit: the 2 x 148 CTAs that fit the GPU are shared out in proportion to the
 // units' tile counts (a ragged batch would otherwise wait for its longest sequence, which would
 // have no more CTAs than the shortest), at least one and at most one per tile.
-__host__ __device__ inline int ctas_of_unit(int unit_tiles, long long all_tiles) {
+__host__ __device__ inline int ctas_of_unit(int unit_tiles, long long all_tiles, bool share) {
   if (unit_tiles <= 0) return 0;
-  long long c = all_tiles > 0 ? (2LL * 148 * unit_tiles) / all_tiles : 1;   // rounded down: all of them are resident at once
+  // rounded down: all of them are resident at once; rounded up where a CTA that has no tile left goes on with other units
+  long long c = all_tiles > 0 ? (2LL * 148 * unit_tiles + (share ? all_tiles - 1 : 0)) / all_tiles : 1;
   if (c < 1) c = 1;
   if (c > unit_tiles) c = unit_tiles;
   return (int)c;
@@ -113,11 +114,10 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
   }
   long long all_tiles = 0;
   for (int i = 0; i < tab.nseq; ++i) all_tiles += tiles_of(tab.s[i].n, off);
-  const int unit_ctas = ctas_of_unit(ntiles, all_tiles * a.c.Hkv);
+  const bool share = a.share != 0;
+  const int unit_ctas = ctas_of_unit(ntiles, all_tiles * a.c.Hkv, share);
   if ((int)blockIdx.x >= unit_ctas) return;                // this unit's share of the CTAs is smaller
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int P = sr.P;
-
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&sh->full[s], 1);
@@ -132,16 +132,12 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
   __syncthreads();
   volatile int* abort_flag = &sh->abort_flag;
 
-  __nv_bfloat16* Kb = a.c.K + sr.b * a.c.ksb + h * a.c.ksh;
-  __nv_bfloat16* Vb = a.c.V + sr.b * a.c.vsb + h * a.c.vsh;
-  int32_t* Cb = a.c.counts + (size_t)unit * a.c.n_max;
-
   if (warp == kConsumers / 32) {
     // ================================================================ producer warp
-    const uint8_t* mask = a.mask + (size_t)unit * a.pair_stride;
-    const float* wl = a.w + (size_t)unit * a.pair_stride;
+    // the unit whose tiles it takes: its own, then (share) the one that has the most left
+    int cs = seq, ch = h, cu = unit, cn = n, cP = sr.P, ct = ntiles;
     uint32_t next_ticket = 0;
-    if (lane == 0) next_ticket = atomicAdd(&a.tickets[unit], 1u);
+    bool ahead = false;              // next_ticket is taken already
     int issued = 0;                  // tiles whose copies were requested
     for (int k = 0;; ++k) {
       const int s = k % kStages;
@@ -155,15 +151,39 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
           for (int kk = max(0, issued - kStages); kk < issued; ++kk) mbar_drain(&sh->full[kk % kStages], (uint32_t)(kk / kStages) & 1u);
         break;
       }
-      const int t = (int)__shfl_sync(0xffffffffu, next_ticket, 0);
+      int t;
+      for (;;) {
+        if (!ahead && lane == 0) next_ticket = atomicAdd(&a.tickets[cu], 1u);
+        ahead = false;
+        t = (int)__shfl_sync(0xffffffffu, next_ticket, 0);
+        if (t < ct || !share) break;
+        // (a count that is out of date costs a look more, no tile: the ticket decides)
+        int left = 0, at = 0;
+        for (int i = lane; i < tab.nseq * a.c.Hkv; i += 32) {
+          const int q = i / a.c.Hkv, nt = tiles_of(tab.s[q].n, off);
+          const int l = nt - (int)*(volatile const uint32_t*)&a.tickets[tab.s[q].b * a.c.Hkv + (i - q * a.c.Hkv)];
+          if (l > left) { left = l; at = i; }
+        }
+        const int most = __reduce_max_sync(0xffffffffu, left);
+        if (most <= 0) break;
+        at = __shfl_sync(0xffffffffu, at, __ffs((int)__ballot_sync(0xffffffffu, left == most)) - 1);
+        cs = at / a.c.Hkv; ch = at - cs * a.c.Hkv;
+        cu = tab.s[cs].b * a.c.Hkv + ch; cn = tab.s[cs].n; cP = tab.s[cs].P; ct = tiles_of(cn, off);
+      }
       TileMeta* m = &sh->meta[s];
-      if (t >= ntiles) {
+      if (t >= ct) {
         if (lane == 0) { m->tile = -1; mbar_arrive(&sh->meta_full[s]); }
         break;
       }
-      if (lane == 0) next_ticket = atomicAdd(&a.tickets[unit], 1u);   // its latency hides behind this tile
+      const uint8_t* mask = a.mask + (size_t)cu * a.pair_stride;
+      const float* wl = a.w + (size_t)cu * a.pair_stride;
+      const __nv_bfloat16* Kb = a.c.K + tab.s[cs].b * a.c.ksb + ch * a.c.ksh;
+      const __nv_bfloat16* Vb = a.c.V + tab.s[cs].b * a.c.vsb + ch * a.c.vsh;
+      const int32_t* Cb = a.c.counts + (size_t)cu * a.c.n_max;
+      if (lane == 0) next_ticket = atomicAdd(&a.tickets[cu], 1u);   // its latency hides behind this tile
+      ahead = true;
       const int j0 = off + KVS_CTILE * t;
-      const int rows = min(KVS_CTILE, n - j0);
+      const int rows = min(KVS_CTILE, cn - j0);
       uint8_t* sk = smem + s * kStageBytes;
       uint8_t* sv = sk + kOperandBytes;
       if (lane == 0) mbar_expect_tx(&sh->full[s], (uint32_t)rows * 2u * kRowBytes);
@@ -180,7 +200,7 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
       }
       // the tile's decision
       const int pp = 32 * t + lane;
-      const bool in_range = pp < P;
+      const bool in_range = pp < cP;
       const bool sel = in_range && mask[pp] != 0;
       m->w[lane] = in_range ? wl[pp] : 0.5f;
       m->cnt[lane] = (lane < rows) ? Cb[j0 + lane] : 0;
@@ -188,7 +208,9 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
       const uint32_t bits = __ballot_sync(0xffffffffu, sel);
       if (lane == 0) {
         m->selbits = bits;
-        m->E0 = a.tile_prefix[(size_t)unit * a.tile_stride + t];
+        m->E0 = a.tile_prefix[(size_t)cu * a.tile_stride + t];
+        m->seq = cs;
+        m->h = ch;
         m->tile = t;
       }
       __syncwarp();
@@ -207,6 +229,11 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
       const int t = m->tile;
       if (t < 0) break;
       if (!consumer_wait(&sh->full[s], nullptr, ph, abort_flag, fail, lane)) break;
+      const int ts = m->seq, th = m->h;                   // (the tile's unit)
+      const int n = tab.s[ts].n, unit = tab.s[ts].b * a.c.Hkv + th;
+      __nv_bfloat16* Kb = a.c.K + tab.s[ts].b * a.c.ksb + th * a.c.ksh;
+      __nv_bfloat16* Vb = a.c.V + tab.s[ts].b * a.c.vsb + th * a.c.vsh;
+      int32_t* Cb = a.c.counts + (size_t)unit * a.c.n_max;
       const int j0 = off + KVS_CTILE * t;
       const int jl = j0 + 2 * i, jr = jl + 1;
       const bool okl = jl < n, okr = jr < n;
@@ -244,7 +271,7 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
       // (test hook: with bit 2 of debug_stall the flag stays unset, so that the waits on it run out)
       if (tid == 0 && !(a.debug_stall & 4u)) st_release_u32(&a.flags[(size_t)unit * a.tile_stride + t], a.epoch);
       const int moved = E0 + __popc(selbits);
-      if (E0 > 0 && unit_ctas > 1) {
+      if (E0 > 0 && (share || unit_ctas > 1)) {
         // This tile's rows land in [j0 - E0, j0 - E0 + 64): those are source rows of at most two
         // earlier tiles (and of this tile itself), which must have been read before they are
         // overwritten; a CTA that owns the whole unit has read them itself, in order
@@ -313,11 +340,24 @@ cudaError_t kvs_launch_compact(const CompactArgs& a, const RoundTable& t, cudaSt
   // the grid is as wide as the longest unit's share, the CTAs beyond a unit's share leave at once
   long long all_tiles = 0;
   for (int i = 0; i < t.nseq; ++i) all_tiles += tiles_of(t.s[i].n, t.off);
+  all_tiles *= a.c.Hkv;
+  // Where the rounding of the shares, or one CTA to each of many short units, leaves a unit with a quarter more tiles a CTA than
+  // the average, CTAs that are done go on with the unit that has most left (64 units of 64 to 1024 tiles, eight
+  // rounds: 1430 -> 1262 us).  Such units always need the flags, so not below: 256 equal units on 296 CTAs, a sixth above the
+  // average, 119 us a round when each CTA keeps to its unit, 159 with the others' help.
+  CompactArgs args = a;
   int per_unit = 1;
-  for (int i = 0; i < t.nseq; ++i) {
-    const int c = ctas_of_unit(tiles_of(t.s[i].n, t.off), all_tiles * a.c.Hkv);
-    if (c > per_unit) per_unit = c;
+  for (int share = 0; share < 2; ++share) {
+    double worst = 0.;                                     // tiles of the CTA that has most of them
+    per_unit = 1;
+    for (int i = 0; i < t.nseq; ++i) {
+      const int nt = tiles_of(t.s[i].n, t.off), c = ctas_of_unit(nt, all_tiles, share != 0);
+      if (c > per_unit) per_unit = c;
+      if (c > 0 && (double)nt / c > worst) worst = (double)nt / c;
+    }
+    args.share = share;
+    if (share == 0 && !(worst >= 4. && worst * (2 * 148) > 1.25 * (double)all_tiles)) break;
   }
   dim3 grid(per_unit, a.c.Hkv, t.nseq);
-  return kvs_launch_chained(merge_compact_kernel, grid, dim3(kThreads), kSmemBytes, st, a, t);
+  return kvs_launch_chained(merge_compact_kernel, grid, dim3(kThreads), kSmemBytes, st, args, t);
 }

@@ -138,6 +138,7 @@ struct CompactArgs {
   int32_t* status_dev;
   uint32_t wait_us;        // time limit of one device-side wait, microseconds
   uint32_t debug_stall;    // test hook: bit 2 = "tile loaded" flags are not published
+  int32_t share;           // set by the launcher: a CTA whose unit has no tile left takes tiles of other units
 };
 
 // ----------------------------------------------------------------------------- launchers
