@@ -221,6 +221,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     misc->wait_us = (int)a.wait_us;
     mbar_fence_init();
   }
+  if (warp == 0 && elect_one()) { prefetch_tmap(&tmK); prefetch_tmap(&tmV); prefetch_tmap(&tmQ); }
   if (warp == 1) tmem_alloc(&misc->tmem_base, 512);
   tc_fence_before();
   __syncthreads();
@@ -246,7 +247,6 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     // queued before the P V products of tile t), so the thread sleeps on one barrier at a time:
     // K(0), K(1), K(2), V(0), K(3), V(1), ...; every tile is requested into L2 a few tiles ahead
     if (elect_one()) {
-      prefetch_tmap(&tmK); prefetch_tmap(&tmV); prefetch_tmap(&tmQ);
       mbar_expect_tx(&misc->qfull, kOperand);
       for (int hf = 0; hf < 2; ++hf)
         tma_load_3d(smem + kSmemQ + hf * kHalf, &tmQ, &misc->qfull, hf * 64, qblk * 128, unit);
@@ -599,24 +599,38 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
       softmax_barrier();
       if (walk == 0 && my_tiles > 1 && *(volatile int*)&misc->again) n_walks = 3;   // (the same for all softmax threads)
     }
-    // ---- the partial of this key range: the four parts of a row's sum are added, and each thread writes 32
-    //      channels of the row of O
-    const size_t pidx = ((size_t)unit * a.splits + split) * a.M + m;
-    if (alive && warp_wait(&misc->pvdone[gi_last % kSBufs], (gi_last / kSBufs) & 1, abort_flag, lane)) {
-      tc_fence_after();
-      if (part == 0 && m < a.M) {
-        const float sum = (misc->part_sum[0][row] + misc->part_sum[1][row]) + (misc->part_sum[2][row] + misc->part_sum[3][row]);
-        a.part_ml[pidx] = make_float2(sum == 0.f ? -INFINITY : m_stab, sum);   // (a NaN sum is not an empty range)
-      }
-      float ov[32];
-      tmem_ld32(tmem + lane_addr + kColO + part * 32, ov);
-      tmem_ld_wait();
-      if (m < a.M) {
-        float4* po = reinterpret_cast<float4*>(a.part_o + pidx * KVS_D + part * 32);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) po[i] = make_float4(ov[4 * i], ov[4 * i + 1], ov[4 * i + 2], ov[4 * i + 3]);
-      }
+    // ---- the stabiliser and sum of this key range: the four parts of a row's sum are added
+    if (alive && warp_wait(&misc->pvdone[gi_last % kSBufs], (gi_last / kSBufs) & 1, abort_flag, lane) && part == 0 && m < a.M) {
+      const float sum = (misc->part_sum[0][row] + misc->part_sum[1][row]) + (misc->part_sum[2][row] + misc->part_sum[3][row]);
+      a.part_ml[((size_t)unit * a.splits + split) * a.M + m] =
+          make_float2(sum == 0.f ? -INFINITY : m_stab, sum);   // (a NaN sum is not an empty range)
     }
+  }
+
+  // ---- O.  A thread reads 32 channels of its row; written from there, the 16 bytes of 32 rows that a warp stores
+  // together lie in 32 lines: 5700 cycles for the 64 KB, a third of the time of a range of two tiles.  They go
+  // through the K ring (nobody reads it any more), pieces of 16 bytes exchanged by the row so that neither side has bank
+  // conflicts, and out row by row (nine rounds of 8 units from 32 K slots on, events: 304 -> 294 us, six launches of up to 32 tiles 92 ->
+  // 86.5, 256 units of 20 tiles 218 -> 212).
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp >= 2 && warp < 2 + kSoftmaxWarps && !*abort_flag) {   // (no wait is left that could set it: the same for all)
+    const int part = (warp - 2) >> 2, row = (warp & 3) * 32 + lane;
+    uint8_t* stage = smem + kSmemK;
+    float ov[32];
+    tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + kColO + part * 32, ov);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      *reinterpret_cast<float4*>(stage + row * (KVS_D * 4) + (((part * 8 + i) ^ (row & 7)) << 4)) =
+          make_float4(ov[4 * i], ov[4 * i + 1], ov[4 * i + 2], ov[4 * i + 3]);
+    softmax_barrier();
+    const int rows = min(kTile, a.M - qblk * kTile);
+    float4* po = reinterpret_cast<float4*>(a.part_o + (((size_t)unit * a.splits + split) * a.M + qblk * kTile) * KVS_D);
+#pragma unroll
+    for (int r = warp - 2; r < kTile; r += kSoftmaxWarps)
+      if (r < rows) po[r * (KVS_D / 4) + lane] = *reinterpret_cast<const float4*>(stage + r * (KVS_D * 4) + ((lane ^ (r & 7)) << 4));
   }
 
   tc_fence_before();
