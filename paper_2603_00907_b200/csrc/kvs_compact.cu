@@ -9,12 +9,17 @@
 // rows
 //   K*    = bf16( K_right + w (K_left - K_right) )        [Eq. kstar_final, weight form]
 //   Vsum* = bf16( Vsum_left + Vsum_right ),  c* = c_left + c_right   [v* = v_m + v_{m+1}]
-// publish "tile loaded", wait (bounded) until every earlier tile whose source rows they are
-// about to overwrite has loaded too, and store the surviving rows at
+// wait (bounded) until every earlier tile whose source rows they are about to overwrite has loaded, and store the surviving
+// rows at
 //   new slot = old slot - (merged pairs before it).
+// Where several CTAs handle tiles of a unit, a publisher warp says that a tile has loaded as soon as its copies have landed.
 // Tickets make the wait safe: a tile only waits for tiles of its unit with smaller tickets, which were taken before its own.
-// Every CTA handles its tiles, of one unit or of several, in the order in which it took them, so
+// Every CTA publishes and handles its tiles, of one unit or of several, in the order in which it took them, so
 // that of all tiles not yet published the one taken first never waits.
+// Bound by HBM in long units, by the chain of ticket, copies, flags and stores in short ones.  8 units of 2048 tiles
+// 185 -> 150 us a launch (events), nine rounds of 8 units from 512 tiles on 252 -> 186, five of 8 units from 64 on 68 -> 64,
+// against barriers of all consumers around every wait, flags set and looked at by consumers with release and acquire, and all
+// of the set-up behind the wait for the kernel in front.
 #include "kvs_internal.h"
 #include "kvs_sm100.cuh"
 
@@ -45,7 +50,8 @@ constexpr int kRowBytes = KVS_D * 2;                       // one bf16 row
 constexpr int kOperandBytes = KVS_CTILE * kRowBytes;       // 16 KB: the K (or Vsum) rows of a tile
 constexpr int kStageBytes = 2 * kOperandBytes;
 constexpr int kConsumers = 256;
-constexpr int kThreads = kConsumers + 32;                  // + the producer warp
+constexpr int kProducer = kConsumers / 32, kPublisher = kProducer + 1;   // warps
+constexpr int kThreads = kConsumers + 64;
 
 struct TileMeta {
   int32_t tile;                  // -1: no more tiles
@@ -58,22 +64,30 @@ struct TileMeta {
 struct Shared {
   uint64_t full[kStages], meta_full[kStages], empty[kStages];
   int abort_flag, wait_us;       // (adjacent: the bounded waits read both through one pointer)
-  int fail;
   TileMeta meta[kStages];
 };
 constexpr int kSmemBytes = kStages * kStageBytes + (int)sizeof(Shared);
 
-__device__ __forceinline__ void consumer_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// The "tile loaded" flags.  What they order is a read before a write: the copy of a tile's rows has completed (its mbarrier
+// says so) before the flag is set, and the flag has been seen before the rows are overwritten.  Nothing that was
+// written has to become visible with them, so they are relaxed: a release and an acquire at GPU scope took 1.5 and
+// 2 thousand cycles a tile (nine rounds of 8 units from 512 tiles on, events: 260 us, relaxed 230).
+__device__ __forceinline__ uint32_t ld_flag(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_flag(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 
-// Wait of all consumer warps on two mbarrier phases; either all 256 threads go on or all leave.
-__device__ __forceinline__ bool consumer_wait(uint64_t* b0, uint64_t* b1, uint32_t parity, volatile int* abort_flag,
-                                              volatile int* fail, int lane) {
-  if (lane == 0) {
-    if (!mbar_wait(b0, parity, abort_flag) || (b1 && !mbar_wait(b1, parity, abort_flag))) *fail = 1;
-  }
+// One lane waits, the warp follows.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int lane) {
+  int ok = 1;
+  if (lane == 0) ok = mbar_wait(bar, parity, abort_flag) ? 1 : 0;
+  ok = __shfl_sync(0xffffffffu, ok, 0);
   __syncwarp();
-  consumer_barrier();
-  return *fail == 0;
+  return ok != 0;
 }
 
 // Persistent CTAs per unit: the 2 x 148 CTAs that fit the GPU are shared out in proportion to the
@@ -94,16 +108,33 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
   extern __shared__ __align__(128) uint8_t smem[];
   Shared* sh = reinterpret_cast<Shared*>(smem + kStages * kStageBytes);
   kvs_pdl_launch_dependents();
-  kvs_pdl_wait();
-
   const int seq = blockIdx.z;
   const SeqRound sr = tab.s[seq];
   const int n = sr.n;
-  if (n <= 0) return;
   const int h = blockIdx.y;
   const int unit = sr.b * a.c.Hkv + h;
   const int off = tab.off;
   const int ntiles = tiles_of(n, off);
+  long long all_tiles = 0;
+  for (int i = 0; i < tab.nseq; ++i) all_tiles += tiles_of(tab.s[i].n, off);
+  const bool share = a.share != 0;
+  const int unit_ctas = ctas_of_unit(ntiles, all_tiles * a.c.Hkv, share);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool ordered = share || unit_ctas > 1;             // others handle tiles of the unit, too
+  if (tid == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&sh->full[s], 1);
+      mbar_init(&sh->meta_full[s], 1);
+      mbar_init(&sh->empty[s], kConsumers / 32 + (ordered ? 1 : 0));
+    }
+    sh->abort_flag = 0;
+    sh->wait_us = (int)a.wait_us;
+    mbar_fence_init();
+  }
+  __syncthreads();
+  // (everything above runs while the kernel before this one may still be draining)
+  kvs_pdl_wait();
+  if (n <= 0) return;
   if (ntiles == 0) {
     // a unit that ends inside the protected prefix has nothing to move; its slot map is the identity
     if (a.new_index && blockIdx.x == 0) {
@@ -112,27 +143,10 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
     }
     return;
   }
-  long long all_tiles = 0;
-  for (int i = 0; i < tab.nseq; ++i) all_tiles += tiles_of(tab.s[i].n, off);
-  const bool share = a.share != 0;
-  const int unit_ctas = ctas_of_unit(ntiles, all_tiles * a.c.Hkv, share);
   if ((int)blockIdx.x >= unit_ctas) return;                // this unit's share of the CTAs is smaller
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&sh->full[s], 1);
-      mbar_init(&sh->meta_full[s], 1);
-      mbar_init(&sh->empty[s], kConsumers / 32);
-    }
-    sh->abort_flag = 0;
-    sh->wait_us = (int)a.wait_us;
-    sh->fail = 0;
-    mbar_fence_init();
-  }
-  __syncthreads();
   volatile int* abort_flag = &sh->abort_flag;
 
-  if (warp == kConsumers / 32) {
+  if (warp == kProducer) {
     // ================================================================ producer warp
     // the unit whose tiles it takes: its own, then (share) the one that has the most left
     int cs = seq, ch = h, cu = unit, cn = n, cP = sr.P, ct = ntiles;
@@ -142,10 +156,7 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
     for (int k = 0;; ++k) {
       const int s = k % kStages;
       const uint32_t ph = (uint32_t)(k / kStages) & 1u;
-      int ok = 1;
-      if (lane == 0) ok = mbar_wait(&sh->empty[s], ph ^ 1u, abort_flag) ? 1 : 0;
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) {
+      if (!warp_wait(&sh->empty[s], ph ^ 1u, abort_flag, lane)) {
         // give the copies of the last stages a bounded time to land before the CTA leaves
         if (lane == 0)
           for (int kk = max(0, issued - kStages); kk < issued; ++kk) mbar_drain(&sh->full[kk % kStages], (uint32_t)(kk / kStages) & 1u);
@@ -198,17 +209,23 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
           bulk_load(sv + r * kRowBytes, Vb + (int64_t)(j0 + r) * a.c.vst, kRowBytes, &sh->full[s]);
         }
       }
-      // the tile's decision
+      // the tile's decision (all of it requested before the first of it is used)
       const int pp = 32 * t + lane;
-      const bool in_range = pp < cP;
-      const bool sel = in_range && mask[pp] != 0;
-      m->w[lane] = in_range ? wl[pp] : 0.5f;
-      m->cnt[lane] = (lane < rows) ? Cb[j0 + lane] : 0;
-      m->cnt[lane + 32] = (lane + 32 < rows) ? Cb[j0 + lane + 32] : 0;
-      const uint32_t bits = __ballot_sync(0xffffffffu, sel);
+      const int32_t E0 = a.tile_prefix[(size_t)cu * a.tile_stride + t];
+      const int32_t c0 = Cb[j0 + min(lane, rows - 1)], c1 = Cb[j0 + min(lane + 32, rows - 1)];   // (those past the end are not used)
+      uint8_t chosen = 0;
+      float weight = 0.5f;
+      if (32 * t < cP) {
+        chosen = mask[min(pp, cP - 1)];
+        weight = wl[min(pp, cP - 1)];
+      }
+      m->w[lane] = weight;
+      m->cnt[lane] = c0;
+      m->cnt[lane + 32] = c1;
+      const uint32_t bits = __ballot_sync(0xffffffffu, pp < cP && chosen != 0);
       if (lane == 0) {
         m->selbits = bits;
-        m->E0 = a.tile_prefix[(size_t)cu * a.tile_stride + t];
+        m->E0 = E0;
         m->seq = cs;
         m->h = ch;
         m->tile = t;
@@ -216,19 +233,37 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh->meta_full[s]);
     }
+  } else if (warp == kPublisher) {
+    // ================================================================ publisher
+    // (up to two tiles before the consumers get to them; a publisher that also waited for the other tiles' flags was late with
+    // its next tile: nine rounds of 8 units from 512 tiles on 220 us, so 187)
+    for (int k = 0; ordered; ++k) {
+      const int s = k % kStages;
+      const uint32_t ph = (uint32_t)(k / kStages) & 1u;
+      if (!warp_wait(&sh->meta_full[s], ph, abort_flag, lane)) break;
+      const TileMeta* m = &sh->meta[s];
+      if (m->tile < 0) break;
+      uint32_t* flag = a.flags + (size_t)(tab.s[m->seq].b * a.c.Hkv + m->h) * a.tile_stride + m->tile;
+      if (!warp_wait(&sh->full[s], ph, abort_flag, lane)) break;
+      if (lane == 0) {
+        // (test hook: with bit 2 of debug_stall the flag stays unset, so that the waits on it run out)
+        if (!(a.debug_stall & 4u)) st_flag(flag, a.epoch);
+        mbar_arrive(&sh->empty[s]);
+      }
+    }
   } else {
     // ================================================================ consumer warps
     const int i = tid >> 3;          // pair in tile
     const int c0 = tid & 7;          // chunks c0 and c0 + 8 (16 bytes each)
-    volatile int* fail = &sh->fail;
+    // (no warp waits for another one: barriers of all eight around the waits were the kernel's largest stall)
     for (int k = 0;; ++k) {
       const int s = k % kStages;
       const uint32_t ph = (uint32_t)(k / kStages) & 1u;
-      if (!consumer_wait(&sh->meta_full[s], nullptr, ph, abort_flag, fail, lane)) break;
+      if (!warp_wait(&sh->meta_full[s], ph, abort_flag, lane)) break;
       const TileMeta* m = &sh->meta[s];
       const int t = m->tile;
       if (t < 0) break;
-      if (!consumer_wait(&sh->full[s], nullptr, ph, abort_flag, fail, lane)) break;
+      if (!warp_wait(&sh->full[s], ph, abort_flag, lane)) break;
       const int ts = m->seq, th = m->h;                   // (the tile's unit)
       const int n = tab.s[ts].n, unit = tab.s[ts].b * a.c.Hkv + th;
       __nv_bfloat16* Kb = a.c.K + tab.s[ts].b * a.c.ksb + th * a.c.ksh;
@@ -267,28 +302,21 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
         }
         cl += cr;
       }
-      // the tile's source rows are out of global memory: later tiles may overwrite them
-      // (test hook: with bit 2 of debug_stall the flag stays unset, so that the waits on it run out)
-      if (tid == 0 && !(a.debug_stall & 4u)) st_release_u32(&a.flags[(size_t)unit * a.tile_stride + t], a.epoch);
       const int moved = E0 + __popc(selbits);
-      if (E0 > 0 && (share || unit_ctas > 1)) {
-        // This tile's rows land in [j0 - E0, j0 - E0 + 64): those are source rows of at most two
-        // earlier tiles (and of this tile itself), which must have been read before they are
-        // overwritten; a CTA that owns the whole unit has read them itself, in order
-        const int first = (j0 - E0 - off) / KVS_CTILE;
-        const int last = min(t - 1, first + 1);
-        for (int tt = last - tid; tt >= first; tt -= kConsumers) {
-          const uint32_t* f = &a.flags[(size_t)unit * a.tile_stride + tt];
-          int spins = 0;
-          const uint64_t t0 = globaltimer_ns();
-          while (ld_acquire_u32(f) < a.epoch) {
-            const bool late = (++spins & 255) == 0 && globaltimer_ns() - t0 > (uint64_t)(uint32_t)sh->wait_us * 1000ull;
-            if (late || spins > KVS_SPIN_LIMIT || *abort_flag) { *fail = 1; *abort_flag = 1; break; }
-            __nanosleep(20);
-          }
+      if (ordered && E0 > 0) {
+        // This tile's rows land in [j0 - E0, j0 - E0 + 64): those are source rows of at most two earlier tiles (and of
+        // this tile itself), which must have been read before they are overwritten; a CTA that owns the whole unit has
+        // read them itself, in order.
+        const int before = (KVS_CTILE * t - E0) / KVS_CTILE + lane;
+        const uint32_t* flag = a.flags + (size_t)unit * a.tile_stride + before;
+        bool open = lane < 2 && before < t;
+        int spins = 0;
+        const uint64_t since = globaltimer_ns();
+        while (open && (open = ld_flag(flag) < a.epoch)) {
+          const bool late = (++spins & 255) == 0 && globaltimer_ns() - since > (uint64_t)(uint32_t)sh->wait_us * 1000ull;
+          if (late || spins > KVS_SPIN_LIMIT || *abort_flag) { *abort_flag = 1; break; }
         }
-        consumer_barrier();
-        if (*fail) break;
+        if (__any_sync(0xffffffffu, open)) break;
       }
       if (moved != 0) {
 #pragma unroll
