@@ -210,54 +210,9 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
     misc->wait_us = (int)a.wait_us;
     mbar_fence_init();
   }
-  if (warp == 0 && elect_one()) {
-    prefetch_tmap(&tmKp); prefetch_tmap(&tmVp); prefetch_tmap(&tmQ); prefetch_tmap(&tmOhi); prefetch_tmap(&tmOlo);
-  }
   if (warp == 1) tmem_alloc(&misc->tmem_base, 512);
-  // test hook: the producer requests no K tile, so that the waits on them run out
-  const bool withhold_k = (a.debug_stall & 2u) != 0;
-  // tensor-map coordinates of the pair members: slot = 2 * rho + parity
-  const int par_l = off & 1, par_r = par_l ^ 1;
-  const int rho_l0 = off >> 1, rho_r0 = (off + 1) >> 1;
-  auto request_q = [&](int unit) {
-    mbar_expect_tx(&misc->qfull, (kExact ? 2 : 3) * kOperand);
-    for (int hf = 0; hf < 2; ++hf) {
-      tma_load_3d(smem + kSmemQ + hf * kHalf, &tmQ, &misc->qfull, hf * 64, qblk * kQB, unit);
-      tma_load_3d(smem + kSmemOhi + hf * kHalf, &tmOhi, &misc->qfull, hf * 64, qblk * kQB, unit);
-      if (!kExact) tma_load_3d(smem + kSmemOlo + hf * kHalf, &tmOlo, &misc->qfull, hf * 64, qblk * kQB, unit);
-    }
-  };
-  auto request_c = [&](int unit) {
-    mbar_expect_tx(&misc->cfull, sizeof(misc->qconst));
-    bulk_load(misc->qconst, a.qc2 + ((size_t)unit * a.M_pad + qblk * kQB) * 2, sizeof(misc->qconst), &misc->cfull);
-  };
-  auto request_k = [&](int p0, int h, int b) {
-    if (withhold_k) return;
-    mbar_expect_tx(&misc->kfull, 2 * kOperand);
-    for (int hf = 0; hf < 2; ++hf) {
-      tma_load_5d(smem + kSmemKl + hf * kHalf, &tmKp, &misc->kfull, hf * 64, par_l, rho_l0 + p0, h, b);
-      tma_load_5d(smem + kSmemKr + hf * kHalf, &tmKp, &misc->kfull, hf * 64, par_r, rho_r0 + p0, h, b);
-    }
-  };
-  auto request_v = [&](int p0, int h, int b) {
-    mbar_expect_tx(&misc->vfull, 2 * kOperand);
-    for (int hf = 0; hf < 2; ++hf) {
-      tma_load_5d(smem + kSmemVl + hf * kHalf, &tmVp, &misc->vfull, hf * 64, par_l, rho_l0 + p0, h, b);
-      tma_load_5d(smem + kSmemVr + hf * kHalf, &tmVp, &misc->vfull, hf * 64, par_r, rho_r0 + p0, h, b);
-    }
-  };
   // (everything above runs while the kernel before this one may still be draining)
   kvs_pdl_wait();
-  // The first tile's operands are requested by the thread that made the barriers, before the others know of them: the
-  // queries' constants and the barrier of the CTA take 1100 cycles (ten rounds of 16 units from 16 K slots on, events: 342 -> 338 us,
-  // five of 8 units from 4 K on 67.4 -> 65.5).
-  if (threadIdx.x == 0) {
-    const int b = tab.s[walk0.seq].b, p0 = walk0.t * kPairs;
-    request_q(unit0);
-    if (kShares) request_c(unit0);
-    request_k(p0, walk0.h, b);
-    request_v(p0, walk0.h, b);
-  }
   // the queries' constants: with one unit they are there before the first tile (a wait for a copy of them in the
   // statistics warps costs 12 registers)
   if (!kShares && threadIdx.x < kQB / 2) {
@@ -269,15 +224,23 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, misc->tmem_base, 0);   // (uniform for the compiler too)
   volatile int* abort_flag = &misc->abort_flag;
+  // test hook: the producer requests no K tile, so that the waits on them run out
+  const bool withhold_k = (a.debug_stall & 2u) != 0;
+
+  // tensor-map coordinates of the pair members: slot = 2 * rho + parity
+  const int par_l = off & 1, par_r = par_l ^ 1;
+  const int rho_l0 = off >> 1, rho_r0 = (off + 1) >> 1;
+
   if (warp == 0) {
     // ================================================================ TMA producer
     if (elect_one()) {
+      prefetch_tmap(&tmKp); prefetch_tmap(&tmVp); prefetch_tmap(&tmQ); prefetch_tmap(&tmOhi); prefetch_tmap(&tmOlo);
       // K of a tile is free again before its Vsum rows are (the last logits come before the last T
       // product), and the K of the tile after that cannot be free before these Vsum rows have been
       // used: the requests go out in the fixed order K, V, K, V, ... behind blocking (bounded) waits.
       // Every tile is first requested into L2 one tile ahead, so that the load that fills the (single)
       // stage finds it there.  A segment's query operands come after its first K rows.
-      uint32_t li = 0, kli = 0, vli = 0, seg = 0, qli = 1, cli = kShares ? 1 : 0;   // (the first requests are out already)
+      uint32_t li = 0, kli = 0, vli = 0, seg = 0, qli = 0, cli = 0;
       bool ok = true;
       Walk w = walk0;
       for (bool more = true; ok && more; more = kShares && w.next(tab, a.Hkv), ++seg) {
@@ -291,25 +254,42 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
         };
         auto load_q = [&] {
           if (!mbar_wait(&misc->qfree, (seg & 1) ^ 1, abort_flag)) return false;
-          request_q(unit);
+          mbar_expect_tx(&misc->qfull, (kExact ? 2 : 3) * kOperand);
+          for (int hf = 0; hf < 2; ++hf) {
+            tma_load_3d(smem + kSmemQ + hf * kHalf, &tmQ, &misc->qfull, hf * 64, qblk * kQB, unit);
+            tma_load_3d(smem + kSmemOhi + hf * kHalf, &tmOhi, &misc->qfull, hf * 64, qblk * kQB, unit);
+            if (!kExact) tma_load_3d(smem + kSmemOlo + hf * kHalf, &tmOlo, &misc->qfull, hf * 64, qblk * kQB, unit);
+          }
           ++qli;
           return true;
         };
         auto load_c = [&] {
           if (!mbar_wait(&misc->cfree, (seg & 1) ^ 1, abort_flag)) return false;
-          request_c(unit);
+          mbar_expect_tx(&misc->cfull, sizeof(misc->qconst));
+          bulk_load(misc->qconst, a.qc2 + ((size_t)unit * a.M_pad + qblk * kQB) * 2, sizeof(misc->qconst), &misc->cfull);
           ++cli;
           return true;
         };
+        if (seg == 0 && (!load_q() || (kShares && !load_c()))) break;
         for (int j = 0; j < w.count; ++j, ++li) {
           const int p0 = (w.t + j) * kPairs;
           if (!mbar_wait(&misc->kfree, (li & 1) ^ 1, abort_flag)) { ok = false; break; }
-          if (li > 0) request_k(p0, w.h, b);
+          if (!withhold_k) {
+            mbar_expect_tx(&misc->kfull, 2 * kOperand);
+            for (int hf = 0; hf < 2; ++hf) {
+              tma_load_5d(smem + kSmemKl + hf * kHalf, &tmKp, &misc->kfull, hf * 64, par_l, rho_l0 + p0, w.h, b);
+              tma_load_5d(smem + kSmemKr + hf * kHalf, &tmKp, &misc->kfull, hf * 64, par_r, rho_r0 + p0, w.h, b);
+            }
+          }
           ++kli;
           if (j + 1 < w.count) prefetch(p0 + kPairs, false);
           if (kShares && j == 0 && seg > 0 && !load_q()) { ok = false; break; }
           if (!mbar_wait(&misc->vfree, (li & 1) ^ 1, abort_flag)) { ok = false; break; }
-          if (li > 0) request_v(p0, w.h, b);
+          mbar_expect_tx(&misc->vfull, 2 * kOperand);
+          for (int hf = 0; hf < 2; ++hf) {
+            tma_load_5d(smem + kSmemVl + hf * kHalf, &tmVp, &misc->vfull, hf * 64, par_l, rho_l0 + p0, w.h, b);
+            tma_load_5d(smem + kSmemVr + hf * kHalf, &tmVp, &misc->vfull, hf * 64, par_r, rho_r0 + p0, w.h, b);
+          }
           if (j + 1 < w.count) prefetch(p0 + kPairs, true);
           ++vli;
           if (kShares && j == 0 && seg > 0 && !load_c()) { ok = false; break; }
