@@ -57,10 +57,11 @@ constexpr float kFarLogit = 1048576.f;     // 2^20
 constexpr int kSBufs = 3;                  // logit / P' buffers in tensor memory
 
 struct Misc {
-  uint64_t kfull[kKStages], vfull[kVStages], kfree[kKStages], vfree[kVStages], sfull[kSBufs], pready[kSBufs][2], pvdone[kSBufs], verdict, qfull;
+  uint64_t kfull[kKStages], vfull[kVStages], kfree[kKStages], vfree[kVStages], sfull[kSBufs], pready[kSBufs][2], pvdone[kSBufs], verdict, qfull, done;
   uint32_t tmem_base;
   int abort_flag, wait_us;                 // (adjacent: the bounded waits read both through one pointer)
   int again;                               // the range is walked again with true maxima
+  int k_issued, v_issued;                  // requests of the producer
   alignas(16) float cnt[kSoftmaxWarps][64];   // per warp: the counts of its 64 slots (read as float4)
   float part_max[4][kTile], part_sum[4][kTile];   // the four parts (team x column half) of every row's maximum and sum
 };
@@ -216,6 +217,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     }
     mbar_init(&misc->verdict, kSoftmaxWarps);
     mbar_init(&misc->qfull, 1);
+    mbar_init(&misc->done, 2);             // all products: the commits of both issuers
     misc->again = 0;
     misc->abort_flag = 0;
     misc->wait_us = (int)a.wait_us;
@@ -283,11 +285,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
         }
         if (ok && walk == 0) n_walks = walks();
       }
-      if (*abort_flag) {
-        // drain: give the copies already issued a bounded time to land before the CTA leaves
-        for (int gi = max(0, kgi - kKStages); gi < kgi && !withhold_k; ++gi) mbar_drain(&misc->kfull[gi % kKStages], (gi / kKStages) & 1);
-        for (int gi = max(0, vgi - kVStages); gi < vgi; ++gi) mbar_drain(&misc->vfull[gi % kVStages], (gi / kVStages) & 1);
-      }
+      misc->k_issued = kgi; misc->v_issued = vgi;
     }
   } else if (warp == 1) {
     // ================================================================ issuer of the S products
@@ -322,6 +320,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
         tc_commit(&misc->kfree[s]);
         if (gi == my_tiles - 1) end = walks() * my_tiles;
       }
+      tc_commit(&misc->done);                              // (behind a walk that broke off, too)
     }
   } else if (warp == kPvWarp<kNorms>) {
     // ================================================================ issuer of the P V products
@@ -362,6 +361,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
           if (gi == my_tiles - 1) end = walks() * my_tiles;
         }
       }
+      tc_commit(&misc->done);
     }
   } else if (warp >= 2 + kSoftmaxWarps) {
     // ================================================================ pair-norm warps
@@ -615,7 +615,21 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp >= 2 && warp < 2 + kSoftmaxWarps && !*abort_flag) {   // (no wait is left that could set it: the same for all)
+  const bool gave_up = *abort_flag != 0;                   // (no wait is left that could set it: the same for all)
+  // Nothing may be in flight when the CTA leaves: its shared and tensor memory are the next CTA's from then on.  Whole walks
+  // have waited for their copies and products, but for the last arrivals that hand the stages back; behind one that
+  // broke off, in whichever role and after whichever request, any copy and any product may be under way.
+  if (threadIdx.x == 0) {
+    const int nk = misc->k_issued, nv = misc->v_issued;
+    mbar_drain(&misc->done, 0);
+    if (gave_up) mbar_drain(&misc->qfull, 0);
+    if (!(gave_up && withhold_k))
+      for (int gi = max(0, nk - kKStages); gi < nk; ++gi)
+        mbar_drain(gave_up ? &misc->kfull[gi % kKStages] : &misc->kfree[gi % kKStages], (gi / kKStages) & 1);
+    for (int gi = max(0, nv - kVStages); gi < nv; ++gi)
+      mbar_drain(gave_up ? &misc->vfull[gi % kVStages] : &misc->vfree[gi % kVStages], (gi / kVStages) & 1);
+  }
+  if (warp >= 2 && warp < 2 + kSoftmaxWarps && !gave_up) {
     const int part = (warp - 2) >> 2, row = (warp & 3) * 32 + lane;
     uint8_t* stage = smem + kSmemK;
     float ov[32];
@@ -640,7 +654,7 @@ flash_partial_tc(const FlashTcArgs a, const RoundTable tab, const __grid_constan
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
-  if (threadIdx.x == 0 && misc->abort_flag && a.status_dev) atomicExch(a.status_dev, (int)KVS_ERR_TIMEOUT);
+  if (threadIdx.x == 0 && gave_up && a.status_dev) atomicExch(a.status_dev, (int)KVS_ERR_TIMEOUT);
 }
 
 }  // namespace

@@ -72,10 +72,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
   return true;
 }
-// Time a role gives copies already in flight to land before its CTA leaves after an abort.
+// Time a role gives copies or products already in flight to arrive on a barrier before its CTA leaves: the memory of the
+// barriers and of the operands belongs to the next CTA of the SM from then on.
 __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+  if (mbar_try_wait(bar, parity)) return;
   const uint64_t t1 = globaltimer_ns();
-  while (!mbar_try_wait(bar, parity) && globaltimer_ns() - t1 < 200000000ull) {}
+  while (!mbar_try_wait_hint(bar, parity, 10000u) && globaltimer_ns() - t1 < 200000000ull) {}
 }
 
 // Loads that stay where they are written: the compiler may move a plain load of a value that is

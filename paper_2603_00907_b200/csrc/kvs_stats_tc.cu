@@ -61,9 +61,10 @@ constexpr int kBoundThreads = 544;
 static_assert(KVS_STATS_GROUPS == kGroups, "the launcher sizes the partials with KVS_STATS_GROUPS");
 
 struct Misc {
-  uint64_t kfull, vfull, kfree, vfree, tfull[2], tfree[2], qfull, qfree, cfull, cfree;
+  uint64_t kfull, vfull, kfree, vfree, tfull[2], tfree[2], qfull, qfree, cfull, cfree, done;
   uint32_t tmem_base;
   int abort_flag, wait_us;                 // (adjacent: the bounded waits read both through one pointer)
+  uint32_t k_issued, v_issued, q_issued, c_issued;   // requests of the producer
   // per two queries (2k, 2k+1) of the block: (c_2k, c_2k+1, h_2k, h_2k+1) with c = -(max + log2 Z) and
   // h = |o|^2 (or <E, o>): neighbours sit side by side for the packed two-float arithmetic
   alignas(16) float qconst[2 * kQB];
@@ -206,6 +207,7 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
     mbar_init(&misc->qfree, kIssuers);     // a segment's last products: the query operands may be replaced
     mbar_init(&misc->cfull, 1);            // the queries' constants of the segment
     mbar_init(&misc->cfree, kStatWarps);
+    mbar_init(&misc->done, kIssuers);      // all products of the CTA
     misc->abort_flag = 0;
     misc->wait_us = (int)a.wait_us;
     mbar_fence_init();
@@ -295,13 +297,7 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
           if (kShares && j == 0 && seg > 0 && !load_c()) { ok = false; break; }
         }
       }
-      if (*abort_flag) {
-        // drain: give the copies already issued a bounded time to land before the CTA leaves
-        if (kli > 0 && !withhold_k) mbar_drain(&misc->kfull, (kli - 1) & 1);
-        if (vli > 0) mbar_drain(&misc->vfull, (vli - 1) & 1);
-        if (qli > 0) mbar_drain(&misc->qfull, (qli - 1) & 1);
-        if (cli > 0) mbar_drain(&misc->cfull, (cli - 1) & 1);
-      }
+      misc->k_issued = kli; misc->v_issued = vli; misc->q_issued = qli; misc->c_issued = cli;
     }
   } else if (warp < kFirstStat) {
     // ================================================================ product issuers
@@ -355,6 +351,7 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
         }
         if (ok) tc_commit(&misc->qfree);
       }
+      tc_commit(&misc->done);                              // (behind a walk that broke off, too)
     }
   } else {
     // ================================================================ statistics warps
@@ -476,14 +473,33 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
   }
 
   // ================================================================== common exit
+  // Nothing may be in flight when the CTA leaves: its shared and tensor memory are the next CTA's from then on.  A whole walk
+  // has waited for its copies and products, but for the last commits that hand the operands back; behind one that
+  // broke off, in whichever role and after whichever request, any copy and any product may be under way.
   tc_fence_before();
   __syncthreads();
+  const bool gave_up = *abort_flag != 0;                   // (no wait is left that could set it)
   if (warp == 1) {
+    if (gave_up && lane == 0) mbar_drain(&misc->done, 0);
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
-  if (threadIdx.x == 0 && misc->abort_flag && a.status_dev) atomicExch(a.status_dev, (int)KVS_ERR_TIMEOUT);
+  if (threadIdx.x == 0) {
+    const uint32_t nk = misc->k_issued, nv = misc->v_issued, nq = misc->q_issued, nc = misc->c_issued;
+    mbar_drain(&misc->done, 0);
+    if (gave_up) {
+      if (nk > 0 && !withhold_k) mbar_drain(&misc->kfull, (nk - 1) & 1);
+      if (nv > 0) mbar_drain(&misc->vfull, (nv - 1) & 1);
+      if (nq > 0) mbar_drain(&misc->qfull, (nq - 1) & 1);
+      if (nc > 0) mbar_drain(&misc->cfull, (nc - 1) & 1);
+      if (a.status_dev) atomicExch(a.status_dev, (int)KVS_ERR_TIMEOUT);
+    } else {
+      mbar_drain(&misc->kfree, (nk - 1) & 1);
+      mbar_drain(&misc->vfree, (nv - 1) & 1);
+      mbar_drain(&misc->qfree, (nq - 1) & 1);
+    }
+  }
 }
 
 }  // namespace
