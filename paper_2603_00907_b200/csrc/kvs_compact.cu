@@ -9,17 +9,18 @@
 // rows
 //   K*    = bf16( K_right + w (K_left - K_right) )        [Eq. kstar_final, weight form]
 //   Vsum* = bf16( Vsum_left + Vsum_right ),  c* = c_left + c_right   [v* = v_m + v_{m+1}]
-// wait (bounded) until every earlier tile whose source rows they are about to overwrite has loaded, and store the surviving
-// rows at
+// wait until the tile may be stored, that is until every earlier tile whose source rows it overwrites has loaded, and store the
+// surviving rows at
 //   new slot = old slot - (merged pairs before it).
 // Where several CTAs handle tiles of a unit, a publisher warp says that a tile has loaded as soon as its copies have landed.
+// A gate warp waits (bounded) for the other tiles in place of all consumers and opens a tile for them: it is stored by
+// all of them or, behind a wait that ran out, by none.
 // Tickets make the wait safe: a tile only waits for tiles of its unit with smaller tickets, which were taken before its own.
 // Every CTA publishes and handles its tiles, of one unit or of several, in the order in which it took them, so
 // that of all tiles not yet published the one taken first never waits.
-// Bound by HBM in long units, by the chain of ticket, copies, flags and stores in short ones.  8 units of 2048 tiles
-// 185 -> 150 us a launch (events), nine rounds of 8 units from 512 tiles on 252 -> 186, five of 8 units from 64 on 68 -> 64,
-// against barriers of all consumers around every wait, flags set and looked at by consumers with release and acquire, and all
-// of the set-up behind the wait for the kernel in front.
+// Bound by HBM in long units, by the chain of ticket, copies, flags and stores in short ones.  8 units of 2048 tiles 149 us a
+// launch (events), nine rounds of 8 units from 512 tiles on 173, five of 8 units from 64 on 62; with barriers of all consumers
+// around every wait, and flags set and looked at by consumers, 185, 248 and 73.
 #include "kvs_internal.h"
 #include "kvs_sm100.cuh"
 
@@ -50,8 +51,12 @@ constexpr int kRowBytes = KVS_D * 2;                       // one bf16 row
 constexpr int kOperandBytes = KVS_CTILE * kRowBytes;       // 16 KB: the K (or Vsum) rows of a tile
 constexpr int kStageBytes = 2 * kOperandBytes;
 constexpr int kConsumers = 256;
-constexpr int kProducer = kConsumers / 32, kPublisher = kProducer + 1;   // warps
-constexpr int kThreads = kConsumers + 64;
+constexpr int kProducer = kConsumers / 32, kPublisher = kProducer + 1, kGate = kProducer + 2;   // warps
+constexpr int kThreads = kConsumers + 96;
+// Barriers of the gate's verdicts: a consumer arrives on `empty` of a tile before it waits for the verdict, and is past the
+// verdict on tile k when it arrives for tile k + kStages, without which tile k + 2 kStages has no stage.
+constexpr int kOpen = 2 * kStages;
+constexpr uint32_t kNever = 0xffffffffu;
 
 struct TileMeta {
   int32_t tile;                  // -1: no more tiles
@@ -63,7 +68,9 @@ struct TileMeta {
 };
 struct Shared {
   uint64_t full[kStages], meta_full[kStages], empty[kStages];
+  uint64_t open[kOpen];          // the rows of the tile may be stored
   int abort_flag, wait_us;       // (adjacent: the bounded waits read both through one pointer)
+  uint32_t closed;               // written by the gate only: it has opened this many of the CTA's tiles and will open no more
   TileMeta meta[kStages];
 };
 constexpr int kSmemBytes = kStages * kStageBytes + (int)sizeof(Shared);
@@ -72,9 +79,12 @@ constexpr int kSmemBytes = kStages * kStageBytes + (int)sizeof(Shared);
 // says so) before the flag is set, and the flag has been seen before the rows are overwritten.  Nothing that was
 // written has to become visible with them, so they are relaxed: a release and an acquire at GPU scope took 1.5 and
 // 2 thousand cycles a tile (nine rounds of 8 units from 512 tiles on, events: 260 us, relaxed 230).
-__device__ __forceinline__ uint32_t ld_flag(const uint32_t* p) {
+// They are looked at with an atomic, which goes to the one place where the line lives.  A load leaves copies of a line that is
+// about to be written in the caches in between: a CTA that looked a little too early saw the flag 2 us late (a launch of 8
+// units of 256 tiles with loads 25.5 us, so 22.5; 64 units of 24 tiles 20.9 and 19.0; ragged rounds of 4 K to 64 K slots 950 and 928).
+__device__ __forceinline__ uint32_t see_flag(uint32_t* p) {
   uint32_t v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  asm volatile("atom.relaxed.gpu.global.or.b32 %0, [%1], 0;" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_flag(uint32_t* p, uint32_t v) {
@@ -85,6 +95,32 @@ __device__ __forceinline__ void st_flag(uint32_t* p, uint32_t v) {
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int lane) {
   int ok = 1;
   if (lane == 0) ok = mbar_wait(bar, parity, abort_flag) ? 1 : 0;
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  __syncwarp();
+  return ok != 0;
+}
+
+// The consumers' waits, which end with the phase or with the gate: they never give up on a tile that the gate has opened or
+// may still open.  The gate itself gives up on a tile after three time limits at the most (decision, flags, copies);
+// far beyond that the wait ends all the same.
+__device__ __forceinline__ uint32_t ld_closed(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_closed(uint32_t* p, uint32_t v) {
+  asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ bool follow(uint64_t* bar, uint32_t parity, Shared* sh, uint32_t k, int lane) {
+  int ok = 1;
+  if (lane == 0 && !mbar_try_wait(bar, parity)) {
+    const uint64_t since = globaltimer_ns();
+    while (!mbar_try_wait_hint(bar, parity, 10000u)) {
+      const bool late = globaltimer_ns() - since > (uint64_t)(uint32_t)sh->wait_us * 8000ull + 100000000ull;
+      if (late) *(volatile int*)&sh->abort_flag = 1;
+      if (late || ld_closed(&sh->closed) <= k) { ok = 0; break; }
+    }
+  }
   ok = __shfl_sync(0xffffffffu, ok, 0);
   __syncwarp();
   return ok != 0;
@@ -125,9 +161,11 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&sh->full[s], 1);
       mbar_init(&sh->meta_full[s], 1);
-      mbar_init(&sh->empty[s], kConsumers / 32 + (ordered ? 1 : 0));
+      mbar_init(&sh->empty[s], kConsumers / 32 + 1 + (ordered ? 1 : 0));
     }
+    for (int s = 0; s < kOpen; ++s) mbar_init(&sh->open[s], 1);
     sh->abort_flag = 0;
+    sh->closed = kNever;
     sh->wait_us = (int)a.wait_us;
     mbar_fence_init();
   }
@@ -156,12 +194,7 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
     for (int k = 0;; ++k) {
       const int s = k % kStages;
       const uint32_t ph = (uint32_t)(k / kStages) & 1u;
-      if (!warp_wait(&sh->empty[s], ph ^ 1u, abort_flag, lane)) {
-        // give the copies of the last stages a bounded time to land before the CTA leaves
-        if (lane == 0)
-          for (int kk = max(0, issued - kStages); kk < issued; ++kk) mbar_drain(&sh->full[kk % kStages], (uint32_t)(kk / kStages) & 1u);
-        break;
-      }
+      if (!warp_wait(&sh->empty[s], ph ^ 1u, abort_flag, lane)) break;
       int t;
       for (;;) {
         if (!ahead && lane == 0) next_ticket = atomicAdd(&a.tickets[cu], 1u);
@@ -233,6 +266,9 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh->meta_full[s]);
     }
+    // No copy may be in flight when the CTA leaves, whoever gave up and when.
+    if (lane == 0)
+      for (int kk = max(0, issued - kStages); kk < issued; ++kk) mbar_drain(&sh->full[kk % kStages], (uint32_t)(kk / kStages) & 1u);
   } else if (warp == kPublisher) {
     // ================================================================ publisher
     // (up to two tiles before the consumers get to them; a publisher that also waited for the other tiles' flags was late with
@@ -246,11 +282,47 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
       uint32_t* flag = a.flags + (size_t)(tab.s[m->seq].b * a.c.Hkv + m->h) * a.tile_stride + m->tile;
       if (!warp_wait(&sh->full[s], ph, abort_flag, lane)) break;
       if (lane == 0) {
+        mbar_arrive(&sh->empty[s]);
         // (test hook: with bit 2 of debug_stall the flag stays unset, so that the waits on it run out)
         if (!(a.debug_stall & 4u)) st_flag(flag, a.epoch);
-        mbar_arrive(&sh->empty[s]);
       }
     }
+  } else if (warp == kGate) {
+    // ================================================================ gate
+    uint32_t k = 0;
+    bool shut = false;
+    for (;; ++k) {
+      const int s = (int)(k % kStages);
+      const uint32_t ph = (k / kStages) & 1u;
+      shut = !warp_wait(&sh->meta_full[s], ph, abort_flag, lane);
+      if (shut) break;
+      const TileMeta* m = &sh->meta[s];
+      const int t = m->tile, E0 = m->E0;
+      if (t < 0) break;
+      uint32_t* flags = a.flags + (size_t)(tab.s[m->seq].b * a.c.Hkv + m->h) * a.tile_stride;
+      if (ordered && E0 > 0) {
+        // The tile's rows land in [j0 - E0, j0 - E0 + 64): those are source rows of at most two earlier tiles (and of
+        // this tile itself), which must have been read before they are overwritten; a CTA that owns the whole unit has
+        // read them itself, in order.
+        const int before = (KVS_CTILE * t - E0) / KVS_CTILE + lane;
+        shut = lane < 2 && before < t;
+        int spins = 0;
+        const uint64_t since = globaltimer_ns();
+        while (shut && (shut = see_flag(flags + before) < a.epoch)) {
+          const bool late = (++spins & 255) == 0 && globaltimer_ns() - since > (uint64_t)(uint32_t)sh->wait_us * 1000ull;
+          if (late || spins > KVS_SPIN_LIMIT || *abort_flag) { *abort_flag = 1; break; }
+        }
+        shut = __any_sync(0xffffffffu, shut);
+        if (shut) break;
+      }
+      shut = !warp_wait(&sh->full[s], ph, abort_flag, lane);
+      if (shut) break;
+      if (lane == 0) {
+        mbar_arrive(&sh->empty[s]);
+        mbar_arrive(&sh->open[k % kOpen]);
+      }
+    }
+    if (lane == 0 && shut) st_closed(&sh->closed, k);
   } else {
     // ================================================================ consumer warps
     const int i = tid >> 3;          // pair in tile
@@ -259,11 +331,11 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
     for (int k = 0;; ++k) {
       const int s = k % kStages;
       const uint32_t ph = (uint32_t)(k / kStages) & 1u;
-      if (!warp_wait(&sh->meta_full[s], ph, abort_flag, lane)) break;
+      if (!follow(&sh->meta_full[s], ph, sh, k, lane)) break;
       const TileMeta* m = &sh->meta[s];
       const int t = m->tile;
       if (t < 0) break;
-      if (!warp_wait(&sh->full[s], ph, abort_flag, lane)) break;
+      if (!follow(&sh->full[s], ph, sh, k, lane)) break;
       const int ts = m->seq, th = m->h;                   // (the tile's unit)
       const int n = tab.s[ts].n, unit = tab.s[ts].b * a.c.Hkv + th;
       __nv_bfloat16* Kb = a.c.K + tab.s[ts].b * a.c.ksb + th * a.c.ksh;
@@ -303,21 +375,7 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
         cl += cr;
       }
       const int moved = E0 + __popc(selbits);
-      if (ordered && E0 > 0) {
-        // This tile's rows land in [j0 - E0, j0 - E0 + 64): those are source rows of at most two earlier tiles (and of
-        // this tile itself), which must have been read before they are overwritten; a CTA that owns the whole unit has
-        // read them itself, in order.
-        const int before = (KVS_CTILE * t - E0) / KVS_CTILE + lane;
-        const uint32_t* flag = a.flags + (size_t)unit * a.tile_stride + before;
-        bool open = lane < 2 && before < t;
-        int spins = 0;
-        const uint64_t since = globaltimer_ns();
-        while (open && (open = ld_flag(flag) < a.epoch)) {
-          const bool late = (++spins & 255) == 0 && globaltimer_ns() - since > (uint64_t)(uint32_t)sh->wait_us * 1000ull;
-          if (late || spins > KVS_SPIN_LIMIT || *abort_flag) { *abort_flag = 1; break; }
-        }
-        if (__any_sync(0xffffffffu, open)) break;
-      }
+      if (!follow(&sh->open[k % kOpen], (uint32_t)(k / kOpen) & 1u, sh, k, lane)) break;
       if (moved != 0) {
 #pragma unroll
         for (int u = 0; u < 2; ++u) {

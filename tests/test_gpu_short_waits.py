@@ -81,3 +81,74 @@ def test_decode_leaves_nothing_behind(kb, hkv, batch, n, rows):
     clean = call()
     assert clean[0].item() == 0
     _outcomes(kb, call, clean)
+
+
+# KV heads, lengths, share of the pairs that merge: units of many tiles for all CTAs, for two CTAs each, for one CTA each,
+# units of different lengths whose CTAs help one another (the waits of a CTA are then for tiles of several units)
+@pytest.mark.parametrize("hkv,lens,share", [(8, [30000], 0.5), (8, [2600], 0.1), (8, [6000] * 16, 0.5), (8, [1200] * 36, 0.5),
+                                            (2, [40000] + [3000 + 40 * i for i in range(40)], 0.3)])
+@pytest.mark.parametrize("token_major", [False, True])
+def test_a_compaction_stores_a_tile_whole_or_not_at_all(kb, hkv, lens, share, token_major):
+    import torch
+    batch, n_max, recent, off = len(lens), max(lens) + 3, 4, 32
+    g = torch.Generator(device="cuda")
+    g.manual_seed(batch + hkv)
+    shape = (batch, n_max, hkv, 128) if token_major else (batch, hkv, n_max, 128)
+    K0, V0 = (torch.randn(shape, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    if token_major:
+        K0, V0 = K0.transpose(1, 2), V0.transpose(1, 2)
+    counts0 = torch.randint(1, 1 << 20, (batch, hkv, n_max), generator=g, device="cuda", dtype=torch.int32)
+    w = torch.rand(batch, hkv, n_max // 2, generator=g, device="cuda")
+    mask = torch.zeros(batch, hkv, n_max // 2, dtype=torch.uint8, device="cuda")
+    merged = []
+    for b, n in enumerate(lens):
+        pairs = (n - off - recent) // 2
+        merged.append(int(share * pairs))
+        order = torch.rand(hkv, pairs, generator=g, device="cuda").argsort(-1)
+        mask[b].scatter_(1, order[:, :merged[-1]], 1)
+    p = kb.make_params(K0, V0, hkv, recent)
+    ws = torch.empty(kb.kvs_workspace_size(p, n_max, 0), dtype=torch.uint8, device="cuda")
+    index = torch.zeros(batch, hkv, n_max, dtype=torch.int32, device="cuda")
+
+    def call(new_index=None):
+        K, V, counts = (x.clone(memory_format=torch.preserve_format) for x in (K0, V0, counts0))
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        kb.kvs_compact(p, K, V, counts, mask, w, lens, merged, ws, new_index=new_index, status_dev=status)
+        return [status, K, V, counts]
+
+    clean = call(index)
+    assert clean[0].item() == 0
+
+    def rows(a, b):
+        """[batch, heads, slots]: where key, value sum and count of the slot are the same in both caches."""
+        return (a[1] == b[1]).all(-1) & (a[2] == b[2]).all(-1) & (a[3] == b[3])
+
+    seen = set()
+    moved = ~rows(clean, [None, K0, V0, counts0])          # slots that the compaction changes
+    for limit in LIMITS_US:
+        kb.kvs_debug_set_wait(limit, 0)
+        try:
+            got = call()
+            torch.cuda.synchronize()
+        finally:
+            kb.kvs_debug_set_wait(0, 0)
+        seen.add(got[0].item())
+        done, still = rows(got, clean), rows(got, [None, K0, V0, counts0])
+        for b, n in enumerate(lens):
+            left = n - merged[b]
+            # the tile that writes slot d is the one of the slots that move there
+            tile = torch.zeros(hkv, left, dtype=torch.int64, device="cuda")
+            src = torch.arange(n, device="cuda").expand(hkv, n)
+            tile.scatter_(1, index[b, :, :n].long(), (src - off).clamp(min=0) // 64)
+            ntiles = (n - off + 63) // 64
+            m, d = moved[b, :, :left], done[b, :, :left]
+            assert bool((d | still[b, :, :left]).all())
+            stored, missing = (torch.zeros(hkv, ntiles, dtype=torch.int32, device="cuda").scatter_add_(1, tile, x.int())
+                               for x in (m & d, m & ~d))
+            assert not bool(((stored > 0) & (missing > 0)).any()), limit
+            if got[0].item() == 0:
+                assert int(missing.sum()) == 0
+        again = call()
+        assert again[0].item() == 0 and all(torch.equal(x, y) for x, y in zip(again[3:], clean[3:]))
+        assert bool(rows(again, clean)[:, :, :min(n - k for n, k in zip(lens, merged))].all())
+    assert KVS_ERR_TIMEOUT in seen and seen <= {0, KVS_ERR_TIMEOUT}
