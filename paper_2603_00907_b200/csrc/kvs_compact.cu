@@ -12,14 +12,15 @@
 // wait until the tile may be stored, that is until every earlier tile whose source rows it overwrites has loaded, and store the
 // surviving rows at
 //   new slot = old slot - (merged pairs before it).
-// Where several CTAs handle tiles of a unit, a publisher warp says that a tile has loaded as soon as its copies have landed.
+// Where several CTAs handle tiles of a unit, a publisher warp says that a tile has loaded, as soon as its copies have landed or
+// a few tiles later.
 // A gate warp waits (bounded) for the other tiles in place of all consumers and opens a tile for them: it is stored by
 // all of them or, behind a wait that ran out, by none.
 // Tickets make the wait safe: a tile only waits for tiles of its unit with smaller tickets, which were taken before its own.
-// Every CTA publishes and handles its tiles, of one unit or of several, in the order in which it took them, so
-// that of all tiles not yet published the one taken first never waits.
-// Bound by HBM in long units, by the chain of ticket, copies, flags and stores in short ones.  8 units of 2048 tiles 149 us a
-// launch (events), nine rounds of 8 units from 512 tiles on 173, five of 8 units from 64 on 62; with barriers of all consumers
+// Every CTA handles its tiles, of one unit or of several, in the order in which it took them, and publishes one without waiting
+// for anything but tiles that it took before, so that of all tiles not yet published the one taken first never waits.
+// Bound by HBM in long units, by the chain of ticket, copies, flags and stores in short ones.  8 units of 2048 tiles 152 us a
+// launch (events), nine rounds of 8 units from 512 tiles on 185, five of 8 units from 64 on 67; with barriers of all consumers
 // around every wait, and flags set and looked at by consumers, 185, 248 and 73.
 #include "kvs_internal.h"
 #include "kvs_sm100.cuh"
@@ -75,20 +76,20 @@ struct Shared {
 };
 constexpr int kSmemBytes = kStages * kStageBytes + (int)sizeof(Shared);
 
-// The "tile loaded" flags.  What they order is a read before a write: the copy of a tile's rows has completed (its mbarrier
-// says so) before the flag is set, and the flag has been seen before the rows are overwritten.  Nothing that was
-// written has to become visible with them, so they are relaxed: a release and an acquire at GPU scope took 1.5 and
-// 2 thousand cycles a tile (nine rounds of 8 units from 512 tiles on, events: 260 us, relaxed 230).
+// The "tile loaded" flags order a read before a write: the copies of a tile's rows and counts, complete when the flag is set,
+// before the stores that overwrite them in another CTA.  Release and acquire are what the memory model has for that.  The
+// acquire is free in the gate, the release is not: with relaxed flags 8 units of 256 tiles take 22.5 us a launch and
+// so 24.5, of 2048 149 and 152, 128 of 256 300 and 309, all rounds of a ragged batch of 4 K to 64 K slots 927 and 977.
 // They are looked at with an atomic, which goes to the one place where the line lives.  A load leaves copies of a line that is
 // about to be written in the caches in between: a CTA that looked a little too early saw the flag 2 us late (a launch of 8
-// units of 256 tiles with loads 25.5 us, so 22.5; 64 units of 24 tiles 20.9 and 19.0; ragged rounds of 4 K to 64 K slots 950 and 928).
+// units of 256 tiles with loads 34.4 us, so 23.2; 64 units of 24 tiles 23.0 and 20.9).
 __device__ __forceinline__ uint32_t see_flag(uint32_t* p) {
   uint32_t v;
-  asm volatile("atom.relaxed.gpu.global.or.b32 %0, [%1], 0;" : "=r"(v) : "l"(p) : "memory");
+  asm volatile("atom.acquire.gpu.global.or.b32 %0, [%1], 0;" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_flag(uint32_t* p, uint32_t v) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // One lane waits, the warp follows.
@@ -273,19 +274,31 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
     // ================================================================ publisher
     // (up to two tiles before the consumers get to them; a publisher that also waited for the other tiles' flags was late with
     // its next tile: nine rounds of 8 units from 512 tiles on 220 us, so 187)
+    // A tile that nobody overwrites soon -- the first that does so follows E0 slots later -- waits for up to two more tiles, so that
+    // one release serves three: 128 units of 256 tiles 331 -> 309 us a launch, 8 of 2048 158 -> 152.  With no more
+    // tiles than stages, the last one's stage comes free with tiles taken before the first.
+    uint32_t* mine = nullptr;        // of lane i: the i-th flag to be set
+    int due = 0;
     for (int k = 0; ordered; ++k) {
       const int s = k % kStages;
       const uint32_t ph = (uint32_t)(k / kStages) & 1u;
       if (!warp_wait(&sh->meta_full[s], ph, abort_flag, lane)) break;
       const TileMeta* m = &sh->meta[s];
-      if (m->tile < 0) break;
-      uint32_t* flag = a.flags + (size_t)(tab.s[m->seq].b * a.c.Hkv + m->h) * a.tile_stride + m->tile;
-      if (!warp_wait(&sh->full[s], ph, abort_flag, lane)) break;
-      if (lane == 0) {
-        mbar_arrive(&sh->empty[s]);
-        // (test hook: with bit 2 of debug_stall the flag stays unset, so that the waits on it run out)
-        if (!(a.debug_stall & 4u)) st_flag(flag, a.epoch);
+      const bool more = m->tile >= 0;
+      bool in_time = false;
+      if (more) {
+        if (lane == due) mine = a.flags + (size_t)(tab.s[m->seq].b * a.c.Hkv + m->h) * a.tile_stride + m->tile;
+        in_time = m->E0 >= 3 * unit_ctas * KVS_CTILE;
+        if (!warp_wait(&sh->full[s], ph, abort_flag, lane)) break;
+        if (lane == 0) mbar_arrive(&sh->empty[s]);
+        ++due;
       }
+      if (!in_time || due == kStages) {
+        // (test hook: with bit 2 of debug_stall the flags stay unset, so that the waits on them run out)
+        if (lane < due && !(a.debug_stall & 4u)) st_flag(mine, a.epoch);
+        due = 0;
+      }
+      if (!more) break;
     }
   } else if (warp == kGate) {
     // ================================================================ gate
