@@ -424,6 +424,30 @@ merge_compact_kernel(const CompactArgs a, const RoundTable tab) {
 
 }  // namespace
 
+// Persistent CTAs, two per SM over all units of the launch, in proportion to the units' lengths; the grid is as wide as the
+// longest unit's part, the CTAs beyond a unit's part leave at once.
+// Where the rounding of the parts, or one CTA to each of many units, leaves a unit with a quarter more tiles a CTA than
+// the average, CTAs that are done go on with the unit that has most left.  All units then need the flags, and a CTA
+// changes its unit for few tiles at a time where units are short, so only from 40 tiles of the busiest CTA on.  Us a launch
+// without and with the others' help: 160 units of 63 tiles 130 and 109, 256 of 65 to 124 256 and 234, 128 of 72 to 125 160 and 128, 64 of 265 to
+// 444 219 and 213; but 192 of 17 90 and 141, 256 of 20 to 38 86 and 109, of 11 to 37 80 and 93, 128 of 11 to 36 37 and 40; and
+// less than a quarter above the average 80 of 63 64 and 62, 96 of 67 73 and 76, 32 of 134 to 376 93 and 96.
+int kvs_detail_compact_shares(const int32_t* tiles, int32_t nseq, int32_t Hkv, int32_t* per_unit) {
+  long long all_tiles = 0;
+  for (int i = 0; i < nseq; ++i) all_tiles += tiles[i];
+  all_tiles *= Hkv;
+  for (int share = 0;; ++share) {
+    double worst = 0.;                                     // tiles of the CTA that has most of them
+    *per_unit = 1;
+    for (int i = 0; i < nseq; ++i) {
+      const int c = ctas_of_unit(tiles[i], all_tiles, share != 0);
+      if (c > *per_unit) *per_unit = c;
+      if (c > 0 && (double)tiles[i] / c > worst) worst = (double)tiles[i] / c;
+    }
+    if (share || !(worst >= 40. && worst * (2 * 148) > 1.25 * (double)all_tiles)) return share;
+  }
+}
+
 cudaError_t kvs_launch_compact(const CompactArgs& a, const RoundTable& t, cudaStream_t st) {
   static KvsPerDeviceOnce configured;
   cudaError_t ce = configured.run([] {
@@ -435,28 +459,10 @@ cudaError_t kvs_launch_compact(const CompactArgs& a, const RoundTable& t, cudaSt
   const int ntiles = (nmax - t.off + KVS_CTILE - 1) / KVS_CTILE;
   // (units that end inside the protected prefix still get their identity slot map)
   if (nmax <= 0 || (ntiles <= 0 && !a.new_index)) return cudaSuccess;
-  // persistent CTAs: two per SM over all units of the launch, in proportion to the units' lengths;
-  // the grid is as wide as the longest unit's share, the CTAs beyond a unit's share leave at once
-  long long all_tiles = 0;
-  for (int i = 0; i < t.nseq; ++i) all_tiles += tiles_of(t.s[i].n, t.off);
-  all_tiles *= a.c.Hkv;
-  // Where the rounding of the shares, or one CTA to each of many short units, leaves a unit with a quarter more tiles a CTA than
-  // the average, CTAs that are done go on with the unit that has most left (64 units of 64 to 1024 tiles, eight
-  // rounds: 1430 -> 1262 us).  Such units always need the flags, so not below: 256 equal units on 296 CTAs, a sixth above the
-  // average, 119 us a round when each CTA keeps to its unit, 159 with the others' help.
   CompactArgs args = a;
-  int per_unit = 1;
-  for (int share = 0; share < 2; ++share) {
-    double worst = 0.;                                     // tiles of the CTA that has most of them
-    per_unit = 1;
-    for (int i = 0; i < t.nseq; ++i) {
-      const int nt = tiles_of(t.s[i].n, t.off), c = ctas_of_unit(nt, all_tiles, share != 0);
-      if (c > per_unit) per_unit = c;
-      if (c > 0 && (double)nt / c > worst) worst = (double)nt / c;
-    }
-    args.share = share;
-    if (share == 0 && !(worst >= 4. && worst * (2 * 148) > 1.25 * (double)all_tiles)) break;
-  }
+  int32_t tiles[KVS_SEQ_CHUNK], per_unit = 1;
+  for (int i = 0; i < t.nseq; ++i) tiles[i] = tiles_of(t.s[i].n, t.off);
+  args.share = kvs_detail_compact_shares(tiles, t.nseq, a.c.Hkv, &per_unit);
   dim3 grid(per_unit, a.c.Hkv, t.nseq);
   return kvs_launch_chained(merge_compact_kernel, grid, dim3(kThreads), kSmemBytes, st, args, t);
 }

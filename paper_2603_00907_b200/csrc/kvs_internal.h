@@ -194,6 +194,9 @@ cudaError_t kvs_launch_mask_prefix(const SelectArgs& a, const RoundTable& t, cud
 cudaError_t kvs_launch_adjacent_cosine(const void* x, int64_t sb, int64_t sh, int64_t st, int H, int n_max,
                                        float* out, const RoundTable& t, cudaStream_t stream);
 cudaError_t kvs_launch_compact(const CompactArgs& a, const RoundTable& t, cudaStream_t st);
+// Whether the compaction of nseq * Hkv units of `tiles` tiles each lets CTAs help other units; *per_unit: the CTAs of the
+// longest unit (host only; with C linkage for the tests).
+extern "C" int kvs_detail_compact_shares(const int32_t* tiles, int32_t nseq, int32_t Hkv, int32_t* per_unit);
 
 // Runs a per-device set-up call (raising a kernel's dynamic shared-memory limit) once for every
 // device ordinal that launches through it: the attribute belongs to the device's copy of the kernel.

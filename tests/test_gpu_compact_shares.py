@@ -51,3 +51,15 @@ def test_units_of_different_lengths(hkv, lens, share, token_major):
             x, y = x[b][:, :m], y[0][:, :m]
             assert torch.equal(x if x.dtype == torch.int32 else x.view(torch.int16), y if y.dtype == torch.int32 else y.view(torch.int16))
     assert status.item() == 0
+
+
+# Sizes at which the CTAs do help one another, and one that a shared launch leaves to itself for its short units.
+HELPED = [(8, [28000, 12000, 18000, 3000, 600, 0, 20, 9000], 0.5), (8, [4096] * 20, 0.9), (8, [8000, 5000, 7600, 4300] * 8, 0.02),
+          (8, [6000, 7500, 4800] * 6, 0.4)]
+NOT_HELPED = [(8, [1120] * 24, 0.5)]
+
+
+@pytest.mark.parametrize("hkv,lens,share", HELPED + NOT_HELPED)
+@pytest.mark.parametrize("token_major", [False, True])
+def test_units_that_are_helped(hkv, lens, share, token_major):
+    test_units_of_different_lengths(hkv, lens, share, token_major)
