@@ -1,6 +1,6 @@
 // Combine of the attention partials that the key ranges of a query row produce.
 //
-// One warp per (query row, unit): the partial maxima, sums and outputs of the row's key ranges
+// One warp (half a one where rows are very many) per (query row, unit): the partial maxima, sums and outputs of the row's key ranges
 // are merged into the row's softmax normaliser and attention output
 //   o_q = sum_j alpha_qj Vsum_j / c_j,  alpha = softmax_j(scale <q, K_j> + ln c_j)   [Eq. attn_def_vec
 // with merged slots].  For the observation window the kernel writes what the statistics pass needs
@@ -13,14 +13,15 @@ constexpr int kThreads = 256;
 
 // kLanes lanes (a warp, or half of one) own a query row, each one 128 / kLanes of its channels.
 // kBatch: partial outputs of a row that are requested together.  With few rows the kernel is a chain of L2
-// round trips, and shorter with eight (1024 rows of 9-37 ranges: 8.5-10 -> 5.3 us); with more rows the registers of a
-// batch cost occupancy.  Between them four (58 registers: four CTAs to an SM): 16 units of 189 rows
-// and 2 to 7 ranges 14.6 us a call, one by one 18.3, in eights 15.6; 16 units of 224 rows 83.9, 88.4 and 84.6; 32
-// units of 256 rows 85.6, 84.8 and 88.9.  With very many rows half warps, which request 32 bytes a lane
-// at once: 65536 rows of one range 27.0 -> 25.0 us by events, ten rounds of 65536 rows of one to three 356 -> 336, 13 rounds of
-// 8192 rows of nine 175 -> 161; two or four partials together 25-27, 358 and 171.
+// round trips, and shorter with eight; with more rows the registers of a batch cost occupancy, and four are better; with very many
+// rows half warps, which request 32 bytes a lane at once.  Us a call in eights, in fours and one by one in half warps:
+// 1024 rows of 16 ranges 16.5, 18.4, 20.0; 2048 rows of 8 20.1, 21.6, 24.1, of 2 22.9, 23.3, 23.6; 3072 of 3 26.6, 26.5, 27.5; 4096 of
+// 4 21.1, 18.8, 21.2; 6144 of 3 30.6, 29.9, 29.4; 8192 of 2 28.5, 27.0, 25.8; 16384 of 1 47.0, 44.7, 41.3; 65536 171, 160, 148.
+// (Two or four partials together in half warps: 65536 rows of one range 25-27 us by events, one by one 25.0.)
+// The bounds on the CTAs of an SM leave ptxas the registers of a batch (71 in eights, 59 in fours); without them it takes 48 and
+// spills, and 256 rows of 16 ranges take 0.7 us longer.
 template <int kBatch, int kLanes>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, kBatch == 1 ? 0 : kBatch == 4 ? 4 : 2)
 combine_partials(const CombineArgs a, const RoundTable tab) {
   constexpr int kVec = 32 / kLanes;                        // float4 of a lane
   constexpr int kChannels = 4 * kVec;
