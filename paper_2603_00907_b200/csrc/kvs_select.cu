@@ -1,7 +1,7 @@
 // Scores, merge weights and the exact selection of a round.
 //
 // A cluster of up to eight CTAs owns a (sequence, KV head) unit; a CTA owns a run of compaction tiles
-// (32 candidate pairs each), a thread one pair of every 1024.  The cluster
+// (32 candidate pairs each), a warp a run of these, a lane one pair of each.  The cluster
 //   1. adds the statistics kernel's partial sums of every pair in a fixed order and forms the pair's
 //      score and left-key weight (for long rounds a kernel of its own does that, see below),
 //   2. finds the bit pattern of the R-th smallest score (scores are non-negative floats: their bit patterns order
@@ -106,6 +106,10 @@ finalize_kernel(const StatsTcArgs a, const RoundTable tab) {
   finish_pair(a, unit, tab.off, p, pair_sums(a, unit, p));
 }
 
+// A key: the bits of a score, which is not negative (nor has a NaN its sign here: every key lies in the first interval).
+constexpr uint32_t kKeyBits = 0x7fffffffu;
+// Passes until the interval is one pattern: the widest bin of the first pass has 2^30 of them, a later pass divides by 2^12.
+constexpr int kPasses = 4;
 // The digit of the first pass: 64 bins to an octave of the score from 2^-56 to 2^8; what lies outside joins the first
 // or the last bin.  (It grows with the score, and the bins are so narrow that few scores share the cutoff's.)
 constexpr int kFirstBin = (127 - 56) << 6;
@@ -156,7 +160,7 @@ select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
 #pragma unroll 1
     for (int u = 0, p = p_first; u < steps && p < p_end; ++u, p += 32) {
       const float x = finish_pair(sa, unit, tab.off, p, pair_sums(sa, unit, p));
-      if (steps <= kKeep) s_key[u * kThreads + tid] = __float_as_uint(x);
+      if (steps <= kKeep) s_key[u * kThreads + tid] = __float_as_uint(x) & kKeyBits;
     }
   } else if (kMode == kFusedFew) {
 #pragma unroll 1
@@ -166,19 +170,21 @@ select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
       const float sx = finish_pair(sa, unit, tab.off, p, x);
       const float sy = two ? finish_pair(sa, unit, tab.off, p + 32, y) : 0.f;
       if (steps <= kKeep) {
-        s_key[u * kThreads + tid] = __float_as_uint(sx);
-        if (two) s_key[(u + 1) * kThreads + tid] = __float_as_uint(sy);
+        s_key[u * kThreads + tid] = __float_as_uint(sx) & kKeyBits;
+        if (two) s_key[(u + 1) * kThreads + tid] = __float_as_uint(sy) & kKeyBits;
       }
     }
   } else if (kMode == kScores && steps <= kKeep) {
 #pragma unroll 4
-    for (int u = 0; u < steps; ++u) s_key[u * kThreads + tid] = p_first + 32 * u < p_end ? score[p_first + 32 * u] : 0u;
+    for (int u = 0; u < steps; ++u) s_key[u * kThreads + tid] = p_first + 32 * u < p_end ? score[p_first + 32 * u] & kKeyBits : 0u;
   }
+  // (pairs are at most 4096 in the fused modes, but a unit with a long protected suffix has more tiles, and more steps than
+  // are kept: then the scores just written are read again)
   // the key of a step (every thread reads only what it has written itself)
   auto key_of = [&](int u) -> uint32_t {
     const int p = p_first + 32 * u;
     if (p >= p_end) return 0u;
-    return kFromMask ? (uint32_t)mask[p] : steps <= kKeep ? s_key[u * kThreads + tid] : score[p];
+    return kFromMask ? (uint32_t)mask[p] : steps <= kKeep ? s_key[u * kThreads + tid] : score[p] & kKeyBits;
   };
   auto cluster_barrier = [&] { if (kCluster) cluster.sync(); else __syncthreads(); };
   auto of_rank = [&](auto* x, int r) { return kCluster ? *cluster.map_shared_rank(x, r) : *x; };
@@ -187,10 +193,10 @@ select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
   //      [lo, lo + width) that holds it into up to 4096 bins, until the interval is one pattern or is taken as a whole.
   uint32_t cutoff = 0, k = kFromMask ? 0u : (uint32_t)sr.R;
   if (!kFromMask) {
-    uint32_t lo = 0, width = 0x80000000u;
+    uint32_t lo = 0, width = kKeyBits + 1u;
     __syncthreads();
 #pragma unroll 1
-    for (int pass = 0;; ++pass) {
+    for (int pass = 0; pass < kPasses; ++pass) {
       uint32_t* hist = s_hist[pass & 1];
       if (pass >= 2) {
         for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
@@ -226,18 +232,28 @@ select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
         }
         const uint32_t own = (h[0] + h[1]) + (h[2] + h[3]);
         before += warp_scan(own) - own;
+        bool found = false;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          if (before < k && k <= before + h[i]) { s_pick[0] = 4 * (32 * hit + lane) + i; s_pick[1] = k - before; s_pick[2] = h[i]; }
+          if (before < k && k <= before + h[i]) {
+            s_pick[0] = 4 * (32 * hit + lane) + i; s_pick[1] = k - before; s_pick[2] = h[i];
+            found = true;
+          }
           before += h[i];
         }
+        if (!__any_sync(0xffffffffu, found) && lane == 0) s_pick[2] = 0;
       }
       __syncthreads();
       const uint32_t bin = s_pick[0], in_bin = s_pick[2];
+      if (in_bin == 0) {                                   // no bin holds it: never, as long as 1 <= R <= P
+        if (tid == 0 && sa.status_dev) atomicExch(sa.status_dev, (int)KVS_ERR_CUDA);
+        k = 0;
+        break;
+      }
       k = s_pick[1];
       if (pass == 0) {
         lo = bin == 0 ? 0u : (bin + kFirstBin) << 17;
-        width = (bin == kBins - 1 ? 0x80000000u : (bin + kFirstBin + 1) << 17) - lo;
+        width = (bin == kBins - 1 ? kKeyBits + 1u : (bin + kFirstBin + 1) << 17) - lo;
       } else {
         width = min(1u << shift, width - (bin << shift));
         lo += bin << shift;

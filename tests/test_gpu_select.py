@@ -52,8 +52,8 @@ def test_mask_is_the_smallest_scores(hkv, n, period, first_round):
 
 
 # KV heads, slots, period of the keys, factor of the queries.  Large queries leave most slots with masses far below 2^-56
-# or of 0; a period of 2 gives all pairs one score, fewer and more of them than are ranked directly; the last cases
-# walk more than 32 steps a CTA.
+# or of 0, whose scores share the first bin of the first pass, so that all four passes are needed; a period of 2 gives all pairs
+# one score, and every pass goes on until the interval is that one pattern; the last cases walk more than 32 steps a CTA.
 @pytest.mark.parametrize("hkv,n,period,factor", [
     (2, 300, 2, 1), (2, 2200, 2, 1), (3, 2200, 0, 30), (8, 2084, 0, 4), (3, 8400, 16, 1), (8, 40001, 0, 30), (8, 40001, 2, 1),
     (2, 140000, 64, 1), (160, 66200, 0, 30), (160, 66200, 2, 1)])
@@ -86,4 +86,45 @@ def test_a_pass_takes_the_smallest_scores(hkv, n, period, factor):
     for x, y in ((K, K2), (V, V2), (counts, counts2)):
         assert torch.equal(x[:, :, :n - R].view(torch.int16 if x is not counts else torch.int32),
                            y[:, :, :n - R].view(torch.int16 if x is not counts else torch.int32))
+    assert status.item() == 0
+
+
+# KV heads, slots, pairs, bits of a key channel.  A long protected suffix leaves few pairs (one kernel adds the partials and
+# selects, with and without a CTA to an SM) but more steps of a warp than keys are kept; with undefined keys every score is
+# NaN, of either sign as the sums may have it, and the first pairs are taken.
+@pytest.mark.parametrize("hkv,n,pairs,bits", [(2, 80000, 2000, None), (150, 70000, 600, None), (2, 2200, 1000, 0x7FC0), (2, 2200, 1000, 0xFFC0),
+                                              (3, 9000, 4400, 0xFFC0), (150, 1400, 650, 0x7FC0), (2, 80000, 2000, 0xFFC0),
+                                              (2, 300000, 149000, 0xFFC0)])
+def test_steps_beyond_the_kept_keys_and_undefined_scores(hkv, n, pairs, bits):
+    import torch
+    from paper_2603_00907_b200 import binding as kb, build
+    build.build()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + pairs)
+    K, V = (torch.randn(1, hkv, n, 128, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    if bits is not None:
+        K.view(torch.int16)[0, :, 40, 7] = bits - (1 << 16 if bits >> 15 else 0)
+    counts = torch.ones(1, hkv, n, dtype=torch.int32, device="cuda")
+    q = torch.randn(1, hkv, 4, 128, generator=g, device="cuda").to(torch.bfloat16)
+    p = kb.make_params(K, V, hkv, 4, causal=False, recent=n - 32 - 2 * pairs)
+    ws = torch.empty(kb.kvs_workspace_size(p, n, 0), dtype=torch.uint8, device="cuda")
+    score, w = (torch.zeros(1, hkv, n // 2, device="cuda") for _ in range(2))
+    mask = torch.zeros(1, hkv, n // 2, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    budget = n - pairs // 3
+    _, off, P, R = kb.kvs_round_plan(p, n, budget)[0]
+    assert P == pairs and R == pairs // 3
+    kb.kvs_window_stats(p, K, V, counts, q, [n], [budget], ws, score=score, w=w, mask=mask, status_dev=status)
+    key = score[0, :, :P].view(torch.int32)
+    assert int(key.min()) >= 0
+    assert bits is None or bool(torch.isnan(score[0, :, :P]).all())
+    want = torch.zeros_like(mask)
+    want[0].scatter_(1, torch.sort(key, dim=-1, stable=True).indices[:, :R], 1)
+    assert torch.equal(mask, want) and status.item() == 0
+    # the counts in front of the tiles, the empty ones of the suffix among them
+    index = torch.zeros(1, hkv, n, dtype=torch.int32, device="cuda")
+    kb.kvs_compact(p, K, V, counts, mask, w, [n], [R], ws, new_index=index, status_dev=status)
+    before = torch.zeros(hkv, n, dtype=torch.int32, device="cuda")
+    before[:, off + 1:off + 2 * P:2] = want[0, :, :P].int()
+    assert torch.equal(index[0], torch.arange(n, dtype=torch.int32, device="cuda") - before.cumsum(1, dtype=torch.int32))
     assert status.item() == 0
