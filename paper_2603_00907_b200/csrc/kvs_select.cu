@@ -178,7 +178,7 @@ select_kernel(const StatsTcArgs sa, const SelectArgs a, const RoundTable tab) {
 #pragma unroll 4
     for (int u = 0; u < steps; ++u) s_key[u * kThreads + tid] = p_first + 32 * u < p_end ? score[p_first + 32 * u] & kKeyBits : 0u;
   }
-  // (pairs are at most 4096 in the fused modes, but a unit with a long protected suffix has more tiles, and more steps than
+  // (pairs are at most 3072 in the fused modes, but a unit with a long protected suffix has more tiles, and more steps than
   // are kept: then the scores just written are read again)
   // the key of a step (every thread reads only what it has written itself)
   auto key_of = [&](int u) -> uint32_t {
@@ -367,16 +367,15 @@ cudaError_t launch_select(const StatsTcArgs& sa, const SelectArgs& a, const Roun
   return cudaLaunchKernelEx(&cfg, select_kernel<kMode, kCluster>, sa, a, t);
 }
 
-// Whether the selection kernel adds the partials itself: where they are few (at most two query blocks), and
-//   * a unit has up to 1024 pairs: 8 units of 350 30.3 us a call against 31.1 with a kernel of its own, 32 of 700 40.4 and 43.8;
-//   * there are up to 16 units of up to 3072 pairs, or up to 44000 pairs in all: 16 of 2000 42.5 us and 46.3, 8 of 3000 42.3
-//     and 44.5, 24 of 1760 51.1 and 55.4;
-//   * the units are enough for the GPU: 128 of 2000 175 us and 186.
-// Between them its few CTAs are slow readers: 24 units of 3000 pairs 74 us against 64, 32 of 2000 67 and 61, 64 of 4000
-// 195 and 183, 16 of 4000 63 and 61.
+// Whether the selection kernel adds the partials itself: where they are few (at most two query blocks), and a unit has up to
+// 1536 pairs, or up to 3072 with up to 16 units.  Its few CTAs are slow readers of more.  Us a call of the statistics with a
+// kernel of its own for the partials and without, 64 rows: 8 units of 700 pairs 28.5 and 24.5, of 2000 30.4 and 27.9, of 3000 34.6 and 34.8; 16 of
+// 3000 43.5 and 40.8; 24 of 1500 36.7 and 34.3, of 3000 49.4 and 50.2, of 4000 60.4 and 62.7; 32 of 1500 41.7 and 38.9, of 2000 46.5 and
+// 45.6; 64 of 1500 67.2 and 65.5, of 4000 137 and 139; 128 of 1500 112 and 110; 256 of 1500 208.9 and 208.2, of 3000 371 and 387; 256 rows: 16
+// of 3000 68.6 and 67.1; 32 of 1500 69.4 and 65.7, of 3000 110 and 112; 128 of 1500 217 and 215, of 2000 264 and 274; 256 of 2000 506 and 540.
 bool fused_finalize(const StatsTcArgs& sa, const SelectArgs& a, int units, int pmax) {
-  if (!a.select || sa.nqblk > 2 || pmax > 4096) return false;
-  return pmax <= 1024 || units >= 128 || (pmax <= 3072 && (units <= 16 || pmax * units <= 44000));
+  if (!a.select || sa.nqblk > 2) return false;
+  return pmax <= 1536 || (pmax <= 3072 && units <= 16);
 }
 
 }  // namespace
@@ -387,7 +386,7 @@ cudaError_t kvs_launch_finalize_select(const StatsTcArgs& sa, const SelectArgs& 
   const int pmax = most_pairs(t);
   if (pmax <= 0) return cudaSuccess;
   const int units = a.Hkv * t.nseq;
-  if (fused_finalize(sa, a, units, pmax))                  // (at most 4096 pairs a unit: one CTA)
+  if (fused_finalize(sa, a, units, pmax))                  // (so few pairs a unit: one CTA)
     return units <= 148 ? launch_select<kFusedFew, false>(sa, a, t, 1, st) : launch_select<kFused, false>(sa, a, t, 1, st);
   cudaError_t e = kvs_launch_chained(finalize_kernel, dim3((pmax + 255) / 256, a.Hkv, t.nseq), dim3(256), 0, st, sa, t);
   if (e != cudaSuccess || !a.select) return e;

@@ -11,8 +11,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("hkv,n,period,first_round", [
     (2, 300, 0, 0), (3, 8200, 0, 1), (3, 8400, 64, 0), (8, 20011, 128, 1), (2, 140000, 0, 0), (2, 140000, 512, 1),
     (160, 66200, 512, 0),
-    # both sides of the lines between one kernel and two (1024 pairs; 3072 with up to 16 units or 44000 in all; 4096 from
-    # 128 units on)
+    # one kernel and two, few units and many, around 1024 to 4096 pairs
     (50, 2084, 0, 0), (50, 2086, 32, 0), (17, 5212, 0, 0), (17, 5214, 32, 1), (16, 6181, 64, 1), (16, 6184, 0, 1),
     (128, 8228, 64, 0), (128, 8230, 0, 0)])
 def test_mask_is_the_smallest_scores(hkv, n, period, first_round):
@@ -89,10 +88,11 @@ def test_a_pass_takes_the_smallest_scores(hkv, n, period, factor):
     assert status.item() == 0
 
 
-# KV heads, slots, pairs, bits of a key channel.  A long protected suffix leaves few pairs (one kernel adds the partials and
+# KV heads, slots, pairs, bits of a key channel.  Both sides of the lines between one kernel and two.  A long protected suffix leaves few pairs (one kernel adds the partials and
 # selects, with and without a CTA to an SM) but more steps of a warp than keys are kept; with undefined keys every score is
 # NaN, of either sign as the sums may have it, and the first pairs are taken.
-@pytest.mark.parametrize("hkv,n,pairs,bits", [(2, 80000, 2000, None), (150, 70000, 600, None), (2, 2200, 1000, 0x7FC0), (2, 2200, 1000, 0xFFC0),
+@pytest.mark.parametrize("hkv,n,pairs,bits", [(17, 3200, 1536, None), (17, 3200, 1537, None), (16, 6300, 3072, None), (16, 6300, 3073, None),
+                                              (150, 3200, 1536, None), (150, 3200, 1537, None), (2, 80000, 2000, None), (150, 70000, 600, None), (2, 2200, 1000, 0x7FC0), (2, 2200, 1000, 0xFFC0),
                                               (3, 9000, 4400, 0xFFC0), (150, 1400, 650, 0x7FC0), (2, 80000, 2000, 0xFFC0),
                                               (2, 300000, 149000, 0xFFC0)])
 def test_steps_beyond_the_kept_keys_and_undefined_scores(hkv, n, pairs, bits):
