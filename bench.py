@@ -113,9 +113,9 @@ class ClockSampler(threading.Thread):
 # processed, so the ratio carries over to a full launch).  Each entry names the kernel source it was
 # taken on: once that file changes, the figure is stale and `traffic` is reported as null.
 NCU_TRAFFIC = {
-    "hessian_stats": (1.11, "kvs_stats_tc.cu", "5565af8be512ae8a"),
-    "attn_partials": (1.05, "kvs_flash_tc.cu", "b9f292f6f3f403de"),
-    "merge_compact": (0.90, "kvs_compact.cu", "3624b502768ce023"),
+    "hessian_stats": (1.10, "kvs_stats_tc.cu", "2896b1c48c56b8b3"),
+    "attn_partials": (1.05, "kvs_flash_tc.cu", "bc0da83e495d945d"),
+    "merge_compact": (0.90, "kvs_compact.cu", "e59751afe13165c6"),
 }
 
 

@@ -16,8 +16,10 @@
  *     void*; NULL is the legacy default stream).
  *   - Errors the host can detect return a code before anything is enqueued and leave all
  *     buffers untouched.  Errors only the device can detect (a bounded wait that ran out)
- *     set *status_dev to a kvs_status_t value; the pass then finishes without touching
- *     further cache memory.  status_dev may be NULL.
+ *     set *status_dev to a kvs_status_t value.  The CTA that found one stores nothing from
+ *     then on (a compaction tile of 64 slots is stored whole or not at all); the kernels
+ *     behind it on the stream still run, on what they find, within the buffers of the call.
+ *     The results of that call, its caches included, are unspecified.  status_dev may be NULL.
  *   - bf16 tensors are passed as void* to 16-bit words; layouts are row major with the
  *     head dimension (128) innermost and contiguous.
  *   - A cache "slot" is a triple (key, value SUM, count).  A fresh token has count 1 and
