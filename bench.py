@@ -115,7 +115,7 @@ class ClockSampler(threading.Thread):
 NCU_TRAFFIC = {
     "hessian_stats": (1.10, "kvs_stats_tc.cu", "2896b1c48c56b8b3"),
     "attn_partials": (1.05, "kvs_flash_tc.cu", "bc0da83e495d945d"),
-    "merge_compact": (0.90, "kvs_compact.cu", "e59751afe13165c6"),
+    "merge_compact": (0.90, "kvs_compact.cu", "11b57259ed9949d1"),
 }
 
 

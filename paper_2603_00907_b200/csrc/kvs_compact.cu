@@ -81,8 +81,8 @@ constexpr int kSmemBytes = kStages * kStageBytes + (int)sizeof(Shared);
 // acquire is free in the gate, the release is not: with relaxed flags 8 units of 256 tiles take 22.5 us a launch and
 // so 24.5, of 2048 149 and 152, 128 of 256 300 and 309, all rounds of a ragged batch of 4 K to 64 K slots 927 and 977.
 // They are looked at with an atomic, which goes to the one place where the line lives.  A load leaves copies of a line that is
-// about to be written in the caches in between: a CTA that looked a little too early saw the flag 2 us late (a launch of 8
-// units of 256 tiles with loads 34.4 us, so 23.2; 64 units of 24 tiles 23.0 and 20.9).
+// about to be written in the caches in between: a CTA that looked a little too early saw the flag 2 us late (with a release for
+// every tile, 8 units of 256 tiles with loads 34.4 us, with atomics 23.2; 64 units of 24 tiles 23.0 and 20.9).
 __device__ __forceinline__ uint32_t see_flag(uint32_t* p) {
   uint32_t v;
   asm volatile("atom.acquire.gpu.global.or.b32 %0, [%1], 0;" : "=r"(v) : "l"(p) : "memory");
