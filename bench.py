@@ -113,7 +113,7 @@ class ClockSampler(threading.Thread):
 # processed, so the ratio carries over to a full launch).  Each entry names the kernel source it was
 # taken on: once that file changes, the figure is stale and `traffic` is reported as null.
 NCU_TRAFFIC = {
-    "hessian_stats": (1.10, "kvs_stats_tc.cu", "2896b1c48c56b8b3"),
+    "hessian_stats": (1.10, "kvs_stats_tc.cu", "a8730ecaea5a6679"),
     "attn_partials": (1.05, "kvs_flash_tc.cu", "bc0da83e495d945d"),
     "merge_compact": (0.90, "kvs_compact.cu", "11b57259ed9949d1"),
 }

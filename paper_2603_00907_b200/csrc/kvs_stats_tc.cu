@@ -298,6 +298,13 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
         }
       }
       misc->k_issued = kli; misc->v_issued = vli; misc->q_issued = qli; misc->c_issued = cli;
+      // the last commits, which nobody else waits for, beside the last tile's statistics
+      if (!*abort_flag) {
+        mbar_drain(&misc->done, 0);
+        mbar_drain(&misc->kfree, (kli - 1) & 1);
+        mbar_drain(&misc->vfree, (vli - 1) & 1);
+        mbar_drain(&misc->qfree, (qli - 1) & 1);
+      }
     }
   } else if (warp < kFirstStat) {
     // ================================================================ product issuers
@@ -474,8 +481,8 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
 
   // ================================================================== common exit
   // Nothing may be in flight when the CTA leaves: its shared and tensor memory are the next CTA's from then on.  A whole walk
-  // has waited for its copies and products, but for the last commits that hand the operands back; behind one that
-  // broke off, in whichever role and after whichever request, any copy and any product may be under way.
+  // has waited for its copies and products; behind one that broke off, in whichever role and after whichever request, any copy
+  // and any product may be under way.
   tc_fence_before();
   __syncthreads();
   const bool gave_up = *abort_flag != 0;                   // (no wait is left that could set it)
@@ -485,20 +492,14 @@ hessian_stats_tc(const StatsTcArgs a, const RoundTable tab, const __grid_constan
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && gave_up) {
     const uint32_t nk = misc->k_issued, nv = misc->v_issued, nq = misc->q_issued, nc = misc->c_issued;
     mbar_drain(&misc->done, 0);
-    if (gave_up) {
-      if (nk > 0 && !withhold_k) mbar_drain(&misc->kfull, (nk - 1) & 1);
-      if (nv > 0) mbar_drain(&misc->vfull, (nv - 1) & 1);
-      if (nq > 0) mbar_drain(&misc->qfull, (nq - 1) & 1);
-      if (nc > 0) mbar_drain(&misc->cfull, (nc - 1) & 1);
-      if (a.status_dev) atomicExch(a.status_dev, (int)KVS_ERR_TIMEOUT);
-    } else {
-      mbar_drain(&misc->kfree, (nk - 1) & 1);
-      mbar_drain(&misc->vfree, (nv - 1) & 1);
-      mbar_drain(&misc->qfree, (nq - 1) & 1);
-    }
+    if (nk > 0 && !withhold_k) mbar_drain(&misc->kfull, (nk - 1) & 1);
+    if (nv > 0) mbar_drain(&misc->vfull, (nv - 1) & 1);
+    if (nq > 0) mbar_drain(&misc->qfull, (nq - 1) & 1);
+    if (nc > 0) mbar_drain(&misc->cfull, (nc - 1) & 1);
+    if (a.status_dev) atomicExch(a.status_dev, (int)KVS_ERR_TIMEOUT);
   }
 }
 
